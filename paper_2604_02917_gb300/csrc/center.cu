@@ -1,14 +1,26 @@
 // mv_center_factor: mu = R 1/T, L = (R - mu 1^T)/sqrt(T-1), tr(Sigma) = ||L||_F^2 (Sec. 2.1).
 //
-// One block per asset row.  Pass 1 sums the row in FP64 for mu_i; pass 2
-// accumulates sum_t ((R_it - mu_i) c)^2 in FP64 (and max |.| for the FP8
-// row scale); pass 3 writes L in the storage type, zero-filling columns
-// T..ldL-1.  For the transposed layout (L^T, T x n) pass 3 is replaced by a
-// tiled transpose that reads R again along periods.  Passes 2 and 3 re-read a row the block has just streamed, so
-// they mostly hit L2.  Per-row sums of squares are added in a second,
+// n x T output: one block per asset row sums the row and writes it centred;
+// the second read of the row hits L2.  Transposed output: the same kernel
+// leaves the means, then a tiled transpose reads R again along periods.
+// Sums of squares go to one partial per block, added in a second,
 // single-block kernel in fixed order, so tr(Sigma) is deterministic.
+//
+// Arithmetic.  The results are those of FP64 (mu, tr Sigma to FP64 rounding,
+// every stored entry of L the rounding of the FP64 value), but GB300 retires
+// about 2 FP64 operations per clock and SM, and one FP64 operation per entry
+// of R already costs 0.45 ms at 5440 x 48374 (the copy rate would read R in
+// 0.155 ms).  So an entry meets FP64 only when it has to:
+//  * sum of a row: exact 64-bit integer sums of the entries' significands
+//    (RowSum);
+//  * centred entry: an FP32 pair with a proven error bound, FP64 when the
+//    bound leaves the rounding open (centred());
+//  * sum of squares: an FP32 pair per thread (SquareSum).
+// With FP64 per entry 5440 x 48374 FP32 took 3.55 ms.
 #include <stdio.h>
 #include <string.h>
+
+#include <algorithm>
 
 #include "mv_internal.cuh"
 
@@ -30,165 +42,352 @@ int record_message(int status, const char *msg) {
 
 constexpr int kCenterThreads = 512;
 
+// Sum of FP32 values, exact but for the final rounding.  A value is a 24-bit
+// significand m (signed) times 2^(e - 150); m << (e - eb) is added to a
+// 64-bit integer while e lies in [eb, eb + 30] (under 2^54 each, so 256 of
+// them fit), eb being set so that the first value seen has 8 octaves of
+// headroom.  Anything outside that window (a value 2^8 above or 2^-22 below
+// the first, infinities, NaN) is added in FP64; a larger value also moves
+// the window.  About 10 integer operations per value, against an FP64
+// conversion and addition at 2 per clock and SM.
+struct RowSum {
+    long long acc = 0;
+    double wide = 0.0;
+    int eb = 1 << 20;              // no value seen yet: everything is out of the window
+
+    __device__ __forceinline__ void flush() {
+        if (acc != 0) wide += scalbn((double)acc, eb - 150);
+        acc = 0;
+    }
+    __device__ __forceinline__ void add_wide(float x) {
+        const unsigned b = __float_as_uint(x) & 0x7fffffffu;
+        if (b == 0) return;
+        const int e = (int)(b >> 23);
+        if (e >= 1 && e < 255 && (eb == 1 << 20 || e > eb + 30)) {
+            flush();
+            eb = e > 23 ? e - 22 : 1;      // never 0: the significand of e = 0 has no implicit bit
+            add_inside(x);
+        } else {
+            wide += (double)x;
+        }
+    }
+    __device__ __forceinline__ bool inside(float x) const {
+        return (unsigned)((int)((__float_as_uint(x) >> 23) & 0xff) - eb) <= 30u;
+    }
+    __device__ __forceinline__ void add_inside(float x) {
+        const int b = __float_as_int(x);
+        const int sh = ((b >> 23) & 0xff) - eb;
+        const int m = (b & 0x7fffff) | 0x800000, sg = b >> 31;
+        acc += (long long)((m ^ sg) - sg) * (long long)(1 << sh);
+    }
+    // K values; the window test is one branch for all of them.
+    template <int K>
+    __device__ __forceinline__ void add(const float (&x)[K]) {
+        bool in = true;
+#pragma unroll
+        for (int k = 0; k < K; ++k) in = in && inside(x[k]);
+        if (in) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) add_inside(x[k]);
+        } else {
+#pragma unroll 1
+            for (int k = 0; k < K; ++k) {
+                float v = 0.f;
+#pragma unroll
+                for (int j = 0; j < K; ++j) v = j == k ? x[j] : v;
+                if (inside(v)) add_inside(v); else add_wide(v);
+            }
+        }
+    }
+    __device__ __forceinline__ double total() {
+        flush();
+        return wide;
+    }
+};
+
+// Constants of one row: mean and c = 1/sqrt(T-1) as FP32 pairs, and the
+// absolute part of the error bound of centred().  `wide` is infinite where
+// the FP32 range cannot be relied on (the row's largest |R| outside
+// [2^-30, 2^50], infinities or NaN): every entry then takes the FP64 path.
+struct RowConst {
+    float mh, ml, ch, cl, wide;
+};
+__device__ __forceinline__ RowConst row_const(double mean, double c, float amax) {
+    RowConst k;
+    k.mh = (float)mean;
+    k.ml = (float)(mean - (double)k.mh);
+    k.ch = (float)c;
+    k.cl = (float)(c - (double)k.ch);
+    const bool ok = amax >= 0x1p-30f && amax <= 0x1p50f && fabsf(k.mh) <= 0x1p50f;
+    k.wide = ok ? fmaf(fabsf(k.mh) * k.ch, 0x1p-44f, 0x1p-120f) : INFINITY;
+    return k;
+}
+
+// Sum of squares of FP32 pairs (p, r): s + c carries about 48 bits per
+// thread; values centred in FP64 are added in FP64.
+struct SquareSum {
+    float s = 0.f, c = 0.f;
+    double wide = 0.0;
+    __device__ __forceinline__ void add(float p, float r) {
+        const float q = p * p;
+        float e = fmaf(p, p, -q);                       // p^2 = q + e exactly
+        e = fmaf(fmaf(2.f, p, r), r, e);
+        const float t = s + q, bb = t - s;              // s + q = t + (rounding error), exactly
+        c += ((s - (t - bb)) + (q - bb)) + e;
+        s = t;
+    }
+    __device__ __forceinline__ double total() const { return wide + ((double)s + (double)c); }
+};
+
+// FP32 rounding of d = (x - mean) c.  x - mh is exact as the pair (s, e);
+// the product with the pair (ch, cl) leaves d = p + r with an error below
+// 7 x 2^-48 |p| + 3 x 2^-48 |mh| ch (unit roundoff 2^-24 in each of the
+// pair's low parts), and r +- tol adds 3 x 2^-48 |p| + 2^-48 |mh| ch: inside
+// tol = 2^-44 (|p| + |mh| ch) for rows inside row_const's limits.  Where p + r - tol and p + r +
+// tol round to the same FP32 value that value is the rounding of the FP64
+// result too; elsewhere (about one entry in 2^18) d is formed in FP64.
+// BF16 adds one case: an FP32 value on a BF16 tie does not say which way
+// the FP64 value rounds.  ~17 FP32 operations, against 3 FP64 ones and a
+// conversion.  Returns the stored FP32 value (d64 the FP64 one on that path,
+// `exact` set) and adds d^2 to q.
 template <int DT>
-__device__ __forceinline__ void store_elem(void *L, int64_t idx, double val, float inv_scale) {
+__device__ __forceinline__ float centred(float x, const RowConst &k, double mean, double c, SquareSum &q, double &d64,
+                                         bool &exact) {
+    const float s = x - k.mh, bb = s - x;
+    const float e = ((x - (s - bb)) - (k.mh + bb)) - k.ml;
+    const float p = s * k.ch;
+    float r = fmaf(s, k.ch, -p);
+    r = fmaf(s, k.cl, r);
+    r = fmaf(e, k.ch, r);
+    const float tol = fmaf(fabsf(p), 0x1p-44f, k.wide);
+    const float f = p + (r - tol);
+    exact = !(f == p + (r + tol));
+    if constexpr (DT == MV_BF16) exact = exact || (__float_as_uint(f) & 0xffffu) == 0x8000u;
+    if (exact) {
+        d64 = ((double)x - mean) * c;
+        q.wide = fma(d64, d64, q.wide);
+        return (float)d64;
+    }
+    q.add(p, r);
+    return f;
+}
+
+template <int DT>
+__device__ __forceinline__ void store_elem(void *L, int64_t idx, float val, float inv_scale) {
     if constexpr (DT == MV_F32) {
-        reinterpret_cast<float *>(L)[idx] = (float)val;
+        reinterpret_cast<float *>(L)[idx] = val;
     } else if constexpr (DT == MV_BF16) {
-        reinterpret_cast<__nv_bfloat16 *>(L)[idx] = __double2bfloat16(val);
+        reinterpret_cast<__nv_bfloat16 *>(L)[idx] = __float2bfloat16_rn(val);
     } else {
-        const float q = (float)val * inv_scale;
-        reinterpret_cast<__nv_fp8_storage_t *>(L)[idx] = __nv_cvt_float_to_fp8(q, __NV_SATFINITE, __NV_E4M3);
+        reinterpret_cast<__nv_fp8_storage_t *>(L)[idx] = __nv_cvt_float_to_fp8(val * inv_scale, __NV_SATFINITE, __NV_E4M3);
     }
 }
 
-// One block per asset row.  Pass 1: mu_i = sum_t R_it / T in FP64, and the
-// FP32 range of the row; the FP8 scale max_t |d_it| / 448 follows exactly
-// from it, because d = ((double)x - mu) c is monotone in x.  Pass 2 (WRITE):
-// d_it in FP64, stored in the storage type, and sum_t d_it^2 for the trace;
-// the re-read of the row mostly hits L2.  With WRITE = false (transposed
-// layout) pass 2 is done by transpose_center_kernel.
+// The value to store for an entry of R: for BF16 already rounded to it (from
+// FP64 where the FP32 value would round twice).
+template <int DT>
+__device__ __forceinline__ float centred_value(float x, const RowConst &k, double mean, double c, SquareSum &q) {
+    double d64 = 0.0;
+    bool exact;
+    const float f = centred<DT>(x, k, mean, c, q, d64, exact);
+    if constexpr (DT == MV_BF16)
+        if (exact) return __bfloat162float(__double2bfloat16(d64));
+    return f;
+}
+
+// One block per asset row.  Pass 1: mu_i = sum_t R_it / T and the FP32 range
+// of the row; the FP8 scale max_t |d_it| / 448 follows exactly from it,
+// because d = ((double)x - mu) c is monotone in x.  Pass 2 (WRITE): the
+// centred entries, stored in the storage type, and their squares for the
+// trace; the re-read of the row mostly hits L2.  With WRITE = false
+// (transposed layout) pass 2 is done by transpose_center_kernel, which finds
+// the row's largest |R| in amax.  Entries are read one per lane (rows of a
+// ragged panel share no 16-byte alignment), kUnroll loads in flight.
+constexpr int kCenterUnroll = 8;
 template <int DT, bool WRITE>
 __global__ void __launch_bounds__(kCenterThreads)
-center_kernel(const float *__restrict__ R, int64_t ldR, int T, void *__restrict__ L, int64_t ldL,
-              float *__restrict__ row_scale, double *__restrict__ mu, double *__restrict__ rowsq, int64_t i_base) {
+center_kernel(const float *__restrict__ R, int64_t ldR, unsigned T, void *__restrict__ L, int64_t ldL,
+              float *__restrict__ row_scale, double *__restrict__ mu, double *__restrict__ rowsq,
+              float *__restrict__ amax_out, int64_t i_base) {
+    constexpr int U = kCenterUnroll;
     __shared__ double red[(kCenterThreads / kWarp + 1) * 2];
     const int64_t i = i_base + blockIdx.x;                 // asset; R holds rows i_base ..
     const float *r = R + (int64_t)blockIdx.x * ldR;
-    double s[1] = {0.0};
+    RowSum sum;
     float xmin = INFINITY, xmax = -INFINITY;
-    for (int t = threadIdx.x; t < T; t += kCenterThreads) {
-        const float x = r[t];
-        s[0] += (double)x;
-        if constexpr (DT == MV_FP8_E4M3) {
-            xmin = fminf(xmin, x);
-            xmax = fmaxf(xmax, x);
+    unsigned t = threadIdx.x;
+    int since = 0;
+    for (; t + (U - 1) * kCenterThreads < T; t += U * kCenterThreads) {
+        float x[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) x[k] = r[t + k * kCenterThreads];
+        sum.add(x);
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            xmin = fminf(xmin, x[k]);
+            xmax = fmaxf(xmax, x[k]);
+        }
+        since += U;
+        if (since >= 240) {                                 // at most 256 values in the integer
+            sum.flush();
+            since = 0;
         }
     }
+    for (; t < T; t += kCenterThreads) {                    // fewer than U values
+        const float x[1] = {r[t]};
+        sum.add(x);
+        xmin = fminf(xmin, x[0]);
+        xmax = fmaxf(xmax, x[0]);
+    }
+    double s[1] = {sum.total()};
     block_sum<1, kCenterThreads>(s, red);
     const double mean = s[0] / (double)T;
     const double c = 1.0 / sqrt((double)(T - 1));
+    double mn = (double)xmin, mx = (double)xmax;
+    __syncthreads();
+    block_minmax<kCenterThreads>(mn, mx, red);
     float inv_scale = 1.f;
     if constexpr (DT == MV_FP8_E4M3) {
-        double mn = (double)xmin, mx = (double)xmax;
-        __syncthreads();
-        block_minmax<kCenterThreads>(mn, mx, red);
         const double amax = fmax((mx - mean) * c, (mean - mn) * c);
         const float scale = amax > 0.0 ? (float)(amax / 448.0) : 1.f;
         inv_scale = 1.f / scale;
         if (threadIdx.x == 0) row_scale[i] = scale;
     }
+    const float ra = fmaxf(fabsf((float)mn), fabsf((float)mx));
     if constexpr (WRITE) {
-        double q[1] = {0.0};
-        for (int64_t t = threadIdx.x; t < ldL; t += kCenterThreads) {
-            const double d = t < T ? ((double)r[t] - mean) * c : 0.0;
-            q[0] = fma(d, d, q[0]);
-            store_elem<DT>(L, i * ldL + t, d, inv_scale);
+        const RowConst k = row_const(mean, c, ra);
+        SquareSum q;
+        int64_t o = i * ldL;
+        t = threadIdx.x;
+        for (; t + (U - 1) * kCenterThreads < T; t += U * kCenterThreads) {
+            float x[U];
+#pragma unroll
+            for (int j = 0; j < U; ++j) x[j] = r[t + j * kCenterThreads];
+#pragma unroll
+            for (int j = 0; j < U; ++j)
+                store_elem<DT>(L, o + t + j * kCenterThreads, centred_value<DT>(x[j], k, mean, c, q), inv_scale);
         }
+        for (; t < T; t += kCenterThreads) store_elem<DT>(L, o + t, centred_value<DT>(r[t], k, mean, c, q), inv_scale);
+        for (int64_t z = (int64_t)T + threadIdx.x; z < ldL; z += kCenterThreads) store_elem<DT>(L, o + z, 0.f, inv_scale);
+        double v[1] = {q.total()};
         __syncthreads();
-        block_sum<1, kCenterThreads>(q, red);
-        if (threadIdx.x == 0) rowsq[i] = q[0];
+        block_sum<1, kCenterThreads>(v, red);
+        if (threadIdx.x == 0) rowsq[i] = v[0];
+    } else if (threadIdx.x == 0) {
+        amax_out[i] = ra;
     }
     if (threadIdx.x == 0) mu[i] = mean;
 }
 
-// L^T (T x ldM, row t = period t) from R (n x T).  A block owns 32 assets and
-// one of kSlices period slices, walking it in 32 x 32 tiles through shared
-// memory: read along periods, written along assets; columns n..ldM-1 are
-// written as zeros.  Values as center_kernel's; each block leaves
-// sum_t d_it^2 of its slice in sqpart[slice][i] (added in fixed order by
+// L^T (T x ldM, row t = period t) from R (n x T).  A block owns kTile assets
+// and one of `slices` period slices, walking it in kTile x kTileT tiles
+// through shared memory: read along periods (one row per warp and
+// instruction), written along assets; columns n..ldM-1 are written as zeros.
+// Values as center_kernel's; each block leaves the sum of its squares in
+// sqpart[asset tile x slices + slice] (added in fixed order by
 // trace_kernel).  The slice count is chosen per call to fill the GPU.
 constexpr int kTile = 32;
+constexpr int kTileT = 64;                      // periods per tile
 constexpr int kMaxSlices = 64;                  // period slices per asset tile (grid fill), at most
+constexpr int kTransThreads = 256;
 template <int DT>
-__global__ void __launch_bounds__(kTile * 8)
+__global__ void __launch_bounds__(kTransThreads)
 transpose_center_kernel(const float *__restrict__ R, int64_t ldR, int64_t n, int T, void *__restrict__ M, int64_t ldM,
                         const float *__restrict__ row_scale, const double *__restrict__ mu,
-                        double *__restrict__ sqpart, int64_t i_base, int slices) {
-    __shared__ double tile[kTile][kTile + 1];
+                        const float *__restrict__ amax, double *__restrict__ sqpart, int64_t i_base, int slices) {
+    constexpr int W = kTransThreads / kWarp, RPW = kTile / W;   // warps, asset rows per warp
+    constexpr int H = kTileT / kWarp;                           // loads per row and tile
+    __shared__ float tile[kTile][kTileT + 1];
+    __shared__ double red[kTransThreads / kWarp + 1];
+    __shared__ double s_mean[kTile];
+    __shared__ RowConst s_k[kTile];
     const int64_t i0 = i_base + (int64_t)blockIdx.y * kTile;   // assets; R holds rows i_base ..
     const int slice = blockIdx.x;
-    const int per = ((T + slices - 1) / slices + kTile - 1) / kTile * kTile;
+    const int per = ((T + slices - 1) / slices + kTileT - 1) / kTileT * kTileT;
     const int tb = slice * per, te = min(T, tb + per);
     const double c = 1.0 / sqrt((double)(T - 1));
-    const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;
-    double mloc[4];
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int64_t i = i0 + ty + 8 * j;
-        mloc[j] = i < n ? mu[i] : 0.0;
+    const int lane = threadIdx.x % kWarp, warp = threadIdx.x / kWarp;
+    if (threadIdx.x < kTile) {
+        const int64_t i = i0 + threadIdx.x;
+        s_mean[threadIdx.x] = i < n ? mu[i] : 0.0;
+        s_k[threadIdx.x] = row_const(s_mean[threadIdx.x], c, i < n ? amax[i] : 1.f);
     }
-    float inv = 1.f;
-    if (DT == MV_FP8_E4M3 && i0 + tx < n) inv = 1.f / row_scale[i0 + tx];
-    for (int t0 = tb; t0 < te; t0 += kTile) {
+    __syncthreads();
+    const float inv = (DT == MV_FP8_E4M3 && i0 + lane < n) ? 1.f / row_scale[i0 + lane] : 1.f;
+    SquareSum q;
+    for (int t0 = tb; t0 < te; t0 += kTileT) {
+        float x[RPW][H];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int k = ty + 8 * j;
-            const int64_t i = i0 + k, t = t0 + tx;
-            const double d = (i < n && t < te) ? ((double)R[(i - i_base) * ldR + t] - mloc[j]) * c : 0.0;
-            acc[j] = fma(d, d, acc[j]);
-            tile[k][tx] = d;
+        for (int j = 0; j < RPW; ++j) {
+            const int64_t i = i0 + warp + j * W;
+            const float *row = R + (i - i_base) * ldR + t0 + lane;
+#pragma unroll
+            for (int h = 0; h < H; ++h) x[j][h] = (i < n && lane + h * kWarp < te - t0) ? row[h * kWarp] : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < RPW; ++j) {
+            const int a = warp + j * W;
+            const RowConst k = s_k[a];
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+                if (i0 + a < n && lane + h * kWarp < te - t0)
+                    tile[a][lane + h * kWarp] = centred_value<DT>(x[j][h], k, s_mean[a], c, q);
+                else
+                    tile[a][lane + h * kWarp] = 0.f;
         }
         __syncthreads();
+        if (i0 + lane < ldM) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int k = ty + 8 * j;
-            const int64_t t = t0 + k, i = i0 + tx;
-            if (t < te && i < ldM) store_elem<DT>(M, t * ldM + i, tile[tx][k], i < n ? inv : 1.f);
+            for (int j = 0; j < kTileT / W; ++j) {
+                const int w = warp + j * W;
+                if (t0 + w < te) store_elem<DT>(M, (int64_t)(t0 + w) * ldM + i0 + lane, tile[lane][w], inv);
+            }
         }
         __syncthreads();
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        double v = warp_sum(acc[j]);
-        const int64_t i = i0 + ty + 8 * j;
-        if (tx == 0 && i < n) sqpart[(int64_t)slice * n + i] = v;
-    }
+    double v[1] = {q.total()};
+    block_sum<1, kTransThreads>(v, red);
+    if (threadIdx.x == 0 && i0 < n) sqpart[(i0 / kTile) * slices + slice] = v[0];
 }
 
-// trace(Sigma) = sum_i rowsq_i, each rowsq_i the sum of its `parts` slice
-// partials (parts = 1 for the n x T layout), in a fixed order.
+// trace(Sigma): the sum of the blocks' partials, in a fixed order.
 __global__ void __launch_bounds__(kCenterThreads)
-trace_kernel(const double *__restrict__ rowsq, int64_t n, int parts, double *__restrict__ trace) {
+trace_kernel(const double *__restrict__ part, int64_t count, double *__restrict__ trace) {
     __shared__ double red[(kCenterThreads / kWarp + 1) * 1];
     double s[1] = {0.0};
-    for (int64_t i = threadIdx.x; i < n; i += kCenterThreads) {
-        double r = 0.0;
-        for (int k = 0; k < parts; ++k) r += rowsq[(int64_t)k * n + i];
-        s[0] += r;
-    }
+    for (int64_t i = threadIdx.x; i < count; i += kCenterThreads) s[0] += part[i];
     block_sum<1, kCenterThreads>(s, red);
     if (threadIdx.x == 0) *trace = s[0];
 }
 
 // Centering of the asset rows [i0, i1) of R, whose row i0 is at R_rows.
 // The last chunk of the transposed layout also zero-fills columns n..ldL-1.
-// Period slices of the transposed write: about 8 blocks per SM over the
-// asset tiles of a chunk of `rows` assets.
+// Period slices of the transposed write: about 32 blocks per SM over the
+// asset tiles of a chunk of `rows` assets (several waves, so that the last
+// one costs little).
 static int center_slices(int64_t rows, int64_t T) {
     const int64_t tiles = (rows + kTile - 1) / kTile;
-    int64_t sl = (8 * 152 + tiles - 1) / tiles;
-    const int64_t max_by_T = (T + kTile - 1) / kTile;
+    int64_t sl = (32 * 152 + tiles - 1) / tiles;
+    const int64_t max_by_T = (T + kTileT - 1) / kTileT;
     sl = sl < 1 ? 1 : (sl > kMaxSlices ? kMaxSlices : sl);
     return (int)(sl < max_by_T ? sl : max_by_T);
 }
 
 static void center_chunk(const float *R_rows, int64_t ldR, int64_t n, int64_t T, int out_dtype, bool tn, void *d_L,
-                         int64_t ldL, float *d_row_scale, double *d_mu, double *rowsq, int64_t i0, int64_t i1,
-                         int slices, cudaStream_t s) {
+                         int64_t ldL, float *d_row_scale, double *d_mu, double *rowsq, float *amax, int64_t i0,
+                         int64_t i1, int slices, cudaStream_t s) {
     const unsigned rows = (unsigned)(i1 - i0);
     const int64_t wend = (tn && i1 == n) ? ldL : i1;          // transposed: columns written by this chunk
     const dim3 tgrid((unsigned)slices, (unsigned)((wend - i0 + kTile - 1) / kTile));
 #define MV_CENTER_CASE(DT, RS)                                                                                   \
     if (tn) {                                                                                                    \
-        center_kernel<DT, false><<<rows, kCenterThreads, 0, s>>>(R_rows, ldR, (int)T, nullptr, 0, RS, d_mu,      \
-                                                                 rowsq, i0);                                     \
-        transpose_center_kernel<DT><<<tgrid, kTile * 8, 0, s>>>(R_rows, ldR, n, (int)T, d_L, ldL, RS, d_mu,      \
-                                                                rowsq, i0, slices);                              \
+        center_kernel<DT, false><<<rows, kCenterThreads, 0, s>>>(R_rows, ldR, (unsigned)T, nullptr, 0, RS, d_mu, \
+                                                                 rowsq, amax, i0);                               \
+        transpose_center_kernel<DT><<<tgrid, kTransThreads, 0, s>>>(R_rows, ldR, n, (int)T, d_L, ldL, RS, d_mu,  \
+                                                                    amax, rowsq, i0, slices);                    \
     } else {                                                                                                     \
-        center_kernel<DT, true><<<rows, kCenterThreads, 0, s>>>(R_rows, ldR, (int)T, d_L, ldL, RS, d_mu, rowsq,  \
-                                                                i0);                                             \
+        center_kernel<DT, true><<<rows, kCenterThreads, 0, s>>>(R_rows, ldR, (unsigned)T, d_L, ldL, RS, d_mu,    \
+                                                                rowsq, amax, i0);                                \
     }
     switch (out_dtype) {
         case MV_F32: MV_CENTER_CASE(MV_F32, nullptr) break;
@@ -212,6 +411,11 @@ static int center_args(const void *R, int64_t n, int64_t T, int64_t ldR, int out
     return MV_OK;
 }
 
+// Workspace: the partial sums of squares (one per row, or per asset tile and
+// slice), then the rows' largest |R| (transposed output).
+static size_t center_amax_offset(int64_t n) { return align_up((size_t)((n + kTile - 1) / kTile) * kMaxSlices * 8, 256); }
+static int64_t center_partials(int64_t n, bool tn, int slices) { return tn ? (n + kTile - 1) / kTile * slices : n; }
+
 // Chunked host-to-device pipeline of mv_center_factor_host.
 constexpr int64_t kHostChunkBytes = 64ll << 20;
 
@@ -230,7 +434,7 @@ extern "C" {
 
 size_t mv_center_workspace_size(int64_t n, int64_t T) {
     (void)T;
-    return n > 0 ? align_up((size_t)n * 8 * kMaxSlices, 256) : 0;
+    return n > 0 ? std::max(align_up((size_t)n * 8 * kMaxSlices, 256), center_amax_offset(n) + align_up(4 * (size_t)n, 256)) : 0;
 }
 
 int mv_center_factor(const float *d_R, int64_t n, int64_t T, int64_t ldR, int out_dtype, int layout, void *d_L,
@@ -243,9 +447,10 @@ int mv_center_factor(const float *d_R, int64_t n, int64_t T, int64_t ldR, int ou
     cudaStream_t s = (cudaStream_t)stream;
     const bool tn = layout == MV_LAYOUT_TN;
     double *rowsq = reinterpret_cast<double *>(d_ws);
+    float *amax = reinterpret_cast<float *>(reinterpret_cast<char *>(d_ws) + center_amax_offset(n));
     const int slices = center_slices(n, T);
-    center_chunk(d_R, ldR, n, T, out_dtype, tn, d_L, ldL, d_row_scale, d_mu, rowsq, 0, n, slices, s);
-    trace_kernel<<<1, kCenterThreads, 0, s>>>(rowsq, n, tn ? slices : 1, d_trace);
+    center_chunk(d_R, ldR, n, T, out_dtype, tn, d_L, ldL, d_row_scale, d_mu, rowsq, amax, 0, n, slices, s);
+    trace_kernel<<<1, kCenterThreads, 0, s>>>(rowsq, center_partials(n, tn, slices), d_trace);
     MV_CUDA_TRY(cudaGetLastError());
     return MV_OK;
 }
@@ -269,6 +474,7 @@ int mv_center_factor_host(const float *h_R, int64_t n, int64_t T, int64_t ldR, i
     const int slices = center_slices(m, T);
     char *ws = reinterpret_cast<char *>(d_ws);
     double *rowsq = reinterpret_cast<double *>(ws);
+    float *amax = reinterpret_cast<float *>(ws + center_amax_offset(n));
     const size_t o_stage = mv_center_workspace_size(n, T), stage_bytes = align_up((size_t)m * (size_t)T * 4, 256);
     float *stage[2] = {reinterpret_cast<float *>(ws + o_stage), reinterpret_cast<float *>(ws + o_stage + stage_bytes)};
     // The copies run on a stream of their own, one chunk ahead of the kernels.
@@ -295,11 +501,11 @@ int mv_center_factor_host(const float *h_R, int64_t n, int64_t T, int64_t ldR, i
         if (st == MV_OK && cudaEventRecord(copied[b], cs) != cudaSuccess) st = MV_ERR_CUDA;
         if (st == MV_OK && cudaStreamWaitEvent(s, copied[b], 0) != cudaSuccess) st = MV_ERR_CUDA;
         if (st == MV_OK) {
-            center_chunk(stage[b], T, n, T, out_dtype, tn, d_L, ldL, d_row_scale, d_mu, rowsq, i0, i1, slices, s);
+            center_chunk(stage[b], T, n, T, out_dtype, tn, d_L, ldL, d_row_scale, d_mu, rowsq, amax, i0, i1, slices, s);
             if (cudaEventRecord(used[b], s) != cudaSuccess) st = MV_ERR_CUDA;
         }
     }
-    if (st == MV_OK) trace_kernel<<<1, kCenterThreads, 0, s>>>(rowsq, n, tn ? slices : 1, d_trace);
+    if (st == MV_OK) trace_kernel<<<1, kCenterThreads, 0, s>>>(rowsq, center_partials(n, tn, slices), d_trace);
     // `stream` waits for every copy before the events and the copy stream go away.
     cudaEvent_t fin;
     if (cudaEventCreateWithFlags(&fin, cudaEventDisableTiming) == cudaSuccess) {
