@@ -23,6 +23,8 @@ struct FState {
     int k, done, converged, status;
     int proj_fail, proj_steps, pad0, pad1;
     double t, beta_prev, kkt, nu, tau, nu_kkt, tau_kkt, objective;
+    double inv1pb;              // 1 / (1 + beta_prev)
+    ScaleHint hint;             // scales of the last projection
 };
 
 struct FArgs {
@@ -75,6 +77,8 @@ __global__ void __launch_bounds__(kProjNT) frontier_init_kernel(FArgs a) {
     if (rank == 0 && threadIdx.x == 0) {
         FState f{};
         f.t = 1.0;
+        f.inv1pb = 1.0;
+        f.hint = P.scales();
         f.nu = f.nu_kkt = o.nu;
         f.tau = f.tau_kkt = o.tau;
         f.kkt = INFINITY;
@@ -89,26 +93,28 @@ template <int CL>
 __global__ void __launch_bounds__(kProjNT) frontier_step_kernel(FArgs a) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ ProjSmem psm;
-    __shared__ double sc[4];
+    __shared__ double sc[3];
     const int b = blockIdx.x / CL, rank = cluster_rank<CL>();
     FState *fs = a.fs + b;
     if (*(volatile int *)&fs->done) return;      // uniform over the cluster (see npga_step_kernel)
     const int n = a.n, nl = (n + CL - 1) / CL, r0 = min(n, rank * nl), r1 = min(n, r0 + nl);
     const int k = fs->k;
-    const double beta_prev = fs->beta_prev, t = fs->t, alpha = a.st->alpha;
+    const double beta_prev = fs->beta_prev, inv1pb = fs->inv1pb, t = fs->t, alpha = a.st->alpha;
     const double mn = a.st->mu_min, mx = a.st->mu_max;
     const double nu0 = fs->nu, tau0 = fs->tau;
+    const ScaleHint hint = fs->hint;
     const double gamma = a.gamma, R = a.Rt[b];
-    if (threadIdx.x == 0) {
-        sc[0] = 1.0 / (1.0 + beta_prev);
-        const double tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
-        sc[1] = tn;
-        sc[2] = (t - 1.0) / tn;
-    }
+    auto momentum = [&] {                        // beside the projection's scalar logic (see npga_step_body)
+        if (threadIdx.x == kProjNT - kWarp) {
+            const double tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t)), beta = (t - 1.0) / tn;
+            sc[0] = tn;
+            sc[1] = beta;
+            sc[2] = 1.0 / (1.0 + beta);
+        }
+    };
     ProjElems el = carve_elems(dsm, nl);
     el.n = r1 - r0;
     proj_smem_init(&psm);
-    const double inv1pb = sc[0], tn = sc[1], beta = sc[2];
     const bool check = (a.kkt_every > 0 && k % a.kkt_every == 0) || (k >= a.max_iter);
     double *Xb = a.X + (int64_t)b * n, *Yb = a.Y + (int64_t)b * n, *GXb = a.GX + (int64_t)b * n;
     for (int i = threadIdx.x; i < el.n; i += kProjNT) {
@@ -126,7 +132,7 @@ __global__ void __launch_bounds__(kProjNT) frontier_step_kernel(FArgs a) {
     __syncthreads();
     ClusterProj<CL> P{&psm, el};
     if (check) {
-        P.prepare();
+        P.prepare(hint);
         const ProjOut o = P.solve(R, a.mode, mn, mx, nu0, tau0, kProjBudget);   // see npga_step_body
         double r2 = 0.0;
         for (int i = threadIdx.x; i < el.n; i += kProjNT) {
@@ -163,8 +169,9 @@ __global__ void __launch_bounds__(kProjNT) frontier_step_kernel(FArgs a) {
         el.v[i] = yi - alpha * (2.0 * gyi + 2.0 * gamma * yi);
     }
     __syncthreads();
-    P.prepare();
-    const ProjOut o = P.solve(R, a.mode, mn, mx, nu0, tau0, kProjBudget);
+    P.prepare(hint);
+    const ProjOut o = P.solve(R, a.mode, mn, mx, nu0, tau0, kProjBudget, momentum);
+    const double beta = sc[1];
     for (int i = threadIdx.x; i < el.n; i += kProjNT) {
         const int gi = r0 + i;
         const double xn = fmax(fma(o.nu, el.mu[i], el.v[i]) - o.tau, 0.0);
@@ -175,8 +182,10 @@ __global__ void __launch_bounds__(kProjNT) frontier_step_kernel(FArgs a) {
         write_split(a.Ysplit, a.ldY, a.B, b, gi, yn, a.row_scale);
     }
     if (rank == 0 && threadIdx.x == 0) {
-        fs->t = tn;
+        fs->t = sc[0];
         fs->beta_prev = beta;
+        fs->inv1pb = sc[2];
+        fs->hint = P.scales();
         fs->k = k + 1;
         fs->nu = o.nu;
         fs->tau = o.tau;
@@ -243,6 +252,7 @@ __global__ void frontier_warm_kernel(FState *fs, const double *__restrict__ X, d
         f.status = MV_OK;
         f.t = 1.0;
         f.beta_prev = 0.0;
+        f.inv1pb = 1.0;
         f.kkt = INFINITY;
     }
 }

@@ -24,10 +24,10 @@
 //    of the FP64 values (62-bit magnitudes scaled by the largest element,
 //    converted with integer bit operations, so each image carries the full
 //    FP64 mantissa), so no FP64 add runs per element or in the reduction
-//    tree and the sums are at least as accurate as FP64 ones.  A thread
-//    keeps each image as four 16-bit limbs summed in 32-bit registers; a
-//    warp adds each limb with one redux.sync, and the limbs are recombined
-//    into 128 bits only for the few cross-warp and cross-block additions;
+//    tree and the sums are at least as accurate as FP64 ones.  An image is
+//    three 21-bit limbs; a thread's and a warp's limb sums fit 32 bits (one
+//    redux.sync each), a block's too, and only the cluster totals are
+//    recombined;
 //  * membership w_i > tau is decided in FP32 with a proven error margin;
 //    only elements inside the margin repeat the test in FP64 (same result as
 //    an FP64 evaluation of fma(nu, mu_i, v_i) > tau);
@@ -41,11 +41,18 @@
 // Warm-start shortcut: the support S0 at the hint gives, from the same
 // reduction, the exact solution (nu*, tau*) of the budget and return rows on
 // S0 (tau* alone at nu = 0 when the hint says the return row is inactive).
-// The next reduction, at (nu*, tau*), also counts the elements whose
-// membership differs from S0; none means S0 is the support at (nu*, tau*),
-// so (nu*, tau*) is exact and the search ends after two reductions (the
-// general search needs four when the support does not move).  Otherwise the
-// general search continues from (nu*, tau*).
+// A second, much lighter exchange only asks whether any element's membership
+// at (nu*, tau*) differs from S0 (each thread kept its elements' bits); none
+// means S0 is the support at (nu*, tau*), so (nu*, tau*) is exact and the
+// search ends (the general search needs four reductions when the support
+// does not move).  Otherwise the general search continues from (nu*, tau*).
+// Scale hint: the fixed-point scales follow from the cluster maxima of four
+// exponents, which would cost an exchange of their own before the first
+// reduction.  A caller that projects similar points again and again (the
+// solve loops) passes the exponents of its last projection: the images are
+// made with those and the true maxima travel with the first reduction, which
+// is repeated in the rare case that one of them moved.  The images, and so
+// the results, are the same either way.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -96,69 +103,39 @@ __device__ __forceinline__ double pow2_neg(int s) {
 // Scale s such that every |q| whose exponent field is <= e satisfies |q| 2^s < 2^kFixBits.
 __host__ __device__ __forceinline__ int fixed_scale(int e) { return e == 0 ? 0 : kFixBits + 1022 - e; }
 
-// Signed 128-bit accumulator (two's complement, lo word unsigned).
-struct I128 {
-    unsigned long long lo;
-    long long hi;
-};
-__device__ __forceinline__ void add128(I128 &a, long long x) {
-    const unsigned long long nlo = a.lo + (unsigned long long)x;
-    a.hi += (x >> 63) + (nlo < a.lo ? 1 : 0);
-    a.lo = nlo;
+// Warp-wide sum and maximum of a 32-bit integer (one instruction).
+__device__ __forceinline__ int redux_add(int v) { return __reduce_add_sync(0xffffffffu, v); }
+__device__ __forceinline__ int redux_max(int v) { return __reduce_max_sync(0xffffffffu, v); }
+// Adds the three 21-bit limbs of a fixed-point image (|x| < 2^62: the top
+// limb, arithmetic, lies in [-2^20, 2^20)) to per-thread 32-bit sums.  Eight
+// elements per thread (kProjMaxLocal) and 32 lanes stay below 2^29, a block
+// of kProjMaxLocal below 2^32 (the top limb within int32).
+__device__ __forceinline__ void add_limbs(int (&l)[3], long long x) {
+    l[0] += (int)x & 0x1fffff;
+    l[1] += (int)(x >> 21) & 0x1fffff;
+    l[2] += (int)(x >> 42);
 }
-__device__ __forceinline__ void add128(I128 &a, const I128 &b) {
-    const unsigned long long nlo = a.lo + b.lo;
-    a.hi += b.hi + (nlo < a.lo ? 1 : 0);
-    a.lo = nlo;
-}
-__device__ __forceinline__ double i128_to_double(const I128 &a) {
-    return (double)a.hi * 18446744073709551616.0 + (double)a.lo;
-}
-__device__ __forceinline__ I128 warp_sum_128(I128 v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        I128 w;
-        w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-        w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-        add128(v, w);
-    }
-    return v;
-}
-// Warp-wide sum of a 32-bit integer (one instruction).
-__device__ __forceinline__ int redux_add(int v) {
-    int r;
-    asm volatile("redux.sync.add.s32 %0, %1, 0xffffffff;" : "=r"(r) : "r"(v));
-    return r;
-}
-// v * 2^s as a 128-bit value, s in {0, 16, 32, 48}.
-__device__ __forceinline__ I128 shl128(long long v, int s) {
-    I128 r;
-    r.lo = (unsigned long long)v << s;
-    r.hi = s == 0 ? (v >> 63) : (v >> (64 - s));
-    return r;
-}
-// Adds the four 16-bit limbs of a fixed-point image (|x| < 2^62: the top
-// limb, arithmetic, lies in [-2^14, 2^14]) to per-thread 32-bit sums.
-__device__ __forceinline__ void add_limbs(int (&l)[4], long long x) {
-    l[0] += (int)(x & 0xffff);
-    l[1] += (int)((x >> 16) & 0xffff);
-    l[2] += (int)((x >> 32) & 0xffff);
-    l[3] += (int)(x >> 48);
-}
-// Recombines warp totals of the four limbs.
-__device__ __forceinline__ I128 from_limbs(const int (&t)[4]) {
-    I128 r = shl128(t[0], 0);
-    add128(r, shl128(t[1], 16));
-    add128(r, shl128(t[2], 32));
-    add128(r, shl128(t[3], 48));
-    return r;
+// The value of cluster-wide limb totals (l0, l1 < 2^36; |l2| < 2^35).
+__device__ __forceinline__ double from_limbs(long long l0, long long l1, long long l2) {
+    return fma((double)l2, 4398046511104.0, (double)((l1 << 21) + l0));
 }
 
 // Cluster totals of one support step, as thread 0 of every block holds them.
 struct SupportSums {
     double cnt, sv, sm, smv, smm;
-    long long nan, diff;
+    int nan;
 };
+
+// Exponent fields of the last projection's scales (v, mu, mu v, mu^2); e[0] < 0: none.
+struct ScaleHint {
+    int e[4];
+};
+
+// Words a block contributes to a reduction: 0 |S|, 1 + 3q + l limb l of
+// image q (v, mu, mu v, mu^2), 13 NaNs met, 14 and 15 the largest exponent
+// fields of v and mu v (maxima, not sums).
+constexpr int kProjWords = 16;
+constexpr int kProjNW = kProjNT / kWarp;
 
 struct ProjOut {
     double nu, tau;
@@ -169,21 +146,20 @@ struct ProjOut {
 
 // Shared-memory workspace of one block of the projector.
 struct ProjSmem {
-    I128 part[2][kProjMaxCL][6];        // DSMEM slots: [parity][source rank][sum]
+    alignas(16) int part[2][kProjMaxCL][kProjWords];   // DSMEM slots: [parity][source rank][word]
+    alignas(16) int wred[kProjNW][kProjWords];         // per-warp words
+    alignas(16) int moved[kProjMaxCL];                 // verifying exchange: source rank's membership changes
     double dpart[2][kProjMaxCL];
     int emax[kProjMaxCL][4];
-    I128 wred[kProjNT / kWarp][6];
-    double wredd[kProjNT / kWarp];
-    int wmax[kProjNT / kWarp][4];
-    // broadcast of the scalar state (written by thread 0)
+    double wredd[kProjNW], wredm[kProjNW];
+    int wmax[kProjNW][4];
+    // broadcast of the scalar state (written by warp 0)
     double nu, tau, dbcast, dmin, dmax;
     double mpart[2][kProjMaxCL][2];
     float nu32, tau32;
-    double nu0, tau0;                   // hint whose support a verifying step compares against
-    float nu032, tau032;
-    int verify;
+    int verify, redo;
     int done, status, steps;
-    int s_v, s_m, s_mv, s_mm;
+    int e[4];                           // exponent fields the scales follow from
     double p_v, p_m, p_mv, p_mm;        // 2^-s of the four scales
     int parity;
 };
@@ -193,6 +169,7 @@ __device__ inline void proj_smem_init(ProjSmem *sh) {
     if (threadIdx.x == 0) {
         sh->parity = 0;
         sh->verify = 0;
+        sh->redo = 0;
     }
     __syncthreads();
 }
@@ -231,11 +208,6 @@ __device__ inline ProjElems carve_elems(void *base, int n_local) {
     return e;
 }
 
-__device__ __forceinline__ long long warp_sum_ll(long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 __device__ __forceinline__ int warp_max_i(int v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -268,48 +240,80 @@ struct ClusterProj {
     // (v, x, p, q) and the sweep budget; without scratch the safeguard is off.
     double *dyk = nullptr;
     int dyk_iters = 0;
+    // Per thread: membership bits of its elements at the last reduction's
+    // point, and, while the scales rest on a hint, its largest exponent
+    // fields of v and mu v.
+    unsigned in_bits = 0;
+    int my_ev = 0, my_emv = 0;
+    bool hinted = false;
 
-    // Block-then-cluster sum of the 6 per-warp 128-bit partials in
-    // sh->wred (after a __syncthreads); lane k < 6 of warp 0 of every block
-    // ends with total k (integer sums: exact, so the order of addition does
-    // not matter).  Lane k < 6 adds value k over the warps, lane r < CL
-    // stores the block totals into block r, then lane k adds value k over
-    // the CL blocks.
-    __device__ I128 reduce_partials() {
+    // Block-then-cluster total of the per-warp words in sh->wred (after a
+    // __syncthreads): lane k of warp 0 of every block ends with the total of
+    // word k mod 16 (integer sums and maxima: exact, so the order does not
+    // matter).  Two lanes share a word, each taking half of the warps and
+    // half of the ranks; the words go out as 16-byte pieces, two per lane.
+    __device__ long long reduce_partials() {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         const int par = sh->parity;
-        I128 t{0ull, 0ll};
+        const int word = lane & (kProjWords - 1), half = lane / kProjWords;
+        const bool is_max = word >= 14;
+        auto join = [&](long long a, long long b) { return is_max ? (a > b ? a : b) : a + b; };
+        long long t = 0;
         if (warp == 0) {
-            if (lane < 6)
-                for (int w = 0; w < kProjNT / kWarp; ++w) add128(t, sh->wred[w][lane]);
-            const int me = cluster_rank<CL>();
-            I128 tk[6];
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                tk[k].lo = __shfl_sync(0xffffffffu, t.lo, k);
-                tk[k].hi = __shfl_sync(0xffffffffu, t.hi, k);
-            }
-            if (lane < CL) {
-                I128 *dst;
-                if constexpr (CL > 1) {
-                    dst = cg::this_cluster().map_shared_rank(&sh->part[par][me][0], lane);
-                } else {
-                    dst = &sh->part[par][0][0];
-                }
-#pragma unroll
-                for (int k = 0; k < 6; ++k) dst[k] = tk[k];
-            }
-        }
-        cluster_barrier<CL>();
-        t = I128{0ull, 0ll};
-        if (warp == 0) {
-            if (lane < 6)
-                for (int r = 0; r < CL; ++r) add128(t, sh->part[par][r][lane]);
+            for (int w = 0; w < kProjNW / 2; ++w) t = join(t, (long long)sh->wred[half * (kProjNW / 2) + w][word]);
+            t = join(t, __shfl_xor_sync(0xffffffffu, t, kProjWords));
             if (lane == 0) sh->parity = par ^ 1;
         }
-        // The next exchange writes the other parity; the one after reuses this
-        // one only after another cluster barrier, so no reader is overtaken.
+        // One block: no barrier here.  Warp 0's reads of wred come before the
+        // block barrier that follows in every caller, and so before the next
+        // reduction's writes.
+        if constexpr (CL > 1) {
+            if (warp == 0) {
+                const int me = cluster_rank<CL>();
+                if (lane < kProjWords) sh->part[par][me][word] = (int)(unsigned)t;   // limbs 0, 1 as unsigned
+                __syncwarp();
+                cg::cluster_group cl = cg::this_cluster();
+                int4 *src = reinterpret_cast<int4 *>(&sh->part[par][me][0]);
+                for (int p = lane; p < CL * (kProjWords / 4); p += kWarp) {
+                    const int r = p / (kProjWords / 4), q = p % (kProjWords / 4);
+                    if (r != me) *cl.map_shared_rank(src + q, r) = src[q];
+                }
+            }
+            cluster_barrier<CL>();
+            t = 0;
+            if (warp == 0) {
+                // limbs 0 and 1 of an image are unsigned block totals, every other word is signed
+                const bool uns = word >= 1 && word <= 12 && (word - 1) % 3 != 2;
+#pragma unroll
+                for (int r = 0; r < CL / 2; ++r) {
+                    const int x = sh->part[par][half * (CL / 2) + r][word];
+                    t = join(t, uns ? (long long)(unsigned)x : (long long)x);
+                }
+                t = join(t, __shfl_xor_sync(0xffffffffu, t, kProjWords));
+            }
+            // The next exchange writes the other parity; the one after reuses this
+            // one only after another cluster barrier, so no reader is overtaken.
+        }
         return t;
+    }
+
+    // Whether any thread of the cluster passes a nonzero x; one barrier.
+    // Its slots are rewritten only by the next call, with at least one full
+    // reduction (a cluster barrier) between two calls.
+    __device__ bool any_of(int x) {
+        if constexpr (CL == 1) {
+            return __syncthreads_or(x) != 0;
+        } else {
+            const int any = __syncthreads_or(x);
+            if (threadIdx.x < CL)
+                *cg::this_cluster().map_shared_rank(&sh->moved[cluster_rank<CL>()], (int)threadIdx.x) = any;
+            cluster_barrier<CL>();
+            int t = 0;
+#pragma unroll
+            for (int r = 0; r < CL; ++r) t |= sh->moved[r];
+            return t != 0;
+        }
     }
 
     // Cluster sum of one double per thread, added in a fixed order (every
@@ -320,23 +324,26 @@ struct ClusterProj {
         if (lane == 0) sh->wredd[warp] = x;
         __syncthreads();
         const int par = sh->parity;
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < kProjNT / kWarp; ++w) t += sh->wredd[w];
-            const int me = cluster_rank<CL>();
-            if constexpr (CL > 1) {
-                cg::cluster_group cl = cg::this_cluster();
-                for (int r = 0; r < CL; ++r) *cl.map_shared_rank(&sh->dpart[par][me], r) = t;
-            } else {
-                sh->dpart[par][0] = t;
+        if (warp == 0) {
+            double t = lane < kProjNW ? sh->wredd[lane] : 0.0;
+#pragma unroll
+            for (int o = kProjNW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            t = __shfl_sync(0xffffffffu, t, 0);
+            if (lane < CL) {
+                double *dst = &sh->dpart[par][cluster_rank<CL>()];
+                if constexpr (CL > 1) dst = cg::this_cluster().map_shared_rank(dst, lane);
+                *dst = t;
             }
         }
         cluster_barrier<CL>();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int r = 0; r < CL; ++r) t += sh->dpart[par][r];
-            sh->dbcast = t;
-            sh->parity = par ^ 1;
+        if (warp == 0) {
+            double t = lane < CL ? sh->dpart[par][lane] : 0.0;
+#pragma unroll
+            for (int o = CL / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) {
+                sh->dbcast = t;
+                sh->parity = par ^ 1;
+            }
         }
         __syncthreads();
         const double r = sh->dbcast;
@@ -351,15 +358,15 @@ struct ClusterProj {
         mx = warp_max(mx);
         if (lane == 0) {
             sh->wredd[warp] = mn;
-            sh->wred[warp][0].hi = __double_as_longlong(mx);
+            sh->wredm[warp] = mx;
         }
         __syncthreads();
         const int par = sh->parity;
         if (threadIdx.x == 0) {
             double a = INFINITY, b = -INFINITY;
-            for (int w = 0; w < kProjNT / kWarp; ++w) {
+            for (int w = 0; w < kProjNW; ++w) {
                 a = fmin(a, sh->wredd[w]);
-                b = fmax(b, __longlong_as_double(sh->wred[w][0].hi));
+                b = fmax(b, sh->wredm[w]);
             }
             const int me = cluster_rank<CL>();
             if constexpr (CL > 1) {
@@ -389,6 +396,60 @@ struct ClusterProj {
         mn = sh->dmin;
         mx = sh->dmax;
         __syncthreads();
+    }
+
+    // The scales of the exponent fields sh->e (thread 0), for the conversions
+    // of the totals.
+    __device__ void set_scales() {
+        sh->p_v = pow2_neg(fixed_scale(sh->e[0]));
+        sh->p_m = pow2_neg(fixed_scale(sh->e[1]));
+        sh->p_mv = pow2_neg(fixed_scale(sh->e[2]));
+        sh->p_mm = pow2_neg(fixed_scale(sh->e[3]));
+    }
+
+    // prepare() on the scales of `hint` (none: the plain form).  The largest
+    // exponent fields this thread meets go into the first reduction.
+    __device__ void prepare(const ScaleHint &hint) {
+        if (hint.e[0] < 0) {
+            prepare();
+            return;
+        }
+        const int s0 = fixed_scale(hint.e[0]), s1 = fixed_scale(hint.e[1]), s2 = fixed_scale(hint.e[2]),
+                  s3 = fixed_scale(hint.e[3]);
+        my_ev = my_emv = 0;
+        for (int i = threadIdx.x; i < el.n; i += kProjNT) {
+            const double v = el.v[i], m = el.mu[i];
+            const double mv = m * v;
+            my_ev = max(my_ev, exp_field(v));
+            my_emv = max(my_emv, exp_field(mv));
+            el.V[i] = to_fixed(v, s0);
+            el.M[i] = to_fixed(m, s1);
+            el.MV[i] = to_fixed(mv, s2);
+            el.MM[i] = to_fixed(m * m, s3);
+            el.v32[i] = (float)v;
+            el.mu32[i] = (float)m;
+        }
+        hinted = true;
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sh->e[k] = hint.e[k];
+            set_scales();
+        }
+    }
+    // Images of v and mu v again, on the scales of sh->e (a hint that did not hold).
+    __device__ void rescale() {
+        const int s0 = fixed_scale(sh->e[0]), s2 = fixed_scale(sh->e[2]);
+        for (int i = threadIdx.x; i < el.n; i += kProjNT) {
+            el.V[i] = to_fixed(el.v[i], s0);
+            el.MV[i] = to_fixed(el.mu[i] * el.v[i], s2);
+        }
+    }
+    // The exponent fields behind the present scales.
+    __device__ ScaleHint scales() const {
+        ScaleHint h;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) h.e[k] = sh->e[k];
+        return h;
     }
 
     // Cluster-wide maxima of the exponent fields of |v|, |mu|, |mu v|, mu^2,
@@ -438,18 +499,14 @@ struct ClusterProj {
             for (int r = 0; r < CL; ++r)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) t[k] = max(t[k], sh->emax[r][k]);
-            sh->s_v = fixed_scale(t[0]);
-            sh->s_m = fixed_scale(t[1]);
-            sh->s_mv = fixed_scale(t[2]);
-            sh->s_mm = fixed_scale(t[3]);
-            // 2^-s as exact doubles (s in [-10, 2100]: build the bits, clamp to 0)
-            sh->p_v = pow2_neg(sh->s_v);
-            sh->p_m = pow2_neg(sh->s_m);
-            sh->p_mv = pow2_neg(sh->s_mv);
-            sh->p_mm = pow2_neg(sh->s_mm);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sh->e[k] = t[k];
+            set_scales();
         }
         __syncthreads();
-        const int sv = sh->s_v, sm = sh->s_m, smv = sh->s_mv, smm = sh->s_mm;
+        hinted = false;
+        const int sv = fixed_scale(sh->e[0]), sm = fixed_scale(sh->e[1]), smv = fixed_scale(sh->e[2]),
+                  smm = fixed_scale(sh->e[3]);
         for (int i = threadIdx.x; i < el.n; i += kProjNT) {
             el.V[i] = to_fixed(el.v[i], sv);
             el.M[i] = to_fixed(el.mu[i], sm);
@@ -476,131 +533,156 @@ struct ClusterProj {
         return w > tau;
     }
 
-    // Sums over S = {i : fma(nu, mu_i, v_i) > tau}; totals valid in thread 0.
-    // Also counts NaNs met and (when sh->verify) the elements whose
-    // membership differs from S(sh->nu0, sh->tau0).
+    // Sums over S = {i : fma(nu, mu_i, v_i) > tau}; totals valid in warp 0
+    // (all lanes).  Leaves the thread's membership bits in in_bits.
     __device__ SupportSums support_sums(double nu, double tau, float nu32, float tau32) {
-        int lb[4][4];
+        while (true) {
+            int lb[4][3];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
+            for (int k = 0; k < 4; ++k)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) lb[k][q] = 0;
-        int cnt = 0, diff = 0;
+                for (int q = 0; q < 3; ++q) lb[k][q] = 0;
+            const float anu = fabsf(nu32), atau = isinf(tau32) ? 0.f : fabsf(tau32);
+            bool nan = false;
+            in_bits = 0;
+            unsigned bit = 1;
+            for (int i = threadIdx.x; i < el.n; i += kProjNT, bit <<= 1) {
+                if (member(i, nu, tau, nu32, tau32, anu, atau, nan)) {
+                    in_bits |= bit;
+                    add_limbs(lb[0], el.V[i]);
+                    add_limbs(lb[1], el.M[i]);
+                    add_limbs(lb[2], el.MV[i]);
+                    add_limbs(lb[3], el.MM[i]);
+                }
+            }
+            const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+            __syncwarp();
+            // |S| and the NaN count share a word: at most 256 of each per warp
+            const int cn = redux_add(__popc(in_bits) + (nan ? 1 << 16 : 0));
+            int mine = lane == 0 ? (cn & 0xffff) : (lane == 13 ? cn >> 16 : 0);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int t = redux_add(lb[k][q]);
+                    mine = lane == 1 + 3 * k + q ? t : mine;
+                }
+            if (hinted) {
+                const int a = redux_max(my_ev), b = redux_max(my_emv);
+                mine = lane == 14 ? a : (lane == 15 ? b : mine);
+            }
+            if (lane < kProjWords) sh->wred[warp][lane] = mine;
+            __syncthreads();
+            const long long t = reduce_partials();
+            if (hinted) {
+                hinted = false;
+                if (warp == 0) {
+                    const bool moved = (lane == 14 && t != sh->e[0]) || (lane == 15 && t != sh->e[2]);
+                    const bool redo = __any_sync(0xffffffffu, moved);
+                    const int ev = (int)__shfl_sync(0xffffffffu, t, 14), emv = (int)__shfl_sync(0xffffffffu, t, 15);
+                    if (lane == 0) {
+                        sh->redo = redo;
+                        if (redo) {
+                            sh->e[0] = ev;
+                            sh->e[2] = emv;
+                            set_scales();
+                        }
+                    }
+                }
+                __syncthreads();
+                if (sh->redo) {
+                    rescale();
+                    continue;
+                }
+            }
+            // lane k < 5 converts total k to FP64 (the four images with their scales)
+            SupportSums out{};
+            if (warp == 0) {
+                const int base = lane >= 1 && lane < 5 ? 1 + 3 * (lane - 1) : 1;
+                const long long l0 = __shfl_sync(0xffffffffu, t, base), l1 = __shfl_sync(0xffffffffu, t, base + 1),
+                                l2 = __shfl_sync(0xffffffffu, t, base + 2);
+                const double p = lane == 1 ? sh->p_v : (lane == 2 ? sh->p_m : (lane == 3 ? sh->p_mv : sh->p_mm));
+                const double d = lane == 0 ? (double)t : from_limbs(l0, l1, l2) * p;
+                out.cnt = __shfl_sync(0xffffffffu, d, 0);
+                out.sv = __shfl_sync(0xffffffffu, d, 1);
+                out.sm = __shfl_sync(0xffffffffu, d, 2);
+                out.smv = __shfl_sync(0xffffffffu, d, 3);
+                out.smm = __shfl_sync(0xffffffffu, d, 4);
+                out.nan = (int)__shfl_sync(0xffffffffu, t, 13);
+            }
+            return out;
+        }
+    }
+
+    // Whether the support at (nu, tau) is the one of the last reduction.
+    __device__ bool same_support(double nu, double tau, float nu32, float tau32) {
         const float anu = fabsf(nu32), atau = isinf(tau32) ? 0.f : fabsf(tau32);
-        const bool verify = sh->verify != 0;
-        const double nu0 = sh->nu0, tau0 = sh->tau0;
-        const float nu032 = sh->nu032, tau032 = sh->tau032;
-        const float anu0 = fabsf(nu032), atau0 = isinf(tau032) ? 0.f : fabsf(tau032);
         bool nan = false;
-        for (int i = threadIdx.x; i < el.n; i += kProjNT) {
-            const bool in = member(i, nu, tau, nu32, tau32, anu, atau, nan);
-            if (verify && in != member(i, nu0, tau0, nu032, tau032, anu0, atau0, nan)) ++diff;
-            if (in) {
-                ++cnt;
-                add_limbs(lb[0], el.V[i]);
-                add_limbs(lb[1], el.M[i]);
-                add_limbs(lb[2], el.MV[i]);
-                add_limbs(lb[3], el.MM[i]);
-            }
-        }
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        int tl[4][4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) tl[k][q] = redux_add(lb[k][q]);
-        const int tcnt = redux_add(cnt), tdiff = redux_add(diff), tnan = redux_add(nan ? 1 : 0);
-        if (lane < 6) {
-            I128 w;
-            if (lane == 0) {
-                w = I128{(unsigned long long)tcnt, 0ll};
-            } else if (lane == 5) {
-                w = I128{(unsigned long long)tnan, (long long)tdiff};
-            } else {
-                // lane k (1..4) recombines image k-1; the branch-free select keeps tl in registers
-                int t4[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    t4[q] = lane == 1 ? tl[0][q] : (lane == 2 ? tl[1][q] : (lane == 3 ? tl[2][q] : tl[3][q]));
-                w = from_limbs(t4);
-            }
-            sh->wred[warp][lane] = w;
-        }
-        __syncthreads();
-        const I128 t = reduce_partials();
-        // lane k converts total k to FP64 (the four images with their scales)
-        double d = 0.0;
-        if (warp == 0 && lane < 5) {
-            const double p = lane == 1 ? sh->p_v : (lane == 2 ? sh->p_m : (lane == 3 ? sh->p_mv : sh->p_mm));
-            d = lane == 0 ? (double)t.lo : i128_to_double(t) * p;
-        }
-        SupportSums out;
-        out.cnt = __shfl_sync(0xffffffffu, d, 0);
-        out.sv = __shfl_sync(0xffffffffu, d, 1);
-        out.sm = __shfl_sync(0xffffffffu, d, 2);
-        out.smv = __shfl_sync(0xffffffffu, d, 3);
-        out.smm = __shfl_sync(0xffffffffu, d, 4);
-        out.nan = (long long)__shfl_sync(0xffffffffu, t.lo, 5);
-        out.diff = __shfl_sync(0xffffffffu, t.hi, 5);
-        return out;
+        unsigned now = 0, bit = 1;
+        for (int i = threadIdx.x; i < el.n; i += kProjNT, bit <<= 1)
+            if (member(i, nu, tau, nu32, tau32, anu, atau, nan)) now |= bit;
+        return !any_of(now != in_bits);
     }
 
     // Full search.  Returns (nu, tau, status) identically in all threads.
+    // The scalar logic runs on warp 0 (every lane the same); `side` is run
+    // meanwhile by the last warp, once.
+    template <typename Side>
     __device__ ProjOut search(double R, int mode, double mu_min, double mu_max, double nu_hint, double tau_hint,
-                             int budget) {
-        // Thread-0-owned search state.
+                             int budget, const Side &side) {
+        // Search state of warp 0.
         double lo = -INFINITY, hi = INFINITY, nu = 0.0, tau = -INFINITY, prev_cnt = -1.0;
         bool have_lo = false, have_hi = false, zero_done = false, first = true;
-        bool try_fast = true, verifying = false;
+        bool try_fast = true, refuted = false, side_done = false;
         int outer = 0, inner = 0, status = MV_OK;
         const bool ge = (mode == MV_RETURN_GE);
-        if (threadIdx.x == 0) {
-            sh->steps = 0;
-            sh->done = 0;
-            sh->verify = 0;
-            if (!(R <= mu_max) || (!ge && !(R >= mu_min))) {
-                sh->done = 1;
-                sh->status = MV_ERR_INFEASIBLE;
-                sh->nu = NAN;
-                sh->tau = NAN;
-            } else {
+        if (threadIdx.x < kWarp) {
+            const bool infeasible = !(R <= mu_max) || (!ge && !(R >= mu_min));
+            if (!infeasible) {
                 nu = (nu_hint == nu_hint) ? nu_hint : 0.0;
                 if (ge && !(nu > 0.0)) nu = 0.0;
                 tau = (tau_hint == tau_hint) ? tau_hint : -INFINITY;
-                sh->nu = nu;
-                sh->tau = tau;
+            }
+            if (threadIdx.x == 0) {
+                sh->steps = 0;
+                sh->verify = 0;
+                sh->done = infeasible ? 1 : 0;
+                sh->status = infeasible ? MV_ERR_INFEASIBLE : MV_OK;
+                sh->nu = infeasible ? NAN : nu;
+                sh->tau = infeasible ? NAN : tau;
                 sh->nu32 = (float)nu;
                 sh->tau32 = (float)tau;
-                sh->status = MV_OK;
             }
         }
         __syncthreads();
         double scaleR = 0.0;
-        if (threadIdx.x == 0) scaleR = fmax(fabs(R), fmax(fabs(mu_max), fabs(mu_min)));
+        if (threadIdx.x < kWarp) scaleR = fmax(fabs(R), fmax(fabs(mu_max), fabs(mu_min)));
         while (true) {
             if (sh->done) break;                       // uniform: read after a barrier
             const double enu = sh->nu, etau = sh->tau;
             const float enu32 = sh->nu32, etau32 = sh->tau32;
+            if (sh->verify) {
+                // a candidate built on the support of the last reduction: exact iff the support is the same there
+                const bool same = same_support(enu, etau, enu32, etau32);
+                if (same) {
+                    if (threadIdx.x == 0) sh->steps += 1;
+                    break;                             // (nu, tau) and MV_OK stand in sh
+                }
+                refuted = true;
+            }
             const SupportSums S = support_sums(enu, etau, enu32, etau32);
-            if (threadIdx.x == 0) {
-                sh->steps += 1;
+            if (!side_done && threadIdx.x >= kProjNT - kWarp) side();
+            side_done = true;
+            if (threadIdx.x < kWarp) {
                 const double cnt = S.cnt, sv = S.sv, sm = S.sm, smv = S.smv, smm = S.smm;
-                bool finish = false, handled = false;
+                bool finish = false, handled = false, verify = false;
                 double next_nu = enu, next_tau = etau;
                 if (S.nan != 0) {
                     status = MV_ERR_NUMERIC;
                     finish = true;
                     handled = true;
-                } else if (verifying) {
-                    // the candidate was built on S(nu0, tau0); it is exact iff the support is unchanged
-                    verifying = false;
-                    sh->verify = 0;
-                    if (S.diff == 0) {
-                        nu = enu;
-                        tau = etau;
-                        finish = true;
-                        handled = true;
-                    }
+                } else if (refuted) {
+                    refuted = false;                   // the general search goes on from the candidate
                 } else if (try_fast && cnt > 0.0) {
                     try_fast = false;
                     const double a = cnt, b = sm, c = smm;
@@ -613,18 +695,20 @@ struct ClusterProj {
                     } else {
                         const double det = a * c - b * b;
                         if (det > 1e-13 * a * c) {
-                            nc = (b * (sv - 1.0) - a * (smv - R)) / det;
-                            tc = (fma(nc, b, sv) - 1.0) / a;
+                            // the two divisions as one: lane 0 the multiplier, the others 1/|S|, from which
+                            // the threshold follows with one correction (to an ulp of the division)
+                            const double num = b * (sv - 1.0) - a * (smv - R);
+                            const bool l0 = threadIdx.x == 0;
+                            const double q = (l0 ? num : 1.0) / (l0 ? det : a);
+                            nc = __shfl_sync(0xffffffffu, q, 0);
+                            const double ra = __shfl_sync(0xffffffffu, q, 1);
+                            const double t = fma(nc, b, sv) - 1.0, t0 = t * ra;
+                            tc = fma(fma(-t0, a, t), ra, t0);
                             ok = !ge || nc >= 0.0;
                         }
                     }
                     if (ok && nc == nc && tc == tc && isfinite(nc) && isfinite(tc)) {
-                        sh->nu0 = enu;
-                        sh->tau0 = etau;
-                        sh->nu032 = enu32;
-                        sh->tau032 = etau32;
-                        sh->verify = 1;
-                        verifying = true;
+                        verify = true;
                         next_nu = nc;
                         next_tau = tc;
                         handled = true;
@@ -705,24 +789,30 @@ struct ClusterProj {
                         }
                     }
                 }
-                if (finish) {
-                    sh->done = 1;
-                    sh->status = status;
-                    sh->nu = nu;
-                    sh->tau = tau;
-                    if (status == MV_ERR_NUMERIC || (status == MV_ERR_NOT_CONVERGED && !(tau == tau))) {
-                        sh->nu = enu;
-                        sh->tau = etau;
+                if (threadIdx.x == 0) {
+                    sh->steps += 1;
+                    sh->verify = verify ? 1 : 0;
+                    if (finish) {
+                        sh->done = 1;
+                        sh->status = status;
+                        sh->nu = nu;
+                        sh->tau = tau;
+                        if (status == MV_ERR_NUMERIC || (status == MV_ERR_NOT_CONVERGED && !(tau == tau))) {
+                            sh->nu = enu;
+                            sh->tau = etau;
+                        }
+                    } else {
+                        sh->nu = next_nu;
+                        sh->tau = next_tau;
+                        sh->nu32 = (float)next_nu;
+                        sh->tau32 = (float)next_tau;
                     }
-                } else {
-                    sh->nu = next_nu;
-                    sh->tau = next_tau;
-                    sh->nu32 = (float)next_nu;
-                    sh->tau32 = (float)next_tau;
                 }
             }
             __syncthreads();
         }
+        if (!side_done && threadIdx.x >= kProjNT - kWarp) side();   // infeasible: no reduction ran
+        __syncthreads();
         ProjOut o;
         o.nu = sh->nu;
         o.tau = sh->tau;
@@ -731,6 +821,11 @@ struct ClusterProj {
         o.dykstra = 0;
         __syncthreads();   // all threads read the result before the slots are reused
         return o;
+    }
+
+    __device__ ProjOut search(double R, int mode, double mu_min, double mu_max, double nu_hint, double tau_hint,
+                             int budget) {
+        return search(R, mode, mu_min, mu_max, nu_hint, tau_hint, budget, [] {});
     }
 
     // Dykstra's alternating projections between Delta and H (the safeguard
@@ -816,9 +911,12 @@ struct ClusterProj {
     // The projection: the scalar search, and the Dykstra safeguard when the
     // search does not finish within its budget (scratch permitting), whose
     // (theta, tau) restarts the exact search, with at least 100 outer steps.
+    // `side` runs on the last warp beside the first reduction's scalar logic;
+    // what it leaves in shared memory is visible on return.
+    template <typename Side>
     __device__ ProjOut solve(double R, int mode, double mu_min, double mu_max, double nu_hint, double tau_hint,
-                             int budget) {
-        ProjOut o = search(R, mode, mu_min, mu_max, nu_hint, tau_hint, budget);
+                             int budget, const Side &side) {
+        ProjOut o = search(R, mode, mu_min, mu_max, nu_hint, tau_hint, budget, side);
         if (o.status != MV_ERR_NOT_CONVERGED || dyk == nullptr || dyk_iters <= 0) return o;
         int sweeps = 0;
         double tau_d = -INFINITY;
@@ -828,6 +926,10 @@ struct ClusterProj {
         o.steps += steps;
         o.dykstra = 1;
         return o;
+    }
+    __device__ ProjOut solve(double R, int mode, double mu_min, double mu_max, double nu_hint, double tau_hint,
+                             int budget) {
+        return solve(R, mode, mu_min, mu_max, nu_hint, tau_hint, budget, [] {});
     }
 };
 

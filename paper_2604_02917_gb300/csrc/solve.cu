@@ -464,6 +464,7 @@ __device__ __forceinline__ void init_x_body(SolveState *st, const double *__rest
             st->nu_kkt = o.nu;
             st->tau_kkt = o.tau;
             st->dykstra += o.dykstra;
+            st->hint = P.scales();
         }
         cluster_barrier<CL>();
     } else {
@@ -478,11 +479,13 @@ __device__ __forceinline__ void init_x_body(SolveState *st, const double *__rest
             st->tau = -INFINITY;
             st->nu_kkt = 0.0;
             st->tau_kkt = -INFINITY;
+            st->hint.e[0] = -1;
         }
     }
     if (rank == 0 && threadIdx.x == 0) {
         st->t = 1.0;
         st->beta_prev = 0.0;
+        st->inv1pb = 1.0;
         st->k = 0;
         st->done = (st->status != MV_OK) ? 1 : 0;
         st->converged = 0;
@@ -527,76 +530,101 @@ struct StepArgs {
 
 
 // One NPGA step on a cluster of CL blocks; block r owns assets [r0, r1).
-template <int CL>
+//
+// Bound: latency (one cluster, no bandwidth to speak of).  So the vectors of
+// a thread's first two elements (all of them at the cluster sizes a single
+// solve uses) are loaded in one round trip beside the state and kept in
+// registers to the end; the momentum scalars of this step and the reciprocal
+// the next one needs (a square root and two divisions, about 1.3 us on one
+// lane) run on the last warp beside the projection's first scalar logic; and
+// the projection starts from the scales of the previous one (project.cuh).
+// KEEP: elements per thread kept so (2; 0 in the batch, whose blocks hold up
+// to six per thread and share an SM, so registers count more there).
+template <int CL, int KEEP>
 __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char *dsm, ProjSmem &psm) {
     SolveState *st = a.st;
-    // Every block reads the flag before the first cluster barrier; the flag is
-    // only written after later barriers, so the whole cluster agrees.
-    if (*(volatile int *)&st->done) return;
     const int n = a.n;
     const int rank = cluster_rank<CL>();
     const int nl = (n + CL - 1) / CL;
     const int r0 = min(n, rank * nl);
     const int r1 = min(n, r0 + nl);
-    const int k = st->k;
-    const double beta_prev = st->beta_prev, alpha = st->alpha, t = st->t;
-    const double mn = st->mu_min, mx = st->mu_max;
-    const double nu0 = st->nu, tau0 = st->tau;
-    const double gamma = a.gamma;
     ProjElems el = carve_elems(dsm, nl);
     el.n = r1 - r0;
-    // Scalars are computed once (FP64 is scarce on this part) and broadcast.
-    __shared__ double sc[4];
-    if (threadIdx.x == 0) {
-        sc[0] = 1.0 / (1.0 + beta_prev);
-        if (a.momentum == 1) {             // strongly convex specialisation: t unused, beta fixed
-            sc[1] = t;
-            sc[2] = st->beta_c;
-        } else {
-            const double tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
-            sc[1] = tn;
-            sc[2] = (t - 1.0) / tn;
-        }
+    // One element's vectors.
+    struct Elem {
+        double mu, gy, gx, x, y;
+    };
+    auto load = [&](int gi) { return Elem{a.mu[gi], a.gy[gi], a.gx[gi], a.x[gi], a.y[gi]}; };
+    Elem keep[KEEP > 0 ? KEEP : 1];
+#pragma unroll
+    for (int j = 0; j < KEEP; ++j) {
+        const int i = threadIdx.x + j * kProjNT;
+        keep[j] = i < el.n ? load(r0 + i) : Elem{0.0, 0.0, 0.0, 0.0, 0.0};
     }
+    const int k = st->k;
+    const double beta_prev = st->beta_prev, inv1pb = st->inv1pb, alpha = st->alpha, t = st->t;
+    const double mn = st->mu_min, mx = st->mu_max;
+    const double nu0 = st->nu, tau0 = st->tau;
+    const ScaleHint hint = st->hint;
+    const double gamma = a.gamma;
+    // Every block reads the flag before the first cluster barrier; the flag is
+    // only written after later barriers, so the whole cluster agrees.
+    if (*(volatile int *)&st->done) return;
+    // Scalars computed once (FP64 is scarce on this part) and broadcast.
+    __shared__ double sc[3];
+    auto momentum = [&] {
+        if (threadIdx.x == kProjNT - kWarp) {
+            double tn = t, beta = 0.0;
+            if (a.momentum == 1) {         // strongly convex specialisation: t unused, beta fixed
+                beta = st->beta_c;
+            } else {
+                tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
+                beta = (t - 1.0) / tn;
+            }
+            sc[0] = tn;
+            sc[1] = beta;
+            sc[2] = 1.0 / (1.0 + beta);
+        }
+    };
     proj_smem_init(&psm);
-    const double inv1pb = sc[0], tn = sc[1], beta = sc[2];
     const bool check = (a.kkt_every > 0 && k % a.kkt_every == 0) || (k >= a.max_iter);
 
     // L L^T x^k by linearity from the product at y^k; the point to project:
-    // x - alpha grad f(x) on a KKT test, else the gradient step from y^k
-    // (one pass over the vectors either way).
-    for (int i = threadIdx.x; i < el.n; i += kProjNT) {
-        const int gi = r0 + i;
-        el.mu[i] = a.mu[gi];
-        const double gyi = a.gy[gi];
-        const double gxi = (k == 0) ? gyi : (gyi + beta_prev * a.gx[gi]) * inv1pb;
-        a.gx[gi] = gxi;
-        if (check) {
-            const double xi = a.x[gi];
-            el.v[i] = xi - alpha * (2.0 * gxi + 2.0 * gamma * xi);
-        } else {
-            const double yi = a.y[gi];
-            el.v[i] = yi - alpha * (2.0 * gyi + 2.0 * gamma * yi);
+    // x - alpha grad f(x) on a KKT test, else the gradient step from y^k.
+    auto from_y = [&](const Elem &e) { return e.y - alpha * (2.0 * e.gy + 2.0 * gamma * e.y); };
+    auto first_point = [&](int i, const Elem &e) {
+        const double gxi = (k == 0) ? e.gy : (e.gy + beta_prev * e.gx) * inv1pb;
+        a.gx[r0 + i] = gxi;
+        el.mu[i] = e.mu;
+        el.v[i] = check ? e.x - alpha * (2.0 * gxi + 2.0 * gamma * e.x) : from_y(e);
+    };
+    // f(i, element) over the thread's elements (all of them private to it)
+    auto each = [&](auto f) {
+#pragma unroll
+        for (int j = 0; j < KEEP; ++j) {
+            const int i = threadIdx.x + j * kProjNT;
+            if (i < el.n) f(i, keep[j]);
         }
-    }
-    __syncthreads();
+        for (int i = threadIdx.x + KEEP * kProjNT; i < el.n; i += kProjNT) f(i, load(r0 + i));
+    };
+    each(first_point);
     ClusterProj<CL> P{&psm, el};
     P.dyk = dyk_slice(a.dyk, rank, nl);
     P.dyk_iters = a.dyk_iters;
     if (check) {
-        P.prepare();
+        P.prepare(hint);
         // warm start from this iteration's multipliers: x^k - alpha grad f(x^k)
         // lies next to the point x^k was projected from (y^k -> x^k as the
         // iterates settle), so its support usually matches and the search
-        // stops after the verifying reduction
+        // stops after the verifying exchange
         // (measured the same as the previous test's multipliers: 37.6 against 37.8 us per step)
         const ProjOut o = P.solve(a.R, a.mode, mn, mx, nu0, tau0, a.budget);
         double r2 = 0.0;
-        for (int i = threadIdx.x; i < el.n; i += kProjNT) {
-            const double p = fmax(fma(o.nu, el.mu[i], el.v[i]) - o.tau, 0.0);
-            const double d = p - a.x[r0 + i];
+        each([&](int i, const Elem &e) {
+            const double p = fmax(fma(o.nu, e.mu, el.v[i]) - o.tau, 0.0);
+            const double d = p - e.x;
             r2 = fma(d, d, r2);
-        }
+        });
         r2 = P.reduce_double(r2);          // identical in every block
         const bool conv = r2 <= a.eps * a.eps;
         const bool stop = conv || k >= a.max_iter || !(r2 == r2);
@@ -618,28 +646,24 @@ __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char 
             cluster_barrier<CL>();
             return;
         }
-        __syncthreads();
-        for (int i = threadIdx.x; i < el.n; i += kProjNT) {
-            const int gi = r0 + i;
-            const double yi = a.y[gi];
-            el.v[i] = yi - alpha * (2.0 * a.gy[gi] + 2.0 * gamma * yi);
-        }
-        __syncthreads();
+        each([&](int i, const Elem &e) { el.v[i] = from_y(e); });
     }
-    P.prepare();
-    const ProjOut o = P.solve(a.R, a.mode, mn, mx, nu0, tau0, a.budget);
-    for (int i = threadIdx.x; i < el.n; i += kProjNT) {
+    P.prepare(hint);
+    const ProjOut o = P.solve(a.R, a.mode, mn, mx, nu0, tau0, a.budget, momentum);
+    const double beta = sc[1];
+    each([&](int i, const Elem &e) {
         const int gi = r0 + i;
-        const double xn = fmax(fma(o.nu, el.mu[i], el.v[i]) - o.tau, 0.0);
-        const double xo = a.x[gi];
-        const double yn = xn + beta * (xn - xo);
+        const double xn = fmax(fma(o.nu, e.mu, el.v[i]) - o.tau, 0.0);
+        const double yn = xn + beta * (xn - e.x);
         a.x[gi] = xn;
         a.y[gi] = yn;
         a.y32[gi] = (float)(yn * (a.row_scale ? (double)a.row_scale[gi] : 1.0));
-    }
+    });
     if (rank == 0 && threadIdx.x == 0) {
-        st->t = tn;
+        st->t = sc[0];
         st->beta_prev = beta;
+        st->inv1pb = sc[2];
+        st->hint = P.scales();
         st->k = k + 1;
         st->nu = o.nu;
         st->tau = o.tau;
@@ -659,7 +683,7 @@ __global__ void __launch_bounds__(kProjNT) npga_step_kernel(StepArgs a) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ ProjSmem psm;
     umma::launch_dependents();     // the next fused pass may start streaming L
-    npga_step_body<CL>(a, dsm, psm);
+    npga_step_body<CL, 2>(a, dsm, psm);
 }
 
 // Grouped form: cluster b runs the step of problem b.
@@ -668,7 +692,7 @@ __global__ void __launch_bounds__(kProjNT) npga_step_grouped(const StepArgs *__r
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ ProjSmem psm;
     const StepArgs a = args[blockIdx.x / CL];
-    npga_step_body<CL>(a, dsm, psm);
+    npga_step_body<CL, 0>(a, dsm, psm);
 }
 
 // Sets up the Sec. 3.1 variants once alpha is known: the first backtracking

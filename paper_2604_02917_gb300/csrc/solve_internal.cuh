@@ -37,6 +37,8 @@ struct SolveState {
     double objective;
     double beta_c;                         // constant momentum (momentum = 1)
     int bt_started, backtracks, dykstra, pad3;
+    double inv1pb;                         // 1 / (1 + beta_prev)
+    ScaleHint hint;                        // scales of the last projection
 };
 
 struct Plan {
