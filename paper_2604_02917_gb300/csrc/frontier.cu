@@ -522,7 +522,7 @@ static int frontier_solve(const mv_problem *P, const mv_problem *P_hi, const dou
     // Shared step size from the power method (or Lanczos steps) on L, the
     // fused pass over L^T; the Lanczos vectors use the transposed plan's x
     // and y buffers, which the frontier leaves unused.
-    MV_CUDA_TRY(cudaMemsetAsync(at<char>(d_ws, pt.o_tick_t), 0, 4 * (size_t)pt.t_blocks, s));
+    MV_CUDA_TRY(cudaMemsetAsync(at<char>(d_ws, pt.o_tick_t), 0, 4 * (size_t)pt.t_ticks, s));
     MV_CUDA_TRY(cudaMemsetAsync(at<char>(d_ws, pt.o_tick_n), 0, 4 * (size_t)pt.n_groups, s));
     const float *rs = P->dtype == MV_FP8_E4M3 ? P->row_scale : nullptr;
     launch_setup(st, P->mu, P->power_start, rs, y32, p.n, s, lanczos ? at<float>(d_ws, pt.o_x) : nullptr,

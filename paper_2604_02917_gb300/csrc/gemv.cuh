@@ -25,6 +25,7 @@
 #pragma once
 
 #include "mv_internal.cuh"
+#include "umma.cuh"
 
 namespace mv {
 
@@ -182,6 +183,7 @@ gemv_t_kernel(const void *__restrict__ L, int64_t ld, int n, int T, const float 
               float *__restrict__ zpart, int64_t zstride, float *__restrict__ z, unsigned *__restrict__ tickets,
               int rows_per_split, const volatile int *done, double *__restrict__ z64 = nullptr,
               const float *__restrict__ cscale = nullptr) {
+    umma::launch_dependents();
     if (done != nullptr && *done) return;
     gemv_t_body<DT>(L, ld, n, T, y32, zpart, zstride, z, tickets, rows_per_split, blockIdx.x, blockIdx.y, gridDim.y,
                     z64, cscale);
@@ -278,9 +280,208 @@ __global__ void __launch_bounds__(kGemvThreads)
 gemv_n_kernel(const void *__restrict__ L, int64_t ld, int n, int T, const float *__restrict__ z,
               const float *__restrict__ row_scale, float *__restrict__ gpart, double *__restrict__ g,
               float *__restrict__ g32, unsigned *__restrict__ tickets, int cols_per_split, const volatile int *done) {
+    umma::launch_dependents();
     if (done != nullptr && *done) return;
     gemv_n_body<DT, RW>(L, ld, n, T, z, row_scale, gpart, g, g32, tickets, cols_per_split, blockIdx.x, blockIdx.y,
                         gridDim.y);
+}
+
+// ---------------------------------------------------------------- latency forms
+// The same two products for matrices that do not fill the machine (compressed
+// factors, small universes), where a launch is a chain of L2 round trips, not
+// a stream.  Every value is formed by the same additions in the same order as
+// above, so the forms agree bit for bit; what differs is who forms it:
+//  * gemv_t: 4 bytes of columns per thread instead of 16, four times the
+//    blocks, all rows of a split (at most 64) loaded at once;
+//  * gemv_n: one row per warp instead of four, eight 16-byte loads at once;
+//  * both are launched as programmatic dependents and load L, which no
+//    kernel before them writes, ahead of the wait for their input vector.
+// The last block's sum over the splits keeps 64 (gemv_t) loads in flight:
+// at 5440 x 512 it adds 85 splits, 22 round trips in the wide form.
+constexpr int kLatRows = 64;                 // rows per split the latency gemv_t holds
+constexpr int kLatSub = 4;                   // its column groups per strip of the wide form
+constexpr int kLatPre = 8;                   // 16-byte loads per lane ahead of the wait in gemv_n
+
+// 4 bytes of a row as FP32 values.
+template <int DT>
+__device__ __forceinline__ void unpack4(uint32_t w, float (&f)[Store<DT>::VEC / 4]) {
+    if constexpr (DT == MV_F32) {
+        f[0] = __uint_as_float(w);
+    } else if constexpr (DT == MV_BF16) {
+        Store<DT>::two(w, f);
+    } else {
+        Store<DT>::four(w, f);
+    }
+}
+__device__ __forceinline__ uint32_t ld_stream4(const void *p) {
+    uint32_t v;
+    asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
+// One block: columns [256 CV b, 256 CV (b + 1)), b = blockIdx.x (CV = 4 bytes
+// of columns per thread), rows of split blockIdx.y.  Parameters as
+// gemv_t_body; tickets has one entry per b.
+template <int DT>
+__global__ void __launch_bounds__(kGemvThreads)
+gemv_t_lat_kernel(const void *__restrict__ L, int64_t ld, int n, int T, const float *__restrict__ y32,
+                  float *__restrict__ zpart, int64_t zstride, float *__restrict__ z, unsigned *__restrict__ tickets,
+                  int rows_per_split, const volatile int *done, double *__restrict__ z64,
+                  const float *__restrict__ cscale) {
+    constexpr int CV = Store<DT>::VEC / 4;
+    constexpr int ES = 4 / CV;
+    __shared__ float s_y[kLatRows];
+    __shared__ bool s_last;
+    const int splits = gridDim.y, split = blockIdx.y;
+    const int r0 = split * rows_per_split;
+    const int rows = min(n - r0, rows_per_split);
+    const int64_t col = ((int64_t)blockIdx.x * kGemvThreads + threadIdx.x) * CV;
+    const bool in = col < T;                 // 4 bytes from col stay inside the row's 16-byte padded pitch
+    const char *p = reinterpret_cast<const char *>(L) + ((int64_t)r0 * ld + col) * ES;
+    uint32_t u[kLatRows];
+#pragma unroll
+    for (int i = 0; i < kLatRows; ++i) u[i] = in && i < rows ? ld_stream4(p + (int64_t)i * ld * ES) : 0u;
+    umma::grid_dependency_wait();
+    umma::launch_dependents();
+    if (done != nullptr && *done) return;
+    for (int i = threadIdx.x; i < rows; i += kGemvThreads) s_y[i] = __ldcg(y32 + r0 + i);
+    __syncthreads();
+    float acc[CV];
+#pragma unroll
+    for (int e = 0; e < CV; ++e) acc[e] = 0.f;
+#pragma unroll
+    for (int i = 0; i < kLatRows; ++i) {
+        if (i < rows) {
+            float f[CV];
+            unpack4<DT>(u[i], f);
+#pragma unroll
+            for (int e = 0; e < CV; ++e) acc[e] = fmaf(f[e], s_y[i], acc[e]);
+        }
+    }
+    if (splits > 1) {
+        // rows of zpart are padded to 64 bytes, so a thread may write all its CV columns
+        float *zp = zpart + (int64_t)split * zstride + col;
+#pragma unroll
+        for (int e = 0; e < CV; ++e)
+            if (in) zp[e] = acc[e];
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) s_last = atomicAdd(&tickets[blockIdx.x], 1u) == (unsigned)splits - 1;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        // splits in order, 64 / CV of them in flight
+        constexpr int FL = kLatRows / CV;
+#pragma unroll
+        for (int e = 0; e < CV; ++e) acc[e] = 0.f;
+        const float *q = zpart + col;
+        for (int s0 = 0; in && s0 < splits; s0 += FL) {
+            float v[FL][CV];
+#pragma unroll
+            for (int k = 0; k < FL; ++k)
+#pragma unroll
+                for (int e = 0; e < CV; ++e) v[k][e] = s0 + k < splits ? __ldcg(q + (int64_t)(s0 + k) * zstride + e) : 0.f;
+#pragma unroll
+            for (int k = 0; k < FL; ++k)
+                if (s0 + k < splits)
+#pragma unroll
+                    for (int e = 0; e < CV; ++e) acc[e] += v[k][e];
+        }
+        if (threadIdx.x == 0) tickets[blockIdx.x] = 0u;   // ready for the next launch
+    } else {
+#pragma unroll
+        for (int e = 0; e < CV; ++e) acc[e] = 0.f + acc[e];   // as the sum over one split
+    }
+#pragma unroll
+    for (int e = 0; e < CV; ++e) {
+        if (col + e >= T) continue;
+        if (z != nullptr) z[col + e] = cscale != nullptr ? acc[e] * cscale[col + e] : acc[e];
+        if (z64 != nullptr) z64[col + e] = (double)acc[e] * (cscale != nullptr ? (double)cscale[col + e] : 1.0);
+    }
+}
+
+// One block: 8 rows (one per warp), column split blockIdx.y.  Parameters as
+// gemv_n_body; tickets has one entry per 32 rows, brought to the number of
+// blocks of that group.
+template <int DT>
+__global__ void __launch_bounds__(kGemvThreads)
+gemv_n_lat_kernel(const void *__restrict__ L, int64_t ld, int n, int T, const float *__restrict__ z,
+                  const float *__restrict__ row_scale, float *__restrict__ gpart, double *__restrict__ g,
+                  float *__restrict__ g32, unsigned *__restrict__ tickets, int cols_per_split, const volatile int *done) {
+    using S = Store<DT>;
+    constexpr int VEC = S::VEC;
+    constexpr int ES = (int)sizeof(typename S::elem);
+    constexpr int WARPS = kGemvThreads / kWarp, GROUP = 32;   // rows per block, per ticket
+    extern __shared__ __align__(16) float s_z[];
+    __shared__ bool s_last;
+    const int splits = gridDim.y, split = blockIdx.y;
+    const int c0 = split * cols_per_split;
+    const int ncol = min(T - c0, cols_per_split);
+    const int nfull = ncol / VEC * VEC;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r = blockIdx.x * WARPS + warp;
+    const char *rp = reinterpret_cast<const char *>(L) + ((int64_t)min(r, n - 1) * ld + c0) * ES;
+    uint4 u[kLatPre];
+#pragma unroll
+    for (int k = 0; k < kLatPre; ++k) {
+        const int c = (k * kWarp + lane) * VEC;
+        u[k] = c < nfull ? ld_stream16(rp + (int64_t)c * ES) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    umma::grid_dependency_wait();
+    umma::launch_dependents();
+    if (done != nullptr && *done) return;
+    for (int c = threadIdx.x; c < ncol; c += kGemvThreads) s_z[c] = __ldcg(z + c0 + c);
+    __syncthreads();
+    float acc = 0.f;
+    auto add = [&](const uint4 &w, int c) {
+        float f[VEC];
+        S::unpack(w, f);
+#pragma unroll
+        for (int e = 0; e < VEC; e += 4) {
+            const float4 q = *reinterpret_cast<const float4 *>(s_z + c + e);
+            acc = fmaf(f[e], q.x, acc);
+            acc = fmaf(f[e + 1], q.y, acc);
+            acc = fmaf(f[e + 2], q.z, acc);
+            acc = fmaf(f[e + 3], q.w, acc);
+        }
+    };
+#pragma unroll
+    for (int k = 0; k < kLatPre; ++k) {
+        const int c = (k * kWarp + lane) * VEC;
+        if (c < nfull) add(u[k], c);
+    }
+#pragma unroll 4
+    for (int c = (kLatPre * kWarp + lane) * VEC; c < nfull; c += kWarp * VEC) add(ld_stream16(rp + (int64_t)c * ES), c);
+    for (int c = nfull + lane; c < ncol; c += kWarp)           // ragged tail
+        acc = fmaf(S::load1(L, (int64_t)min(r, n - 1) * ld + c0 + c), s_z[c], acc);
+    acc = warp_sumf(acc);
+    auto publish = [&](int row, double s) {
+        if (row_scale != nullptr) s *= (double)row_scale[row];
+        g[row] = s;
+        if (g32 != nullptr) g32[row] = (float)s;
+    };
+    if (splits == 1) {
+        if (lane == 0 && r < n) publish(r, 0.0 + (double)acc);
+        return;
+    }
+    if (lane == 0 && r < n) gpart[(int64_t)split * n + r] = acc;
+    __threadfence();
+    __syncthreads();
+    const int grp = blockIdx.x * WARPS / GROUP;
+    if (threadIdx.x == 0) {
+        const int blocks = (min(n, (grp + 1) * GROUP) - grp * GROUP + WARPS - 1) / WARPS;
+        s_last = atomicAdd(&tickets[grp], 1u) == (unsigned)(blocks * splits) - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int row = grp * GROUP + threadIdx.x; row < min(n, (grp + 1) * GROUP); row += kGemvThreads) {
+        double s = 0.0;
+#pragma unroll 8
+        for (int sp = 0; sp < splits; ++sp) s += (double)__ldcg(gpart + (int64_t)sp * n + row);
+        publish(row, s);
+    }
+    if (threadIdx.x == 0) tickets[grp] = 0u;
 }
 
 // ---------------------------------------------------------------- grouped form

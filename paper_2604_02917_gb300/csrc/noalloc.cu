@@ -76,7 +76,7 @@ extern "C" int mv_gradient_noalloc(const mv_problem *P, const double *d_y, float
     float *y32 = at<float>(ws, p.o_y32);
     double *lz = at<double>(ws, p.o_gy);
     // The array keeps the previous call's contents: the gemv tickets must start at zero.
-    MV_CUDA_TRY(cudaMemsetAsync(at<char>(ws, p.o_tick_t), 0, 4 * (size_t)p.t_blocks, s));
+    MV_CUDA_TRY(cudaMemsetAsync(at<char>(ws, p.o_tick_t), 0, 4 * (size_t)p.t_ticks, s));
     MV_CUDA_TRY(cudaMemsetAsync(at<char>(ws, p.o_tick_n), 0, 4 * (size_t)p.n_groups, s));
     const float *rs = P->dtype == MV_FP8_E4M3 ? P->row_scale : nullptr;
     launch_to_y32(d_y, rs, y32, p.n, s);

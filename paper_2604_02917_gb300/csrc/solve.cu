@@ -71,6 +71,13 @@ Plan make_plan(int dt, int64_t n, int64_t T, int64_t ld, int grouped_rows, bool 
     p.n_cols = n_bytes / p.esize;                        // 16 KB per row per split by default
     if (p.n_cols > gc) p.n_cols = (int)((gc + 32 * p.vec - 1) / (32 * p.vec) * (32 * p.vec));
     p.n_splits = (int)((gc + p.n_cols - 1) / p.n_cols);
+    // The latency forms (gemv.cuh).  gemv_t: where a split's rows fit its
+    // registers and its tickets (kLatSub per strip) the 256 bytes the wide
+    // form's take anyway.  gemv_n: where the wide grid leaves SMs idle or
+    // with one block (2 per SM).
+    p.t_lat = grouped_rows <= 0 && p.t_rows <= kLatRows && p.t_blocks <= 64 / kLatSub;
+    p.t_ticks = p.t_lat ? p.t_blocks * kLatSub : p.t_blocks;
+    p.n_lat = grouped_rows <= 0 && (int64_t)p.n_groups * p.n_splits < 2 * (int64_t)sms;
     size_t off = 0;
     auto take = [&](size_t bytes) {
         size_t o = off;
@@ -975,63 +982,82 @@ int check_ws(void *ws, size_t ws_bytes, size_t need) {
 
 template <int DT>
 static void launch_gemv_t(const Plan &p, const void *L, const float *w32, float *out32, double *out64,
-                          const float *cscale, void *ws, const int *done, cudaStream_t s) {
+                          const float *cscale, void *ws, const int *done, cudaStream_t s, bool pdl) {
+    float *zpart = at<float>(ws, p.o_zpart);
+    unsigned *ticks = at<unsigned>(ws, p.o_tick_t);
+    if (p.t_lat) {
+        const int strip = kGemvThreads * p.vec / kLatSub;
+        launch_grid(gemv_t_lat_kernel<DT>, dim3((p.gc + strip - 1) / strip, p.t_splits), dim3(kGemvThreads), 0, s, pdl, L,
+                    p.ld, p.gr, p.gc, w32, zpart, p.zstride, out32, ticks, p.t_rows, done, out64, cscale);
+        return;
+    }
     dim3 grid(p.t_blocks, p.t_splits);
-    gemv_t_kernel<DT><<<grid, kGemvThreads, 0, s>>>(L, p.ld, p.gr, p.gc, w32, at<float>(ws, p.o_zpart), p.zstride,
-                                                     out32, at<unsigned>(ws, p.o_tick_t), p.t_rows, done, out64, cscale);
+    gemv_t_kernel<DT><<<grid, kGemvThreads, 0, s>>>(L, p.ld, p.gr, p.gc, w32, zpart, p.zstride, out32, ticks, p.t_rows,
+                                                     done, out64, cscale);
 }
 
 template <int DT>
 static void launch_gemv_n(const Plan &p, const void *L, const float *w32, const float *rscale, double *out64,
-                          float *out32, void *ws, const int *done, cudaStream_t s) {
-    dim3 grid(p.n_groups, p.n_splits);
+                          float *out32, void *ws, const int *done, cudaStream_t s, bool pdl) {
     const size_t smem = (size_t)p.n_cols * 4;
-    gemv_n_kernel<DT, kRW><<<grid, kGemvThreads, smem, s>>>(L, p.ld, p.gr, p.gc, w32, rscale, at<float>(ws, p.o_gpart),
-                                                           out64, out32, at<unsigned>(ws, p.o_tick_n), p.n_cols, done);
+    float *gpart = at<float>(ws, p.o_gpart);
+    unsigned *ticks = at<unsigned>(ws, p.o_tick_n);
+    if (p.n_lat) {
+        constexpr int rows = kGemvThreads / kWarp;
+        launch_grid(gemv_n_lat_kernel<DT>, dim3((p.gr + rows - 1) / rows, p.n_splits), dim3(kGemvThreads), smem, s, pdl, L,
+                    p.ld, p.gr, p.gc, w32, rscale, gpart, out64, out32, ticks, p.n_cols, done);
+        return;
+    }
+    dim3 grid(p.n_groups, p.n_splits);
+    gemv_n_kernel<DT, kRW><<<grid, kGemvThreads, smem, s>>>(L, p.ld, p.gr, p.gc, w32, rscale, gpart, out64, out32, ticks,
+                                                           p.n_cols, done);
 }
 
 // z = L^T y32 into the FP32 T-vector at o_z (y32 pre-multiplied by the FP8 scales).
 template <int DT>
 static void launch_z_t(const Plan &p, const mv_problem *P, const float *y32, void *ws, const int *done,
-                       cudaStream_t s) {
+                       cudaStream_t s, bool pdl) {
     float *z = at<float>(ws, p.o_z);
     if (p.tn)
-        launch_gemv_n<DT>(p, P->L, y32, nullptr, at<double>(ws, p.o_zd), z, ws, done, s);
+        launch_gemv_n<DT>(p, P->L, y32, nullptr, at<double>(ws, p.o_zd), z, ws, done, s, pdl);
     else
-        launch_gemv_t<DT>(p, P->L, y32, z, nullptr, nullptr, ws, done, s);
+        launch_gemv_t<DT>(p, P->L, y32, z, nullptr, nullptr, ws, done, s, pdl);
 }
 
 // g = L z (FP64, FP8 scales applied) and optionally its FP32 copy g32.
 template <int DT>
 static void launch_g_t(const Plan &p, const mv_problem *P, const float *z, void *ws, const int *done, double *g,
-                       float *g32, cudaStream_t s) {
+                       float *g32, cudaStream_t s, bool pdl) {
     const float *rs = P->dtype == MV_FP8_E4M3 ? P->row_scale : nullptr;
     if (p.tn)
-        launch_gemv_t<DT>(p, P->L, z, g32, g, rs, ws, done, s);
+        launch_gemv_t<DT>(p, P->L, z, g32, g, rs, ws, done, s, pdl);
     else
-        launch_gemv_n<DT>(p, P->L, z, rs, g, g32, ws, done, s);
+        launch_gemv_n<DT>(p, P->L, z, rs, g, g32, ws, done, s, pdl);
 }
 
-static void launch_z(const Plan &p, const mv_problem *P, const float *y32, void *ws, const int *done, cudaStream_t s) {
+static void launch_z(const Plan &p, const mv_problem *P, const float *y32, void *ws, const int *done, cudaStream_t s,
+                     bool pdl) {
     switch (p.dt) {
-        case MV_F32: launch_z_t<MV_F32>(p, P, y32, ws, done, s); break;
-        case MV_BF16: launch_z_t<MV_BF16>(p, P, y32, ws, done, s); break;
-        default: launch_z_t<MV_FP8_E4M3>(p, P, y32, ws, done, s); break;
+        case MV_F32: launch_z_t<MV_F32>(p, P, y32, ws, done, s, pdl); break;
+        case MV_BF16: launch_z_t<MV_BF16>(p, P, y32, ws, done, s, pdl); break;
+        default: launch_z_t<MV_FP8_E4M3>(p, P, y32, ws, done, s, pdl); break;
     }
 }
 
 static void launch_g(const Plan &p, const mv_problem *P, const float *z, void *ws, const int *done, double *g,
-                     float *g32, cudaStream_t s) {
+                     float *g32, cudaStream_t s, bool pdl) {
     switch (p.dt) {
-        case MV_F32: launch_g_t<MV_F32>(p, P, z, ws, done, g, g32, s); break;
-        case MV_BF16: launch_g_t<MV_BF16>(p, P, z, ws, done, g, g32, s); break;
-        default: launch_g_t<MV_FP8_E4M3>(p, P, z, ws, done, g, g32, s); break;
+        case MV_F32: launch_g_t<MV_F32>(p, P, z, ws, done, g, g32, s, pdl); break;
+        case MV_BF16: launch_g_t<MV_BF16>(p, P, z, ws, done, g, g32, s, pdl); break;
+        default: launch_g_t<MV_FP8_E4M3>(p, P, z, ws, done, g, g32, s, pdl); break;
     }
 }
 
-// The solve loop and the power graph launch the fused pass as a
-// programmatic dependent of the step / normalisation kernel before it.
-constexpr bool kFusedPdl = true;
+// The solve loop and the power graph launch their kernels as programmatic
+// dependents of the ones before them.  Every kernel launched so waits for its
+// predecessor before it triggers its own dependents, so a kernel that has
+// started may rely on everything before its predecessor.
+constexpr bool kLoopPdl = true;
 
 // g = L L^T y (row-scaled) in one pass over L; capturable (no synchronisation).
 int launch_llt(const Plan &p, const mv_problem *P, const float *y32, void *ws, const int *done, double *g_out,
@@ -1054,6 +1080,9 @@ int set_kernel_attrs() {
                       cudaSuccess &&
                   cudaFuncSetAttribute(gemv_n_kernel<MV_FP8_E4M3, kRW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        big) == cudaSuccess;
+        ok = ok && cudaFuncSetAttribute(gemv_n_lat_kernel<MV_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, big) == cudaSuccess &&
+             cudaFuncSetAttribute(gemv_n_lat_kernel<MV_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, big) == cudaSuccess &&
+             cudaFuncSetAttribute(gemv_n_lat_kernel<MV_FP8_E4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize, big) == cudaSuccess;
         ok = ok && cluster_attrs(npga_step_kernel<1>, 1) && cluster_attrs(npga_step_kernel<2>, 2) &&
              cluster_attrs(npga_step_kernel<4>, 4) && cluster_attrs(npga_step_kernel<8>, 8) &&
              cluster_attrs(npga_step_kernel<16>, 16);
@@ -1069,13 +1098,13 @@ int set_kernel_attrs() {
 }
 
 void gemv_pair(const Plan &p, const mv_problem *P, const float *y32, void *ws, const int *done, double *g_out,
-               cudaStream_t s, float *g32) {
-    launch_z(p, P, y32, ws, done, s);
-    launch_g(p, P, at<float>(ws, p.o_z), ws, done, g_out, g32, s);
+               cudaStream_t s, float *g32, bool pdl) {
+    launch_z(p, P, y32, ws, done, s, pdl);
+    launch_g(p, P, at<float>(ws, p.o_z), ws, done, g_out, g32, s, pdl);
 }
 
 void gemv_t_only(const Plan &p, const mv_problem *P, const float *y32, void *ws, cudaStream_t s) {
-    launch_z(p, P, y32, ws, nullptr, s);
+    launch_z(p, P, y32, ws, nullptr, s, false);
 }
 
 static size_t step_smem(int n, int CL) { return proj_elem_bytes((n + CL - 1) / CL); }
@@ -1190,16 +1219,16 @@ int launch_iteration(const Plan &p, const mv_problem *P, const mv_solve_opts *O,
             MV_TRY(launch_symv(p, P, y32, ws, done, gy, nullptr, s));
         else
             MV_TRY(launch_llt(p, P, y32, ws, done, gy, nullptr, s, p.want_z ? at<float>(ws, p.o_z) : nullptr,
-                              kFusedPdl && ev == nullptr));   // timed runs keep launches apart
+                              kLoopPdl && ev == nullptr));   // timed runs keep launches apart
         if (ev) cudaEventRecord(ev[1], s);
         if (ev) cudaEventRecord(ev[2], s);
         launch_step(p, P, O, ws, s);
         if (ev) cudaEventRecord(ev[3], s);
         return MV_OK;
     }
-    launch_z(p, P, y32, ws, done, s);
+    launch_z(p, P, y32, ws, done, s, kLoopPdl && ev == nullptr);
     if (ev) cudaEventRecord(ev[1], s);
-    launch_g(p, P, at<float>(ws, p.o_z), ws, done, gy, nullptr, s);
+    launch_g(p, P, at<float>(ws, p.o_z), ws, done, gy, nullptr, s, kLoopPdl && ev == nullptr);
     if (ev) cudaEventRecord(ev[2], s);
     launch_step(p, P, O, ws, s);
     if (ev) cudaEventRecord(ev[3], s);
@@ -1291,10 +1320,10 @@ static int launch_power(const Plan &p, const mv_problem *P, int power_iters, voi
             // after the previous power normalisation (the first launch has no
             // kernel before it in the captured graph)
             MV_TRY(launch_llt(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), at<float>(ws, p.o_g32), s, nullptr,
-                              kFusedPdl));
+                              kLoopPdl));
             *count += 2;
         } else {
-            gemv_pair(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), s, at<float>(ws, p.o_g32));
+            gemv_pair(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), s, at<float>(ws, p.o_g32), kLoopPdl);
             *count += 3;
         }
         power_norm_kernel<<<1, kStepThreads, 0, s>>>(at<float>(ws, p.o_g32), rs, y32, p.n);
@@ -1321,10 +1350,10 @@ static int launch_lanczos(const Plan &p, const mv_problem *P, int steps, void *w
             MV_TRY(launch_symv(p, P, y32, ws, nullptr, wd, w, s));
             *count += 2;
         } else if (p.use_llt) {
-            MV_TRY(launch_llt(p, P, y32, ws, nullptr, wd, w, s, nullptr, kFusedPdl));
+            MV_TRY(launch_llt(p, P, y32, ws, nullptr, wd, w, s, nullptr, kLoopPdl));
             *count += 2;
         } else {
-            gemv_pair(p, P, y32, ws, nullptr, wd, s, w);
+            gemv_pair(p, P, y32, ws, nullptr, wd, s, w, kLoopPdl);
             *count += 3;
         }
         lanczos_kernel<<<1, kLanczosThreads, 0, s>>>(w, q[j & 1], q[(j + 1) & 1], at<double>(ws, p.o_lan), rs, y32,
@@ -1417,7 +1446,7 @@ int mv_gradient(const mv_problem *P, const double *d_y, float *d_z, double *d_g,
     cudaStream_t s = (cudaStream_t)stream;
     float *y32 = at<float>(d_ws, p.o_y32);
     double *lz = at<double>(d_ws, p.o_gy);
-    MV_CUDA_TRY(cudaMemsetAsync(at<char>(d_ws, p.o_tick_t), 0, 4 * (size_t)p.t_blocks, s));
+    MV_CUDA_TRY(cudaMemsetAsync(at<char>(d_ws, p.o_tick_t), 0, 4 * (size_t)p.t_ticks, s));
     MV_CUDA_TRY(cudaMemsetAsync(at<char>(d_ws, p.o_tick_n), 0, 4 * (size_t)p.n_groups, s));
     const float *rs = P->dtype == MV_FP8_E4M3 ? P->row_scale : nullptr;
     to_y32_kernel<<<(p.n + 255) / 256, 256, 0, s>>>(d_y, rs, y32, p.n);
@@ -1465,7 +1494,7 @@ int mv_npga_solve(const mv_problem *P, const mv_solve_opts *O_in, double *d_x_in
     const float *rs = P->dtype == MV_FP8_E4M3 ? P->row_scale : nullptr;
     *h_info = mv_solve_info{};
 
-    MV_CUDA_TRY(cudaMemsetAsync(at<char>(d_ws, p.o_tick_t), 0, 4 * (size_t)p.t_blocks, s));
+    MV_CUDA_TRY(cudaMemsetAsync(at<char>(d_ws, p.o_tick_t), 0, 4 * (size_t)p.t_ticks, s));
     MV_CUDA_TRY(cudaMemsetAsync(at<char>(d_ws, p.o_tick_n), 0, 4 * (size_t)p.n_groups, s));
     MV_CUDA_TRY(cudaMemsetAsync(at<char>(d_ws, p.o_err), 0, 16, s));
     if (p.use_llt) MV_CUDA_TRY(cudaMemsetAsync(llt_scratch(at<char>(d_ws, p.o_llt), p.n).tickets, 0, llt_ticket_bytes(), s));

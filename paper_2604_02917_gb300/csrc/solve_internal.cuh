@@ -50,6 +50,8 @@ struct Plan {
     int cl;                                // cluster size of the step kernel
     int t_blocks, t_splits, t_rows;        // gemv_t grid
     int n_groups, n_splits, n_cols;        // gemv_n grid
+    bool t_lat, n_lat;                     // the latency forms of gemv_t and gemv_n (gemv.cuh)
+    int t_ticks;                           // gemv_t tickets in use
     bool use_llt;                          // fused single-pass L L^T y (llt.cuh)
     bool want_z;                           // the loop's fused pass also writes z = L^T y to o_z
     LltPlan lp;
@@ -115,8 +117,10 @@ int set_kernel_attrs();
 // must not write L; see llt_launch).
 int launch_llt(const Plan &p, const mv_problem *P, const float *y32, void *ws, const int *done, double *g_out,
                float *g32, cudaStream_t s, float *z = nullptr, bool pdl = false);
+// pdl: launched as programmatic dependents of the kernels before them (the
+// latency forms load L, which those must not write, before the wait).
 void gemv_pair(const Plan &p, const mv_problem *P, const float *y32, void *ws, const int *done, double *g_out,
-               cudaStream_t s, float *g32 = nullptr);
+               cudaStream_t s, float *g32 = nullptr, bool pdl = false);
 void gemv_t_only(const Plan &p, const mv_problem *P, const float *y32, void *ws, cudaStream_t s);
 void launch_init_x(const Plan &p, const mv_problem *P, const mv_solve_opts *O, const double *x_in, void *ws,
                    cudaStream_t s);
@@ -149,6 +153,23 @@ inline bool cluster_attrs(Kern k, int CL) {
     if (CL > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
         return false;
     return true;
+}
+
+// Ordinary launch, or (pdl) as a programmatic dependent of the kernel before it.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_grid(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl,
+                               Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
 }
 
 template <typename Kern, typename... Args>
