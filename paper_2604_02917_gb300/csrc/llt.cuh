@@ -254,8 +254,10 @@ __host__ __device__ inline LltSmem llt_smem_layout(int rpc, int RB, int W, int C
     return m;
 }
 
+// 72 registers (none spilled): a step of 256 threads x 96 fits beside a CTA.
+constexpr int kLltRegs = 72;
 template <int DT, int C, int RB>
-__global__ void __launch_bounds__(kLltThreads, 1)
+__global__ void __maxnreg__(kLltRegs)
 llt_kernel(const __grid_constant__ CUtensorMap tmL, const LltArgs a) {
     using S = Store<DT>;
     constexpr int EPC = S::VEC;                        // elements per 16-byte chunk
@@ -265,6 +267,7 @@ llt_kernel(const __grid_constant__ CUtensorMap tmL, const LltArgs a) {
     constexpr int V4 = EPC / 4;                        // float4 pieces of one chunk's partials
     constexpr int RPT = kLltRowsPerThread;
     namespace cg = cooperative_groups;
+    umma::launch_dependents();                           // launched the plain way: the step may start beside this pass
     if (a.done != nullptr && *(const volatile int *)a.done) return;
 
     extern __shared__ uint8_t smem_raw[];
@@ -500,6 +503,7 @@ __device__ __forceinline__ void lltt_body(const CUtensorMap *tm, const LltArgs &
     constexpr int BOXB = W * kLltBoxCols * ES;           // bytes of one box
     constexpr int RPT = (ES == 4) ? 2 : 1;               // column chunks per thread in phase B
     namespace cg = cooperative_groups;
+    if (!a.early) umma::launch_dependents();             // else after the wait below
     if (a.done != nullptr && *(const volatile int *)a.done) return;
 
     extern __shared__ uint8_t smem_raw[];
@@ -560,6 +564,7 @@ __device__ __forceinline__ void lltt_body(const CUtensorMap *tm, const LltArgs &
     }
     if (a.early) {
         umma::grid_dependency_wait();                      // y, done and the scratch are the predecessor's
+        umma::launch_dependents();                         // the step may start beside this pass
         if (a.done != nullptr && *(const volatile int *)a.done) {
             if (producer)                                  // the issued stages land before the CTA leaves
                 for (int j = 0; j < kLltStages && j < nj; ++j)
@@ -716,7 +721,7 @@ __device__ __forceinline__ void lltt_body(const CUtensorMap *tm, const LltArgs &
 }
 
 template <int DT, int C>
-__global__ void __launch_bounds__(kLltThreads, 1)
+__global__ void __maxnreg__(kLltRegs)
 lltt_kernel(const __grid_constant__ CUtensorMap tmM, const LltArgs a) {
     lltt_body<DT, C, false>(&tmM, a, (int)(blockIdx.x / C));
 }

@@ -115,9 +115,13 @@ __device__ __forceinline__ void add_limbs(int (&l)[3], long long x) {
     l[1] += (int)(x >> 21) & 0x1fffff;
     l[2] += (int)(x >> 42);
 }
-// The value of cluster-wide limb totals (l0, l1 < 2^36; |l2| < 2^35).
+// The value of cluster-wide limb totals (l0, l1 < 2^36; |l2| < 2^35): the
+// 128-bit sum as its high and low halves, each rounded to FP64.
 __device__ __forceinline__ double from_limbs(long long l0, long long l1, long long l2) {
-    return fma((double)l2, 4398046511104.0, (double)((l1 << 21) + l0));
+    const unsigned long long m = (unsigned long long)((l1 << 21) + l0);
+    const unsigned long long lo = m + ((unsigned long long)l2 << 42);
+    const long long hi = (l2 >> 22) + (lo < m ? 1 : 0);
+    return (double)hi * 18446744073709551616.0 + (double)lo;
 }
 
 // Cluster totals of one support step, as thread 0 of every block holds them.
@@ -221,6 +225,18 @@ __device__ __forceinline__ void cluster_barrier() {
     } else {
         __syncthreads();
     }
+}
+
+// The same barrier in two halves, for work between them; the first exchange
+// of a kernel must follow one, since a peer's shared memory may only be
+// written once the peer runs.
+template <int CL>
+__device__ __forceinline__ void cluster_arrive() {
+    if constexpr (CL > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+template <int CL>
+__device__ __forceinline__ void cluster_wait() {
+    if constexpr (CL > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 template <int CL>
@@ -696,14 +712,16 @@ struct ClusterProj {
                         const double det = a * c - b * b;
                         if (det > 1e-13 * a * c) {
                             // the two divisions as one: lane 0 the multiplier, the others 1/|S|, from which
-                            // the threshold follows with one correction (to an ulp of the division)
+                            // two corrections give the threshold's correctly rounded quotient (Markstein:
+                            // with r = RN(1/a) and q within an ulp, q + (t - q a) r rounds to RN(t / a))
                             const double num = b * (sv - 1.0) - a * (smv - R);
                             const bool l0 = threadIdx.x == 0;
                             const double q = (l0 ? num : 1.0) / (l0 ? det : a);
                             nc = __shfl_sync(0xffffffffu, q, 0);
                             const double ra = __shfl_sync(0xffffffffu, q, 1);
                             const double t = fma(nc, b, sv) - 1.0, t0 = t * ra;
-                            tc = fma(fma(-t0, a, t), ra, t0);
+                            const double t1 = fma(fma(-t0, a, t), ra, t0);
+                            tc = fma(fma(-t1, a, t), ra, t1);
                             ok = !ge || nc >= 0.0;
                         }
                     }
@@ -918,11 +936,18 @@ struct ClusterProj {
                              int budget, const Side &side) {
         ProjOut o = search(R, mode, mu_min, mu_max, nu_hint, tau_hint, budget, side);
         if (o.status != MV_ERR_NOT_CONVERGED || dyk == nullptr || dyk_iters <= 0) return o;
+        ClusterProj safe = *this;              // a copy, so that this one stays in registers
+        return safeguarded(safe, o.steps, R, mode, mu_min, mu_max, budget);
+    }
+    // The safeguard and the search restarted from it.  Out of line: it runs
+    // almost never, and the instructions of a projection that does not need
+    // it should lie together (a step executes them once per launch).
+    __device__ __noinline__ static ProjOut safeguarded(ClusterProj &P, int steps, double R, int mode, double mu_min,
+                                                       double mu_max, int budget) {
         int sweeps = 0;
         double tau_d = -INFINITY;
-        const double theta = dykstra(R, mode, mu_min, mu_max, budget, sweeps, tau_d);
-        const int steps = o.steps;
-        o = search(R, mode, mu_min, mu_max, theta, tau_d, budget > 100 ? budget : 100);
+        const double theta = P.dykstra(R, mode, mu_min, mu_max, budget, sweeps, tau_d);
+        ProjOut o = P.search(R, mode, mu_min, mu_max, theta, tau_d, budget > 100 ? budget : 100);
         o.steps += steps;
         o.dykstra = 1;
         return o;

@@ -527,7 +527,7 @@ struct StepArgs {
     int dyk_iters = 0;
     int budget = kProjBudget;
     int momentum = 0;                      // 1: beta fixed at st->beta_c
-    int pad = 0;
+    int early = 0;                         // 1: launched as a programmatic dependent; 2: and warms up (npga_step_body)
     double bt_rho = 0.5;
     double m_f = 0.0;                      // curvature bound of the constant momentum
     double *gyw = nullptr;                 // backtracking: L L^T y (written), L L^T d, candidate x+
@@ -547,7 +547,17 @@ struct StepArgs {
 // the projection starts from the scales of the previous one (project.cuh).
 // KEEP: elements per thread kept so (2; 0 in the batch, whose blocks hold up
 // to six per thread and share an SM, so registers count more there).
-template <int CL, int KEEP>
+//
+// What is left is mostly instruction fetch: a launch executes about 40 KB of
+// straight-line code once, and after a pass over L not even L2 holds it (the
+// search's set-up took 4500 cycles at n = 200, 8000 behind a pass over L).  So
+// a step launched as a programmatic dependent (a.early) starts beside the
+// product and first projects a small made-up point through the same code,
+// nothing of which leaves shared memory; only then it waits for the product.
+// That takes about 8 us, so only beside a product that lasts longer and
+// sweeps L2 (a.early = 2): with it the 5440 x 48374 FP32 solve went from 15.8 to
+// 15.5 ms, a 200 x 1000 one from 3.4 to 4.5 ms.
+template <int CL, int KEEP, bool EARLY>
 __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char *dsm, ProjSmem &psm) {
     SolveState *st = a.st;
     const int n = a.n;
@@ -556,141 +566,183 @@ __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char 
     const int r0 = min(n, rank * nl);
     const int r1 = min(n, r0 + nl);
     ProjElems el = carve_elems(dsm, nl);
-    el.n = r1 - r0;
     // One element's vectors.
     struct Elem {
         double mu, gy, gx, x, y;
     };
     auto load = [&](int gi) { return Elem{a.mu[gi], a.gy[gi], a.gx[gi], a.x[gi], a.y[gi]}; };
     Elem keep[KEEP > 0 ? KEEP : 1];
-#pragma unroll
-    for (int j = 0; j < KEEP; ++j) {
-        const int i = threadIdx.x + j * kProjNT;
-        keep[j] = i < el.n ? load(r0 + i) : Elem{0.0, 0.0, 0.0, 0.0, 0.0};
-    }
-    const int k = st->k;
-    const double beta_prev = st->beta_prev, inv1pb = st->inv1pb, alpha = st->alpha, t = st->t;
-    const double mn = st->mu_min, mx = st->mu_max;
-    const double nu0 = st->nu, tau0 = st->tau;
-    const ScaleHint hint = st->hint;
     const double gamma = a.gamma;
-    // Every block reads the flag before the first cluster barrier; the flag is
-    // only written after later barriers, so the whole cluster agrees.
-    if (*(volatile int *)&st->done) return;
-    // Scalars computed once (FP64 is scarce on this part) and broadcast.
     __shared__ double sc[3];
-    auto momentum = [&] {
-        if (threadIdx.x == kProjNT - kWarp) {
-            double tn = t, beta = 0.0;
-            if (a.momentum == 1) {         // strongly convex specialisation: t unused, beta fixed
-                beta = st->beta_c;
-            } else {
-                tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
-                beta = (t - 1.0) / tn;
-            }
-            sc[0] = tn;
-            sc[1] = beta;
-            sc[2] = 1.0 / (1.0 + beta);
-        }
-    };
+    cluster_arrive<CL>();
     proj_smem_init(&psm);
-    const bool check = (a.kkt_every > 0 && k % a.kkt_every == 0) || (k >= a.max_iter);
-
-    // L L^T x^k by linearity from the product at y^k; the point to project:
-    // x - alpha grad f(x) on a KKT test, else the gradient step from y^k.
-    auto from_y = [&](const Elem &e) { return e.y - alpha * (2.0 * e.gy + 2.0 * gamma * e.y); };
-    auto first_point = [&](int i, const Elem &e) {
-        const double gxi = (k == 0) ? e.gy : (e.gy + beta_prev * e.gx) * inv1pb;
-        a.gx[r0 + i] = gxi;
-        el.mu[i] = e.mu;
-        el.v[i] = check ? e.x - alpha * (2.0 * gxi + 2.0 * gamma * e.x) : from_y(e);
-    };
-    // f(i, element) over the thread's elements (all of them private to it)
-    auto each = [&](auto f) {
-#pragma unroll
-        for (int j = 0; j < KEEP; ++j) {
-            const int i = threadIdx.x + j * kProjNT;
-            if (i < el.n) f(i, keep[j]);
-        }
-        for (int i = threadIdx.x + KEEP * kProjNT; i < el.n; i += kProjNT) f(i, load(r0 + i));
-    };
-    each(first_point);
     ClusterProj<CL> P{&psm, el};
-    P.dyk = dyk_slice(a.dyk, rank, nl);
-    P.dyk_iters = a.dyk_iters;
-    if (check) {
-        P.prepare(hint);
-        // warm start from this iteration's multipliers: x^k - alpha grad f(x^k)
-        // lies next to the point x^k was projected from (y^k -> x^k as the
-        // iterates settle), so its support usually matches and the search
-        // stops after the verifying exchange
-        // (measured the same as the previous test's multipliers: 37.6 against 37.8 us per step)
-        const ProjOut o = P.solve(a.R, a.mode, mn, mx, nu0, tau0, a.budget);
-        double r2 = 0.0;
+    bool real = !(EARLY && a.early == 2);
+    bool met = false;                      // the cluster's blocks have all started
+    while (true) {
+        // The made-up point: v = 2^-10, mu = 1 or 2, target 1.5 by equality; its
+        // support is everything and the candidate of the first reduction holds.
+        int k = 1, mode = MV_RETURN_EQ, budget = 2;
+        double beta_prev = 0.0, inv1pb = 1.0, alpha = 0.0, t = 1.0, mn = 1.0, mx = 2.0, nu0 = 0.0, tau0 = -1.0, R = 1.5;
+        ScaleHint hint{{1013, 1024, 1014, 1025}};
+        if (real) {
+            if constexpr (EARLY) {
+                umma::grid_dependency_wait();
+                umma::launch_dependents();         // the next fused pass may start streaming L
+            }
+            el.n = r1 - r0;
+#pragma unroll
+            for (int j = 0; j < KEEP; ++j) {
+                const int i = threadIdx.x + j * kProjNT;
+                if (i < el.n) keep[j] = load(r0 + i);
+            }
+            k = st->k;
+            beta_prev = st->beta_prev;
+            inv1pb = st->inv1pb;
+            alpha = st->alpha;
+            t = st->t;
+            mn = st->mu_min;
+            mx = st->mu_max;
+            nu0 = st->nu;
+            tau0 = st->tau;
+            hint = st->hint;
+            mode = a.mode;
+            budget = a.budget;
+            R = a.R;
+            P.dyk = dyk_slice(a.dyk, rank, nl);
+            P.dyk_iters = a.dyk_iters;
+            // Every block reads the flag before the first exchange; the flag is
+            // only written after later barriers, so the whole cluster agrees.
+            if (*(volatile int *)&st->done) {
+                if (!met) cluster_wait<CL>();
+                return;
+            }
+        } else {
+            el.n = min(r1 - r0, KEEP * kProjNT);
+#pragma unroll
+            for (int j = 0; j < KEEP; ++j) keep[j] = Elem{1.0 + (threadIdx.x & 1), 0.0, 0.0, 0.0, 0x1p-10};
+        }
+        P.el.n = el.n;
+        // Scalars computed once (FP64 is scarce on this part) and broadcast.
+        auto momentum = [&](bool now) {
+            if (now && threadIdx.x == kProjNT - kWarp) {
+                double tn = t, beta = 0.0;
+                if (a.momentum == 1) {         // strongly convex specialisation: t unused, beta fixed
+                    beta = real ? st->beta_c : 0.0;
+                } else {
+                    tn = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
+                    beta = (t - 1.0) / tn;
+                }
+                sc[0] = tn;
+                sc[1] = beta;
+                sc[2] = 1.0 / (1.0 + beta);
+            }
+        };
+        const bool check = real && ((a.kkt_every > 0 && k % a.kkt_every == 0) || (k >= a.max_iter));
+
+        // L L^T x^k by linearity from the product at y^k; the point to project:
+        // x - alpha grad f(x) on a KKT test, else the gradient step from y^k.
+        auto from_y = [&](const Elem &e) { return e.y - alpha * (2.0 * e.gy + 2.0 * gamma * e.y); };
+        // f(i, element) over the thread's elements (all of them private to it)
+        auto each = [&](auto f) {
+#pragma unroll
+            for (int j = 0; j < KEEP; ++j) {
+                const int i = threadIdx.x + j * kProjNT;
+                if (i < el.n) f(i, keep[j]);
+            }
+            for (int i = threadIdx.x + KEEP * kProjNT; i < el.n; i += kProjNT) f(i, load(r0 + i));
+        };
         each([&](int i, const Elem &e) {
-            const double p = fmax(fma(o.nu, e.mu, el.v[i]) - o.tau, 0.0);
-            const double d = p - e.x;
-            r2 = fma(d, d, r2);
+            const double gxi = (k == 0) ? e.gy : (e.gy + beta_prev * e.gx) * inv1pb;
+            if (real) a.gx[r0 + i] = gxi;
+            el.mu[i] = e.mu;
+            el.v[i] = check ? e.x - alpha * (2.0 * gxi + 2.0 * gamma * e.x) : from_y(e);
         });
-        r2 = P.reduce_double(r2);          // identical in every block
-        const bool conv = r2 <= a.eps * a.eps;
-        const bool stop = conv || k >= a.max_iter || !(r2 == r2);
+        if (!met) cluster_wait<CL>();
+        met = true;
+        // pass 0: the KKT test's projection; pass 1: the step's.  (One copy of
+        // the search serves both.)  The test starts from this iteration's
+        // multipliers too: x^k - alpha grad f(x^k) lies next to the point x^k was
+        // projected from (y^k -> x^k as the iterates settle), so its support
+        // usually matches and the search stops after the verifying exchange.
+        ProjOut o;
+        for (int pass = check ? 0 : 1;; ++pass) {
+            P.prepare(hint);
+            o = P.solve(R, mode, mn, mx, nu0, tau0, budget, [&] { momentum(pass == 1); });
+            if (pass == 1) break;
+            double r2 = 0.0;
+            each([&](int i, const Elem &e) {
+                const double p = fmax(fma(o.nu, e.mu, el.v[i]) - o.tau, 0.0);
+                const double d = p - e.x;
+                r2 = fma(d, d, r2);
+            });
+            r2 = P.reduce_double(r2);          // identical in every block
+            const bool conv = r2 <= a.eps * a.eps;
+            const bool stop = conv || k >= a.max_iter || !(r2 == r2);
+            if (rank == 0 && threadIdx.x == 0) {
+                const double kkt = sqrt(r2);
+                st->kkt = kkt;
+                st->nu_kkt = o.nu;
+                st->tau_kkt = o.tau;
+                st->proj_steps += o.steps;
+                st->dykstra += o.dykstra;
+                if (o.status != MV_OK) st->proj_fail += 1;
+                if (stop) {
+                    st->done = 1;
+                    st->converged = conv ? 1 : 0;
+                    st->status = conv ? MV_OK : (!(r2 == r2) ? MV_ERR_NUMERIC : MV_ERR_NOT_CONVERGED);
+                }
+            }
+            if (stop) {
+                cluster_barrier<CL>();
+                return;
+            }
+            each([&](int i, const Elem &e) { el.v[i] = from_y(e); });
+        }
+        const double beta = sc[1];
+        each([&](int i, const Elem &e) {
+            const int gi = r0 + i;
+            const double xn = fmax(fma(o.nu, e.mu, el.v[i]) - o.tau, 0.0);
+            const double yn = xn + beta * (xn - e.x);
+            if (real) {
+                a.x[gi] = xn;
+                a.y[gi] = yn;
+                a.y32[gi] = (float)(yn * (a.row_scale ? (double)a.row_scale[gi] : 1.0));
+            }
+        });
+        if (!real) {
+            real = true;
+            continue;
+        }
         if (rank == 0 && threadIdx.x == 0) {
-            const double kkt = sqrt(r2);
-            st->kkt = kkt;
-            st->nu_kkt = o.nu;
-            st->tau_kkt = o.tau;
+            st->t = sc[0];
+            st->beta_prev = beta;
+            st->inv1pb = sc[2];
+            st->hint = P.scales();
+            st->k = k + 1;
+            st->nu = o.nu;
+            st->tau = o.tau;
+            if (o.status != MV_OK) st->proj_fail += 1;
             st->proj_steps += o.steps;
             st->dykstra += o.dykstra;
-            if (o.status != MV_OK) st->proj_fail += 1;
-            if (stop) {
+            if (o.status == MV_ERR_INFEASIBLE || o.status == MV_ERR_NUMERIC) {
                 st->done = 1;
-                st->converged = conv ? 1 : 0;
-                st->status = conv ? MV_OK : (!(r2 == r2) ? MV_ERR_NUMERIC : MV_ERR_NOT_CONVERGED);
+                st->status = o.status;
             }
         }
-        if (stop) {
-            cluster_barrier<CL>();
-            return;
-        }
-        each([&](int i, const Elem &e) { el.v[i] = from_y(e); });
+        cluster_barrier<CL>();   // no block leaves while a peer may still address its shared memory
+        return;
     }
-    P.prepare(hint);
-    const ProjOut o = P.solve(a.R, a.mode, mn, mx, nu0, tau0, a.budget, momentum);
-    const double beta = sc[1];
-    each([&](int i, const Elem &e) {
-        const int gi = r0 + i;
-        const double xn = fmax(fma(o.nu, e.mu, el.v[i]) - o.tau, 0.0);
-        const double yn = xn + beta * (xn - e.x);
-        a.x[gi] = xn;
-        a.y[gi] = yn;
-        a.y32[gi] = (float)(yn * (a.row_scale ? (double)a.row_scale[gi] : 1.0));
-    });
-    if (rank == 0 && threadIdx.x == 0) {
-        st->t = sc[0];
-        st->beta_prev = beta;
-        st->inv1pb = sc[2];
-        st->hint = P.scales();
-        st->k = k + 1;
-        st->nu = o.nu;
-        st->tau = o.tau;
-        if (o.status != MV_OK) st->proj_fail += 1;
-        st->proj_steps += o.steps;
-        st->dykstra += o.dykstra;
-        if (o.status == MV_ERR_INFEASIBLE || o.status == MV_ERR_NUMERIC) {
-            st->done = 1;
-            st->status = o.status;
-        }
-    }
-    cluster_barrier<CL>();   // no block leaves while a peer may still address its shared memory
 }
 
+// 96 registers: beside the fused pass (72 x 544) a step still fits an SM's file.
+constexpr int kStepRegs = 96;
 template <int CL>
-__global__ void __launch_bounds__(kProjNT) npga_step_kernel(StepArgs a) {
+__global__ void __maxnreg__(kStepRegs) npga_step_kernel(StepArgs a) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ ProjSmem psm;
-    umma::launch_dependents();     // the next fused pass may start streaming L
-    npga_step_body<CL, 2>(a, dsm, psm);
+    if (a.early == 0) umma::launch_dependents();     // the next fused pass may start streaming L
+    npga_step_body<CL, 2, true>(a, dsm, psm);
 }
 
 // Grouped form: cluster b runs the step of problem b.
@@ -699,7 +751,7 @@ __global__ void __launch_bounds__(kProjNT) npga_step_grouped(const StepArgs *__r
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ ProjSmem psm;
     const StepArgs a = args[blockIdx.x / CL];
-    npga_step_body<CL, 0>(a, dsm, psm);
+    npga_step_body<CL, 0, false>(a, dsm, psm);
 }
 
 // Sets up the Sec. 3.1 variants once alpha is known: the first backtracking
@@ -1109,7 +1161,20 @@ void gemv_t_only(const Plan &p, const mv_problem *P, const float *y32, void *ws,
 
 static size_t step_smem(int n, int CL) { return proj_elem_bytes((n + CL - 1) / CL); }
 
-static void launch_step(const Plan &p, const mv_problem *P, const mv_solve_opts *O, void *ws, cudaStream_t s) {
+// How a step that may start beside the product before it does (StepArgs::early).
+// A fused pass has to leave it the shared memory (its registers fit:
+// kStepRegs); where it does not, the step is launched the plain way.  The
+// made-up projection needs a product of some 20 us: one that reads more
+// than L2 holds.
+constexpr int64_t kWarmBytes = 128ll << 20;
+static int step_early(const Plan &p) {
+    constexpr size_t sm = 228 * 1024, fixed = 1024 + 64;      // reserved per block, and the pass's static bytes
+    if (p.use_llt && p.lp.smem + fixed + step_smem(p.n, p.cl) + sizeof(ProjSmem) + fixed > sm) return 0;
+    return p.use_llt && (int64_t)p.gr * p.ld * p.esize >= kWarmBytes ? 2 : 1;
+}
+
+static void launch_step(const Plan &p, const mv_problem *P, const mv_solve_opts *O, void *ws, cudaStream_t s,
+                        bool early = false) {
     StepArgs a;
     a.st = at<SolveState>(ws, p.o_state);
     a.gy = at<double>(ws, p.o_gy);
@@ -1146,12 +1211,14 @@ static void launch_step(const Plan &p, const mv_problem *P, const mv_solve_opts 
         }
         return;
     }
+    a.early = early ? step_early(p) : 0;
+    const bool pdl = a.early != 0;
     switch (p.cl) {
-        case 1: launch_cluster(npga_step_kernel<1>, 1, sm, s, a); break;
-        case 2: launch_cluster(npga_step_kernel<2>, 2, sm, s, a); break;
-        case 4: launch_cluster(npga_step_kernel<4>, 4, sm, s, a); break;
-        case 8: launch_cluster(npga_step_kernel<8>, 8, sm, s, a); break;
-        default: launch_cluster(npga_step_kernel<16>, 16, sm, s, a); break;
+        case 1: launch_cluster_pdl(npga_step_kernel<1>, 1, sm, s, pdl, a); break;
+        case 2: launch_cluster_pdl(npga_step_kernel<2>, 2, sm, s, pdl, a); break;
+        case 4: launch_cluster_pdl(npga_step_kernel<4>, 4, sm, s, pdl, a); break;
+        case 8: launch_cluster_pdl(npga_step_kernel<8>, 8, sm, s, pdl, a); break;
+        default: launch_cluster_pdl(npga_step_kernel<16>, 16, sm, s, pdl, a); break;
     }
 }
 
@@ -1222,7 +1289,7 @@ int launch_iteration(const Plan &p, const mv_problem *P, const mv_solve_opts *O,
                               kLoopPdl && ev == nullptr));   // timed runs keep launches apart
         if (ev) cudaEventRecord(ev[1], s);
         if (ev) cudaEventRecord(ev[2], s);
-        launch_step(p, P, O, ws, s);
+        launch_step(p, P, O, ws, s, kLoopPdl && ev == nullptr);
         if (ev) cudaEventRecord(ev[3], s);
         return MV_OK;
     }
@@ -1230,7 +1297,7 @@ int launch_iteration(const Plan &p, const mv_problem *P, const mv_solve_opts *O,
     if (ev) cudaEventRecord(ev[1], s);
     launch_g(p, P, at<float>(ws, p.o_z), ws, done, gy, nullptr, s, kLoopPdl && ev == nullptr);
     if (ev) cudaEventRecord(ev[2], s);
-    launch_step(p, P, O, ws, s);
+    launch_step(p, P, O, ws, s, kLoopPdl && ev == nullptr);
     if (ev) cudaEventRecord(ev[3], s);
     return MV_OK;
 }

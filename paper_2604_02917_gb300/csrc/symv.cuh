@@ -22,6 +22,7 @@
 #pragma once
 
 #include "mv_internal.cuh"
+#include "umma.cuh"
 
 namespace mv {
 
@@ -101,6 +102,7 @@ __device__ __forceinline__ void symv_finish_block(const SymvArgs &a, int b, floa
 }
 
 static __global__ void __launch_bounds__(kSymThreads) symv_kernel(SymvArgs a) {
+    umma::launch_dependents();                // the step may start beside this pass
     if (a.done && *(volatile const int *)a.done) return;
     __shared__ float yI[kSymTile], yJ[kSymTile];
     __shared__ float colred[kSymThreads / kWarp][kSymTile];
