@@ -40,8 +40,6 @@ int record_message(int status, const char *msg) {
     return status;
 }
 
-constexpr int kCenterThreads = 512;
-
 // Sum of FP32 values, exact but for the final rounding.  A value is a 24-bit
 // significand m (signed) times 2^(e - 150); m << (e - eb) is added to a
 // 64-bit integer while e lies in [eb, eb + 30] (under 2^54 each, so 256 of
@@ -123,50 +121,72 @@ __device__ __forceinline__ RowConst row_const(double mean, double c, float amax)
     return k;
 }
 
-// Sum of squares of FP32 pairs (p, r): s + c carries about 48 bits per
-// thread; values centred in FP64 are added in FP64.
+// Two FP32 values per instruction (sm_100 and later): a centred entry is
+// about 28 FP32 operations, and issue slots, not the pipe, bound the kernels.
+__device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+
+// Sum of squares of FP32 pairs (p, r), two at a time: s + c carries about 48
+// bits per thread; values centred in FP64 are added in FP64.
 struct SquareSum {
-    float s = 0.f, c = 0.f;
+    float2 s = make_float2(0.f, 0.f), c = make_float2(0.f, 0.f);
     double wide = 0.0;
-    __device__ __forceinline__ void add(float p, float r) {
-        const float q = p * p;
-        float e = fmaf(p, p, -q);                       // p^2 = q + e exactly
-        e = fmaf(fmaf(2.f, p, r), r, e);
-        const float t = s + q, bb = t - s;              // s + q = t + (rounding error), exactly
-        c += ((s - (t - bb)) + (q - bb)) + e;
+    __device__ __forceinline__ void add(float2 p, float2 r) {
+        const float2 q = __fmul2_rn(p, p);
+        float2 e = __ffma2_rn(p, p, neg2(q));                       // p^2 = q + e exactly
+        e = __ffma2_rn(__ffma2_rn(splat(2.f), p, r), r, e);
+        const float2 t = __fadd2_rn(s, q), bb = sub2(t, s);         // s + q = t + (rounding error), exactly
+        c = __fadd2_rn(c, __fadd2_rn(__fadd2_rn(sub2(s, sub2(t, bb)), sub2(q, bb)), e));
         s = t;
     }
-    __device__ __forceinline__ double total() const { return wide + ((double)s + (double)c); }
+    __device__ __forceinline__ double total() const {
+        return wide + (((double)s.x + (double)c.x) + ((double)s.y + (double)c.y));
+    }
 };
 
-// FP32 rounding of d = (x - mean) c.  x - mh is exact as the pair (s, e);
-// the product with the pair (ch, cl) leaves d = p + r with an error below
-// 7 x 2^-48 |p| + 3 x 2^-48 |mh| ch (unit roundoff 2^-24 in each of the
-// pair's low parts), and r +- tol adds 3 x 2^-48 |p| + 2^-48 |mh| ch: inside
-// tol = 2^-44 (|p| + |mh| ch) for rows inside row_const's limits.  Where p + r - tol and p + r +
-// tol round to the same FP32 value that value is the rounding of the FP64
-// result too; elsewhere (about one entry in 2^18) d is formed in FP64.
-// BF16 adds one case: an FP32 value on a BF16 tie does not say which way
-// the FP64 value rounds.  ~17 FP32 operations, against 3 FP64 ones and a
-// conversion.  Returns the stored FP32 value (d64 the FP64 one on that path,
-// `exact` set) and adds d^2 to q.
+// FP32 roundings of d = (x - mean) c for two entries of a row.  x - mh is
+// exact as the pair (s, e); the product with the pair (ch, cl) leaves d = p + r
+// with an error below 7 x 2^-48 |p| + 3 x 2^-48 |mh| ch (unit roundoff 2^-24
+// in each of the pair's low parts), and r +- tol adds 3 x 2^-48 |p| + 2^-48
+// |mh| ch: inside tol = 2^-44 (|p| + |mh| ch) for rows inside row_const's
+// limits.  Where p + r - tol and p + r + tol round to the same FP32 value that
+// value is the rounding of the FP64 result too; elsewhere (about one entry in
+// 2^18) d is formed in FP64.  BF16 adds one case: an FP32 value on a BF16 tie
+// does not say which way the FP64 value rounds.  Returns the values to store
+// (for BF16 already rounded to it on the FP64 path) and adds the squares of
+// the first `use` entries to q.
 template <int DT>
-__device__ __forceinline__ float centred(float x, const RowConst &k, double mean, double c, SquareSum &q, double &d64,
-                                         bool &exact) {
-    const float s = x - k.mh, bb = s - x;
-    const float e = ((x - (s - bb)) - (k.mh + bb)) - k.ml;
-    const float p = s * k.ch;
-    float r = fmaf(s, k.ch, -p);
-    r = fmaf(s, k.cl, r);
-    r = fmaf(e, k.ch, r);
-    const float tol = fmaf(fabsf(p), 0x1p-44f, k.wide);
-    const float f = p + (r - tol);
-    exact = !(f == p + (r + tol));
-    if constexpr (DT == MV_BF16) exact = exact || (__float_as_uint(f) & 0xffffu) == 0x8000u;
-    if (exact) {
-        d64 = ((double)x - mean) * c;
-        q.wide = fma(d64, d64, q.wide);
-        return (float)d64;
+__device__ __forceinline__ float2 centred(float2 x, const RowConst &k, double mean, double c, int use, SquareSum &q) {
+    const float2 mh = splat(k.mh), ch = splat(k.ch);
+    const float2 s = sub2(x, mh), bb = sub2(s, x);
+    const float2 e = sub2(sub2(sub2(x, sub2(s, bb)), __fadd2_rn(mh, bb)), splat(k.ml));
+    float2 p = __fmul2_rn(s, ch);
+    float2 r = __ffma2_rn(s, ch, neg2(p));
+    r = __ffma2_rn(s, splat(k.cl), r);
+    r = __ffma2_rn(e, ch, r);
+    const float2 tol = __ffma2_rn(make_float2(fabsf(p.x), fabsf(p.y)), splat(0x1p-44f), splat(k.wide));
+    float2 f = __fadd2_rn(p, sub2(r, tol));
+    const float2 f1 = __fadd2_rn(p, __fadd2_rn(r, tol));
+    bool wx = !(f.x == f1.x), wy = !(f.y == f1.y);
+    if constexpr (DT == MV_BF16) {
+        wx = wx || (__float_as_uint(f.x) & 0xffffu) == 0x8000u;
+        wy = wy || (__float_as_uint(f.y) & 0xffffu) == 0x8000u;
+    }
+    if (wx || wy || use < 2) {
+        auto in64 = [&](float v) {
+            const double d = ((double)v - mean) * c;
+            q.wide = fma(d, d, q.wide);
+            return DT == MV_BF16 ? __bfloat162float(__double2bfloat16(d)) : (float)d;
+        };
+        if (wx || use < 1) {
+            if (use >= 1) f.x = in64(x.x);
+            p.x = r.x = 0.f;
+        }
+        if (wy || use < 2) {
+            if (use >= 2) f.y = in64(x.y);
+            p.y = r.y = 0.f;
+        }
     }
     q.add(p, r);
     return f;
@@ -183,95 +203,112 @@ __device__ __forceinline__ void store_elem(void *L, int64_t idx, float val, floa
     }
 }
 
-// The value to store for an entry of R: for BF16 already rounded to it (from
-// FP64 where the FP32 value would round twice).
-template <int DT>
-__device__ __forceinline__ float centred_value(float x, const RowConst &k, double mean, double c, SquareSum &q) {
-    double d64 = 0.0;
-    bool exact;
-    const float f = centred<DT>(x, k, mean, c, q, d64, exact);
-    if constexpr (DT == MV_BF16)
-        if (exact) return __bfloat162float(__double2bfloat16(d64));
-    return f;
-}
-
-// One block per asset row.  Pass 1: mu_i = sum_t R_it / T and the FP32 range
-// of the row; the FP8 scale max_t |d_it| / 448 follows exactly from it,
-// because d = ((double)x - mu) c is monotone in x.  Pass 2 (WRITE): the
-// centred entries, stored in the storage type, and their squares for the
+// One block of NT threads per asset row.  Pass 1: mu_i = sum_t R_it / T and
+// the FP32 range of the row; the FP8 scale max_t |d_it| / 448 follows exactly
+// from it, because d = ((double)x - mu) c is monotone in x.  Pass 2 (WRITE):
+// the centred entries, stored in the storage type, and their squares for the
 // trace; the re-read of the row mostly hits L2.  With WRITE = false
 // (transposed layout) pass 2 is done by transpose_center_kernel, which finds
 // the row's largest |R| in amax.  Entries are read one per lane (rows of a
-// ragged panel share no 16-byte alignment), kUnroll loads in flight.
+// ragged panel share no 16-byte alignment), kCenterUnroll loads in flight.
+// NT: FP64 runs once per thread and warp here (the thread totals and the
+// shuffles over them), about 3000 cycles of the SM's FP64 pipe per block of
+// 512, so long panels take 128 threads per row (more rows in flight instead);
+// panels of fewer rows than that fills take 512.
 constexpr int kCenterUnroll = 8;
-template <int DT, bool WRITE>
-__global__ void __launch_bounds__(kCenterThreads)
+constexpr int kRowThreads = 128, kRowThreadsFew = 512;
+template <int DT, bool WRITE, int NT>
+__global__ void __launch_bounds__(NT)
 center_kernel(const float *__restrict__ R, int64_t ldR, unsigned T, void *__restrict__ L, int64_t ldL,
               float *__restrict__ row_scale, double *__restrict__ mu, double *__restrict__ rowsq,
               float *__restrict__ amax_out, int64_t i_base) {
     constexpr int U = kCenterUnroll;
-    __shared__ double red[(kCenterThreads / kWarp + 1) * 2];
+    __shared__ double red[NT / kWarp + 1];
+    __shared__ float s_lo[NT / kWarp], s_hi[NT / kWarp];
     const int64_t i = i_base + blockIdx.x;                 // asset; R holds rows i_base ..
     const float *r = R + (int64_t)blockIdx.x * ldR;
     RowSum sum;
     float xmin = INFINITY, xmax = -INFINITY;
+    auto range = [&](float x) {
+        if constexpr (DT == MV_FP8_E4M3) {
+            xmin = fminf(xmin, x);
+            xmax = fmaxf(xmax, x);
+        } else {
+            xmax = fmaxf(xmax, fabsf(x));                   // only the largest |x| is needed
+        }
+    };
     unsigned t = threadIdx.x;
     int since = 0;
-    for (; t + (U - 1) * kCenterThreads < T; t += U * kCenterThreads) {
+    for (; t + (U - 1) * NT < T; t += U * NT) {
         float x[U];
 #pragma unroll
-        for (int k = 0; k < U; ++k) x[k] = r[t + k * kCenterThreads];
+        for (int k = 0; k < U; ++k) x[k] = r[t + k * NT];
         sum.add(x);
 #pragma unroll
-        for (int k = 0; k < U; ++k) {
-            xmin = fminf(xmin, x[k]);
-            xmax = fmaxf(xmax, x[k]);
-        }
+        for (int k = 0; k < U; ++k) range(x[k]);
         since += U;
         if (since >= 240) {                                 // at most 256 values in the integer
             sum.flush();
             since = 0;
         }
     }
-    for (; t < T; t += kCenterThreads) {                    // fewer than U values
+    for (; t < T; t += NT) {                                // fewer than U values
         const float x[1] = {r[t]};
         sum.add(x);
-        xmin = fminf(xmin, x[0]);
-        xmax = fmaxf(xmax, x[0]);
+        range(x[0]);
+    }
+    const int lane = threadIdx.x % kWarp, warp = threadIdx.x / kWarp;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        xmin = fminf(xmin, __shfl_xor_sync(0xffffffffu, xmin, o));
+        xmax = fmaxf(xmax, __shfl_xor_sync(0xffffffffu, xmax, o));
+    }
+    if (lane == 0) {
+        s_lo[warp] = xmin;
+        s_hi[warp] = xmax;
     }
     double s[1] = {sum.total()};
-    block_sum<1, kCenterThreads>(s, red);
+    block_sum<1, NT>(s, red);                               // its barriers publish s_lo and s_hi too
+#pragma unroll
+    for (int w = 0; w < NT / kWarp; ++w) {
+        xmin = fminf(xmin, s_lo[w]);
+        xmax = fmaxf(xmax, s_hi[w]);
+    }
     const double mean = s[0] / (double)T;
     const double c = 1.0 / sqrt((double)(T - 1));
-    double mn = (double)xmin, mx = (double)xmax;
-    __syncthreads();
-    block_minmax<kCenterThreads>(mn, mx, red);
-    float inv_scale = 1.f;
+    float inv_scale = 1.f, ra = xmax;
     if constexpr (DT == MV_FP8_E4M3) {
-        const double amax = fmax((mx - mean) * c, (mean - mn) * c);
+        const double amax = fmax(((double)xmax - mean) * c, (mean - (double)xmin) * c);
         const float scale = amax > 0.0 ? (float)(amax / 448.0) : 1.f;
         inv_scale = 1.f / scale;
         if (threadIdx.x == 0) row_scale[i] = scale;
+        ra = fmaxf(fabsf(xmin), fabsf(xmax));
     }
-    const float ra = fmaxf(fabsf((float)mn), fabsf((float)mx));
     if constexpr (WRITE) {
         const RowConst k = row_const(mean, c, ra);
         SquareSum q;
-        int64_t o = i * ldL;
+        const int64_t o = i * ldL;
+        auto write2 = [&](float2 x, unsigned ta, unsigned tb, int use) {
+            const float2 f = centred<DT>(x, k, mean, c, use, q);
+            store_elem<DT>(L, o + ta, f.x, inv_scale);
+            if (use > 1) store_elem<DT>(L, o + tb, f.y, inv_scale);
+        };
         t = threadIdx.x;
-        for (; t + (U - 1) * kCenterThreads < T; t += U * kCenterThreads) {
+        for (; t + (U - 1) * NT < T; t += U * NT) {
             float x[U];
 #pragma unroll
-            for (int j = 0; j < U; ++j) x[j] = r[t + j * kCenterThreads];
+            for (int j = 0; j < U; ++j) x[j] = r[t + j * NT];
 #pragma unroll
-            for (int j = 0; j < U; ++j)
-                store_elem<DT>(L, o + t + j * kCenterThreads, centred_value<DT>(x[j], k, mean, c, q), inv_scale);
+            for (int j = 0; j < U; j += 2) write2(make_float2(x[j], x[j + 1]), t + j * NT, t + (j + 1) * NT, 2);
         }
-        for (; t < T; t += kCenterThreads) store_elem<DT>(L, o + t, centred_value<DT>(r[t], k, mean, c, q), inv_scale);
-        for (int64_t z = (int64_t)T + threadIdx.x; z < ldL; z += kCenterThreads) store_elem<DT>(L, o + z, 0.f, inv_scale);
+        for (; t < T; t += 2 * NT) {
+            const bool two = t + NT < T;
+            write2(make_float2(r[t], two ? r[t + NT] : 0.f), t, t + NT, two ? 2 : 1);
+        }
+        for (int64_t z = (int64_t)T + threadIdx.x; z < ldL; z += NT) store_elem<DT>(L, o + z, 0.f, inv_scale);
         double v[1] = {q.total()};
         __syncthreads();
-        block_sum<1, kCenterThreads>(v, red);
+        block_sum<1, NT>(v, red);
         if (threadIdx.x == 0) rowsq[i] = v[0];
     } else if (threadIdx.x == 0) {
         amax_out[i] = ra;
@@ -315,33 +352,44 @@ transpose_center_kernel(const float *__restrict__ R, int64_t ldR, int64_t n, int
     __syncthreads();
     const float inv = (DT == MV_FP8_E4M3 && i0 + lane < n) ? 1.f / row_scale[i0 + lane] : 1.f;
     SquareSum q;
+    const bool inside = i0 + kTile <= n;               // every asset of the tile exists (and ldM >= n)
+    const float *src = R + (i0 - i_base + warp) * ldR + lane;
     for (int t0 = tb; t0 < te; t0 += kTileT) {
+        const bool full = inside && te - t0 >= kTileT;
         float x[RPW][H];
+        if (full) {
 #pragma unroll
-        for (int j = 0; j < RPW; ++j) {
-            const int64_t i = i0 + warp + j * W;
-            const float *row = R + (i - i_base) * ldR + t0 + lane;
+            for (int j = 0; j < RPW; ++j)
 #pragma unroll
-            for (int h = 0; h < H; ++h) x[j][h] = (i < n && lane + h * kWarp < te - t0) ? row[h * kWarp] : 0.f;
+                for (int h = 0; h < H; ++h) x[j][h] = src[(int64_t)(j * W) * ldR + t0 + h * kWarp];
+        } else {
+#pragma unroll
+            for (int j = 0; j < RPW; ++j)
+#pragma unroll
+                for (int h = 0; h < H; ++h)
+                    x[j][h] = i0 + warp + j * W < n && lane + h * kWarp < te - t0 ? src[(int64_t)(j * W) * ldR + t0 + h * kWarp]
+                                                                                   : 0.f;
         }
 #pragma unroll
         for (int j = 0; j < RPW; ++j) {
             const int a = warp + j * W;
             const RowConst k = s_k[a];
 #pragma unroll
-            for (int h = 0; h < H; ++h)
-                if (i0 + a < n && lane + h * kWarp < te - t0)
-                    tile[a][lane + h * kWarp] = centred_value<DT>(x[j][h], k, s_mean[a], c, q);
-                else
-                    tile[a][lane + h * kWarp] = 0.f;
+            for (int h = 0; h < H; h += 2) {
+                // entries of the tile that exist: all, or those below te of an existing asset
+                int use = 2;
+                if (!full) use = i0 + a >= n ? 0 : min(2, max(0, (te - t0 - lane - h * kWarp + kWarp - 1) / kWarp));
+                const float2 f = centred<DT>(make_float2(x[j][h], x[j][h + 1]), k, s_mean[a], c, use, q);
+                tile[a][lane + h * kWarp] = use > 0 ? f.x : 0.f;
+                tile[a][lane + (h + 1) * kWarp] = use > 1 ? f.y : 0.f;
+            }
         }
         __syncthreads();
         if (i0 + lane < ldM) {
+            const int64_t at = (int64_t)(t0 + warp) * ldM + i0 + lane;
 #pragma unroll
-            for (int j = 0; j < kTileT / W; ++j) {
-                const int w = warp + j * W;
-                if (t0 + w < te) store_elem<DT>(M, (int64_t)(t0 + w) * ldM + i0 + lane, tile[lane][w], inv);
-            }
+            for (int j = 0; j < kTileT / W; ++j)
+                if (full || j * W + warp < te - t0) store_elem<DT>(M, at + (int64_t)(j * W) * ldM, tile[lane][warp + j * W], inv);
         }
         __syncthreads();
     }
@@ -351,6 +399,7 @@ transpose_center_kernel(const float *__restrict__ R, int64_t ldR, int64_t n, int
 }
 
 // trace(Sigma): the sum of the blocks' partials, in a fixed order.
+constexpr int kCenterThreads = 512;
 __global__ void __launch_bounds__(kCenterThreads)
 trace_kernel(const double *__restrict__ part, int64_t count, double *__restrict__ trace) {
     __shared__ double red[(kCenterThreads / kWarp + 1) * 1];
@@ -377,17 +426,19 @@ static void center_chunk(const float *R_rows, int64_t ldR, int64_t n, int64_t T,
                          int64_t ldL, float *d_row_scale, double *d_mu, double *rowsq, float *amax, int64_t i0,
                          int64_t i1, int slices, cudaStream_t s) {
     const unsigned rows = (unsigned)(i1 - i0);
+    const bool few = rows < 152 * 8;                           // one row per block: about 8 blocks of 128 per SM
     const int64_t wend = (tn && i1 == n) ? ldL : i1;          // transposed: columns written by this chunk
     const dim3 tgrid((unsigned)slices, (unsigned)((wend - i0 + kTile - 1) / kTile));
+#define MV_CENTER_ROWS(DT, WRITE, NT, RS)                                                                        \
+    center_kernel<DT, WRITE, NT><<<rows, NT, 0, s>>>(R_rows, ldR, (unsigned)T, WRITE ? d_L : nullptr, ldL, RS,   \
+                                                     d_mu, rowsq, amax, i0)
 #define MV_CENTER_CASE(DT, RS)                                                                                   \
     if (tn) {                                                                                                    \
-        center_kernel<DT, false><<<rows, kCenterThreads, 0, s>>>(R_rows, ldR, (unsigned)T, nullptr, 0, RS, d_mu, \
-                                                                 rowsq, amax, i0);                               \
+        if (few) MV_CENTER_ROWS(DT, false, kRowThreadsFew, RS); else MV_CENTER_ROWS(DT, false, kRowThreads, RS); \
         transpose_center_kernel<DT><<<tgrid, kTransThreads, 0, s>>>(R_rows, ldR, n, (int)T, d_L, ldL, RS, d_mu,  \
                                                                     amax, rowsq, i0, slices);                    \
     } else {                                                                                                     \
-        center_kernel<DT, true><<<rows, kCenterThreads, 0, s>>>(R_rows, ldR, (unsigned)T, d_L, ldL, RS, d_mu,    \
-                                                                rowsq, amax, i0);                                \
+        if (few) MV_CENTER_ROWS(DT, true, kRowThreadsFew, RS); else MV_CENTER_ROWS(DT, true, kRowThreads, RS);   \
     }
     switch (out_dtype) {
         case MV_F32: MV_CENTER_CASE(MV_F32, nullptr) break;
@@ -395,6 +446,7 @@ static void center_chunk(const float *R_rows, int64_t ldR, int64_t n, int64_t T,
         default: MV_CENTER_CASE(MV_FP8_E4M3, d_row_scale) break;
     }
 #undef MV_CENTER_CASE
+#undef MV_CENTER_ROWS
 }
 
 static int center_args(const void *R, int64_t n, int64_t T, int64_t ldR, int out_dtype, int layout, void *d_L,
