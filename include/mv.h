@@ -310,7 +310,9 @@ int mv_npga_solve(const mv_problem *P, const mv_solve_opts *opts, double *d_x_in
  *  ld = ldS: each NPGA iteration reads the upper triangle of Sigma once
  *  (n^2/2 FP32, held in L2 for n up to about 5500) instead of L twice.
  *  d_ws: mv_sigma_workspace_size(P) bytes (256-byte aligned; the BF16
- *  split or expansion of L, 2 n T or 4 n T bytes).  Blocking: returns
+ *  split or expansion of L, 2 n T or 4 n T bytes, and 20 MB for partial
+ *  sums of tiles cut along T, which the call does without if they are not
+ *  there: then MV_BF16 needs no workspace at all).  Blocking: returns
  *  after the GEMM, MV_ERR_TIMEOUT if a pipeline wait gave up.
  * ------------------------------------------------------------------------ */
 size_t mv_sigma_workspace_size(const mv_problem *P);

@@ -2,10 +2,11 @@
 // NPGA with grad f(x) = 2 Sigma x, O(n^2) per iteration) formed once on the
 // tcgen05 tensor cores.
 //
-// Sigma is symmetric, so only the 128 x 128 tiles (I, J) with I <= J are
-// multiplied (one CTA per tile, nb (nb + 1) / 2 of them); the epilogue writes
-// each tile and its mirror, so the stored Sigma is exactly symmetric.  On a
-// diagonal tile only the entries with col >= row are kept and mirrored.
+// Sigma is symmetric, so only the 256 x 256 tiles (I, J) with I <= J are
+// multiplied, each by a pair of CTAs (cluster of 2, cta_group::2 MMAs); the
+// epilogue writes each tile and its mirror, so the stored Sigma is exactly
+// symmetric.  On a diagonal tile only the entries with col >= row are kept
+// and mirrored.
 //
 // Operands are BF16, K-major (row t of L along T), FP32 accumulation:
 //   MV_BF16  L itself, one K-segment;
@@ -18,18 +19,35 @@
 //            into one accumulator (the dropped D D^T and the rounding of D
 //            are below 2^-16 |L_i| |L_j| per product term).
 //
-// Pipeline per CTA as in gemm.cuh: warp 0 (one thread) TMA producer over a
-// 6-stage ring, warp 1 (one thread) MMA issuer (128 x 128 x 16 per
-// instruction), warps 2..5 the epilogue, which also carries the running
-// sum in FP32 registers (see the accumulation note below).  Every wait is bounded in time; a
-// timeout is recorded in the device error word and the call returns
-// MV_ERR_TIMEOUT.
+// Bound: tensor.  A CTA of a pair loads its 128 rows of the I panel and its
+// 128 of the J panel: 64 KB per k-step of 3 x 256 x 256 x 64 multiply-adds
+// (FP32), half of what a CTA alone on a 128 x 128 tile needs per
+// multiply-add, which had made the L2 the limit (1.16 PFLOP/s).
+//
+// Work split.  P pairs fit the chip (one per two SMs).  All tiles but the
+// last N mod P run whole; those last r tiles would leave most of a wave
+// idle, so each is cut into floor(P / r) K-ranges whose partial sums go to
+// the workspace and are added in range order by a second kernel.  With few
+// tiles (small n) all of them are cut.
+//
+// Pipeline per CTA as in gemm_chunk.cuh's pair kernel: warp 0 (one thread)
+// TMA producer, warp 1 of rank 0 (one thread) MMA issuer, warps 2..9 the
+// epilogue, which also carries the running sum in FP32 registers (see the
+// accumulation note below).  Every wait is bounded in time; a timeout is
+// recorded in the device error word and the call returns MV_ERR_TIMEOUT.
+#include <cooperative_groups.h>
+
 #include "gemm.cuh"
 
 namespace mv {
 
-constexpr int kSigTile = 128;                 // BM = BN
-constexpr uint32_t kSigBox = kSigTile * kBK * 2;   // one 128 x 64 BF16 operand box (16 KB)
+int sm_count();          // solve.cu
+
+constexpr int kSigTile = 256;                      // rows and columns of a pair's tile
+constexpr int kSigHalf = kSigTile / 2;             // rows of each panel that one CTA loads
+constexpr uint32_t kSigBox = kSigHalf * kBK * 2;   // one 128 x 64 BF16 operand box (16 KB)
+constexpr int kSigEpiWarps = 8;                    // 128 rows x 2 column groups of 128
+constexpr int kSigThreads = 64 + 32 * kSigEpiWarps;
 // Stage geometry by number of products per k-step: one (BF16, FP8) = boxes
 // A, B and 6 stages; three (FP32 split) = boxes H_I, D_I, H_J, D_J and 3 stages.
 // A tensor-memory partial sums at most 64 MMAs (16 k-steps x 4, or 5 x 12).
@@ -43,16 +61,16 @@ constexpr size_t kSigSmem = 1024 + 6 * (size_t)2 * kSigBox + (2 * 6 + 4) * 8 + 1
 
 // Tile order: the upper triangle is walked in super-blocks of kSigGroup x
 // kSigGroup tiles (row-major inside each, super-blocks row-major over the
-// upper triangle), so the ~150 CTAs that run at the same time share about
+// upper triangle), so the pairs that run at the same time share about
 // 2 kSigGroup operand panels and read them from L2 rather than HBM.
-constexpr int kSigGroup = 12;
+constexpr int kSigGroup = 6;
 
-__device__ __forceinline__ void tile_of(int t, int nb, int &I, int &J) {
+__host__ __device__ __forceinline__ void tile_of(int t, int nb, int &I, int &J) {
     const int nsb = (nb + kSigGroup - 1) / kSigGroup;
     for (int P = 0; P < nsb; ++P) {
-        const int i0 = P * kSigGroup, ri = min(nb, i0 + kSigGroup) - i0;
+        const int i0 = P * kSigGroup, ri = nb - i0 < kSigGroup ? nb - i0 : kSigGroup;
         for (int Q = P; Q < nsb; ++Q) {
-            const int j0 = Q * kSigGroup, rj = min(nb, j0 + kSigGroup) - j0;
+            const int j0 = Q * kSigGroup, rj = nb - j0 < kSigGroup ? nb - j0 : kSigGroup;
             if (Q == P) {                             // triangle of ri (ri + 1) / 2 tiles
                 const int cnt = ri * (ri + 1) / 2;
                 if (t < cnt) {
@@ -80,39 +98,68 @@ __device__ __forceinline__ void tile_of(int t, int nb, int &I, int &J) {
     I = J = 0;                                        // not reached: t < nb (nb + 1) / 2
 }
 
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+// Whole tiles first, then `cut` tiles of `parts` K-ranges each.
+struct SigSplit {
+    int whole, cut, parts;
+};
+constexpr int kSigMaxParts = 64;
+static SigSplit sigma_split(int64_t tiles, int pairs, int chunks) {
+    SigSplit w;
+    w.whole = (int)(tiles / pairs * pairs);
+    w.cut = (int)(tiles - w.whole);
+    w.parts = w.cut > 0 ? std::min(std::min(pairs / w.cut, chunks), kSigMaxParts) : 1;
+    if (w.parts < 2) {
+        w.whole = (int)tiles;
+        w.cut = 0;
+        w.parts = 1;
+    }
+    return w;
 }
 
 // Accumulation.  The tensor core adds each MMA's products into the FP32
 // accumulator with a rounding that loses up to about an ulp of the running
 // sum, with one sign when the terms have one sign (the diagonal of Sigma):
 // over thousands of MMAs that is a bias of order 1e-4.  So a tile is
-// accumulated in chunks of at most 64 MMAs (SigGeo::CHUNK k-steps), alternately into two
-// 128-column tensor-memory buffers; the epilogue warps add every finished
-// chunk into FP32 registers (round-to-nearest, fixed order) while the MMA
-// warp fills the other buffer.
+// accumulated in chunks of at most 64 MMAs (SigGeo::CHUNK k-steps), alternately
+// into two 256-column tensor-memory buffers; the epilogue warps add every
+// finished chunk into FP32 registers (round-to-nearest, fixed order) while
+// the MMA warp fills the other buffer.
 template <int NSEG>
-__global__ void __launch_bounds__(kGemmThreads, 1)
-sigma_gemm_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmD, int n, int K,
-                  int nb, const float *__restrict__ rs, float *__restrict__ Sig, int64_t ldS) {
+__global__ void __launch_bounds__(kSigThreads, 1)
+sigma_pair_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmD, int n, int K,
+                  int nb, SigSplit w, const float *__restrict__ rs, float *__restrict__ Sig, int64_t ldS,
+                  float *__restrict__ part) {
     using Geo = SigGeo<NSEG>;
     constexpr int S = Geo::S;
+    constexpr uint32_t COLS = 2 * kSigTile;           // tensor-memory columns: all 512
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *smem = smem_raw + ((1024u - (uint32_t)(reinterpret_cast<uintptr_t>(smem_raw) & 1023u)) & 1023u);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + S * Geo::STAGE);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * S + 4);
     const uint32_t full0 = umma::smem_u32(bars), empty0 = umma::smem_u32(bars + S);
-    const uint32_t accf0 = umma::smem_u32(bars + 2 * S), acce0 = umma::smem_u32(bars + 2 * S + 2);
+    const uint32_t tfull0 = umma::smem_u32(bars + 2 * S), tempty0 = umma::smem_u32(bars + 2 * S + 2);
     // box b of stage s
     auto box = [&](int st, int b) { return umma::smem_u32(smem + (size_t)st * Geo::STAGE + (size_t)b * kSigBox); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = umma::cluster_ctarank();    // 0: issues the MMAs
+    const int unit = (int)blockIdx.x >> 1;
+    int tile = unit, range = 0, slot = -1;            // slot: the partial's place, -1 for a whole tile
+    if (unit >= w.whole) {
+        slot = unit - w.whole;
+        tile = w.whole + slot / w.parts;
+        range = slot % w.parts;
+    }
     int I, J;
-    tile_of(blockIdx.x, nb, I, J);
-    const int m0 = I * kSigTile, n0 = J * kSigTile;
+    tile_of(tile, nb, I, J);
+    const int m0 = I * kSigTile + (int)rank * kSigHalf;    // this CTA's rows of the tile and of panel I
+    const int b0 = J * kSigTile + (int)rank * kSigHalf;    // its rows of panel J
     const int steps = (K + kBK - 1) / kBK;
-    const int nchunks = (steps + Geo::CHUNK - 1) / Geo::CHUNK;
+    const int all = (steps + Geo::CHUNK - 1) / Geo::CHUNK;
+    // chunks [c0, c1) of this unit
+    const int c0 = slot < 0 ? 0 : (int)((int64_t)all * range / w.parts);
+    const int c1 = slot < 0 ? all : (int)((int64_t)all * (range + 1) / w.parts);
+    const int k0 = c0 * Geo::CHUNK, k1 = min(steps, c1 * Geo::CHUNK);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
@@ -120,62 +167,61 @@ sigma_gemm_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant
             umma::mbar_init(empty0 + 8 * s, 1);
         }
         for (int b = 0; b < 2; ++b) {
-            umma::mbar_init(accf0 + 8 * b, 1);     // tcgen05.commit of a chunk
-            umma::mbar_init(acce0 + 8 * b, 128);   // the four epilogue warps drained it
+            umma::mbar_init(tfull0 + 8 * b, 1);                  // tcgen05.commit of a chunk
+            umma::mbar_init(tempty0 + 8 * b, 2 * kSigEpiWarps);  // both CTAs' epilogue warps drained it
         }
         umma::mbar_fence_init();
     }
     if (warp == 1) {
-        umma::tmem_alloc(umma::smem_u32(tmem_slot), 2 * kSigTile);
-        umma::tmem_relinquish();
+        umma::tmem_alloc_pair(umma::smem_u32(tmem_slot), COLS);
+        umma::tmem_relinquish_pair();
     }
     umma::fence_before_sync();
-    __syncthreads();
+    cooperative_groups::this_cluster().sync();        // both CTAs' barriers exist
     umma::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    const uint32_t full_r0 = umma::mapa_rank(full0, 0);
 
     if (warp == 0) {
         if (lane == 0) {
             umma::prefetch_tensormap(&tmH);
             if (NSEG > 1) umma::prefetch_tensormap(&tmD);
-            for (int g = 0; g < steps; ++g) {
-                const int s = g % S;
-                const uint32_t ph = (uint32_t)(g / S) & 1u;
-                if (!umma::mbar_wait(empty0 + 8 * s, ph ^ 1u, kWaitNs)) {
+            for (int g = k0; g < k1; ++g) {
+                const int j = g - k0, s = j % S;
+                if (!umma::mbar_wait(empty0 + 8 * s, ((uint32_t)(j / S) & 1u) ^ 1u, kWaitNs)) {
                     atomicExch(&g_gemm_err, 1);
                     break;
                 }
-                const uint32_t fb = full0 + 8 * s;
-                umma::mbar_arrive_expect_tx(fb, Geo::STAGE);
+                const uint32_t fb = full_r0 + 8u * (uint32_t)s;
+                if (rank == 0) umma::mbar_arrive_expect_tx(full0 + 8 * s, 2 * Geo::STAGE);
                 if (NSEG == 3) {                       // H_I, D_I, H_J, D_J
-                    umma::tma_load_2d(box(s, 0), &tmH, g * kBK, m0, fb);
-                    umma::tma_load_2d(box(s, 1), &tmD, g * kBK, m0, fb);
-                    umma::tma_load_2d(box(s, 2), &tmH, g * kBK, n0, fb);
-                    umma::tma_load_2d(box(s, 3), &tmD, g * kBK, n0, fb);
+                    umma::tma_load_2d_pair(box(s, 0), &tmH, g * kBK, m0, fb);
+                    umma::tma_load_2d_pair(box(s, 1), &tmD, g * kBK, m0, fb);
+                    umma::tma_load_2d_pair(box(s, 2), &tmH, g * kBK, b0, fb);
+                    umma::tma_load_2d_pair(box(s, 3), &tmD, g * kBK, b0, fb);
                 } else {                               // A_I, A_J
-                    umma::tma_load_2d(box(s, 0), &tmH, g * kBK, m0, fb);
-                    umma::tma_load_2d(box(s, 1), &tmH, g * kBK, n0, fb);
+                    umma::tma_load_2d_pair(box(s, 0), &tmH, g * kBK, m0, fb);
+                    umma::tma_load_2d_pair(box(s, 1), &tmH, g * kBK, b0, fb);
                 }
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma::idesc_bf16_f32(kBM, kSigTile);
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc = umma::idesc_bf16_f32(kSigTile, kSigTile);
             bool ok = true;
-            for (int c = 0; c < nchunks && ok; ++c) {
-                const int b = c & 1;
-                if (c >= 2 && !umma::mbar_wait(acce0 + 8 * b, (uint32_t)((c >> 1) - 1) & 1u, 4 * kWaitNs)) {
+            for (int c = c0; c < c1 && ok; ++c) {
+                const int i = c - c0, b = i & 1;
+                if (i >= 2 && !umma::mbar_wait(tempty0 + 8 * b, (uint32_t)((i >> 1) - 1) & 1u, 2 * kWaitNs)) {
                     atomicExch(&g_gemm_err, 4);
                     break;
                 }
                 umma::fence_after_sync();
                 const uint32_t acc = tmem + (uint32_t)(b * kSigTile);
-                const int g0 = c * Geo::CHUNK, g1 = min(steps, g0 + Geo::CHUNK);
+                const int g0 = c * Geo::CHUNK, g1 = min(k1, g0 + Geo::CHUNK);
                 for (int g = g0; g < g1; ++g) {
-                    const int s = g % S;
-                    const uint32_t ph = (uint32_t)(g / S) & 1u;
-                    if (!umma::mbar_wait(full0 + 8 * s, ph, kWaitNs)) {
+                    const int j = g - k0, s = j % S;
+                    if (!umma::mbar_wait(full0 + 8 * s, (uint32_t)(j / S) & 1u, kWaitNs)) {
                         atomicExch(&g_gemm_err, 2);
                         ok = false;
                         break;
@@ -187,79 +233,119 @@ sigma_gemm_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant
                         const uint64_t hj = umma::desc_kmajor_sw128(box(s, 2)), dj = umma::desc_kmajor_sw128(box(s, 3));
 #pragma unroll
                         for (int k = 0; k < kBK / 16; ++k) {
-                            umma::mma_bf16(acc, hi + 2 * k, hj + 2 * k, idesc, (g != g0 || k != 0) ? 1u : 0u);
-                            umma::mma_bf16(acc, hi + 2 * k, dj + 2 * k, idesc, 1u);
-                            umma::mma_bf16(acc, di + 2 * k, hj + 2 * k, idesc, 1u);
+                            umma::mma_bf16_pair(acc, hi + 2 * k, hj + 2 * k, idesc, (g != g0 || k != 0) ? 1u : 0u);
+                            umma::mma_bf16_pair(acc, hi + 2 * k, dj + 2 * k, idesc, 1u);
+                            umma::mma_bf16_pair(acc, di + 2 * k, hj + 2 * k, idesc, 1u);
                         }
                     } else {
                         const uint64_t da = umma::desc_kmajor_sw128(box(s, 0)), db = umma::desc_kmajor_sw128(box(s, 1));
 #pragma unroll
                         for (int k = 0; k < kBK / 16; ++k)
-                            umma::mma_bf16(acc, da + 2 * k, db + 2 * k, idesc, (g != g0 || k != 0) ? 1u : 0u);
+                            umma::mma_bf16_pair(acc, da + 2 * k, db + 2 * k, idesc, (g != g0 || k != 0) ? 1u : 0u);
                     }
-                    umma::mma_commit(empty0 + 8 * s);
+                    umma::mma_commit_pair(empty0 + 8 * s, (uint16_t)3);
                 }
-                if (ok) umma::mma_commit(accf0 + 8 * b);
+                if (ok) umma::mma_commit_pair(tfull0 + 8 * b, (uint16_t)3);
             }
         }
         __syncwarp();
     } else {
-        const int lane_base = (warp & 3) * 32;
-        const int row = m0 + lane_base + lane;
-        const uint32_t tl = tmem + ((uint32_t)lane_base << 16);
-        float acc[kSigTile];
+        const int q = warp & 3, grp = (warp - 2) >> 2;       // tile rows 32 q .., columns 128 grp ..
+        const int row = m0 + 32 * q + lane, cb = J * kSigTile + grp * 128;
+        const uint32_t tempty_r0 = umma::mapa_rank(tempty0, 0);
+        float acc[128];
 #pragma unroll
-        for (int j = 0; j < kSigTile; ++j) acc[j] = 0.f;
+        for (int j = 0; j < 128; ++j) acc[j] = 0.f;
         bool ok = true;
-        for (int c = 0; c < nchunks; ++c) {
-            const int b = c & 1;
-            if (!umma::mbar_wait(accf0 + 8 * b, (uint32_t)(c >> 1) & 1u, 4 * kWaitNs)) {
+        for (int c = c0; c < c1; ++c) {
+            const int i = c - c0, b = i & 1;
+            if (!umma::mbar_wait(tfull0 + 8 * b, (uint32_t)(i >> 1) & 1u, 4 * kWaitNs)) {
                 ok = false;
                 break;
             }
             umma::fence_after_sync();
+            const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * kSigTile + grp * 128);
 #pragma unroll
-            for (int q = 0; q < kSigTile / 32; ++q) {
+            for (int p = 0; p < 4; ++p) {
                 uint32_t r[32];
-                umma::tmem_ld_32x32b_x32(tl + (uint32_t)(b * kSigTile + q * 32), r);
+                umma::tmem_ld_32x32b_x32(ta + (uint32_t)(p * 32), r);
                 umma::tmem_ld_wait();
 #pragma unroll
-                for (int j = 0; j < 32; ++j) acc[q * 32 + j] += __uint_as_float(r[j]);
+                for (int j = 0; j < 32; ++j) acc[p * 32 + j] += __uint_as_float(r[j]);
             }
             umma::fence_before_sync();
-            mbar_arrive(acce0 + 8 * b);
+            __syncwarp();
+            if (lane == 0) umma::mbar_arrive_cluster(tempty_r0 + 8u * (uint32_t)b);
         }
-        if (ok) {
+        if (!ok) {
+            if (lane == 0) atomicExch(&g_gemm_err, 3);
+        } else if (slot >= 0) {                              // a K-range's partial, added by sigma_join_kernel
+            float *dst = part + ((int64_t)slot * kSigTile + (int)rank * kSigHalf + 32 * q + lane) * kSigTile + grp * 128;
+#pragma unroll
+            for (int j = 0; j < 128; j += 4)
+                *reinterpret_cast<float4 *>(dst + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+        } else {
             const bool diag = I == J;
             const float sr = (rs != nullptr && row < n) ? rs[row] : 1.f;
             if (rs != nullptr) {
 #pragma unroll
-                for (int j = 0; j < kSigTile; ++j) acc[j] *= sr * (n0 + j < n ? __ldg(rs + n0 + j) : 0.f);
+                for (int j = 0; j < 128; ++j) acc[j] *= sr * (cb + j < n ? __ldg(rs + cb + j) : 0.f);
             }
             if (row < n) {
                 float *srow = Sig + (int64_t)row * ldS;
-                if (!diag && n0 + kSigTile <= n) {
+                if (!diag && cb + 128 <= n) {
 #pragma unroll
-                    for (int j = 0; j < kSigTile; j += 4)
-                        *reinterpret_cast<float4 *>(srow + n0 + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+                    for (int j = 0; j < 128; j += 4)
+                        *reinterpret_cast<float4 *>(srow + cb + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
                 } else {
 #pragma unroll
-                    for (int j = 0; j < kSigTile; ++j)
-                        if (n0 + j < n && (!diag || n0 + j >= row)) srow[n0 + j] = acc[j];
+                    for (int j = 0; j < 128; ++j)
+                        if (cb + j < n && (!diag || cb + j >= row)) srow[cb + j] = acc[j];
                 }
             }
             // mirror: for fixed j the 32 lanes write 32 consecutive floats
 #pragma unroll
-            for (int j = 0; j < kSigTile; ++j)
-                if (row < n && n0 + j < n && (!diag || n0 + j > row)) Sig[(int64_t)(n0 + j) * ldS + row] = acc[j];
-        } else if (lane == 0) {
-            atomicExch(&g_gemm_err, 3);
+            for (int j = 0; j < 128; ++j)
+                if (row < n && cb + j < n && (!diag || cb + j > row)) Sig[(int64_t)(cb + j) * ldS + row] = acc[j];
         }
     }
     umma::fence_before_sync();
-    __syncthreads();
+    cooperative_groups::this_cluster().sync();        // the peer no longer reads or signals this CTA
     umma::fence_after_sync();
-    if (warp == 1) umma::tmem_dealloc(tmem, 2 * kSigTile);
+    if (warp == 1) umma::tmem_dealloc_pair(tmem, COLS);
+}
+
+// The cut tiles: partials added in range order, scaled, written with their
+// mirror.  One block of 32 x 8 threads per 32 x 32 piece of a tile.
+__global__ void __launch_bounds__(256)
+sigma_join_kernel(const float *__restrict__ part, SigSplit w, int nb, int n, const float *__restrict__ rs,
+                  float *__restrict__ Sig, int64_t ldS) {
+    __shared__ float t[32][33];
+    int I, J;
+    tile_of(w.whole + (int)blockIdx.y, nb, I, J);
+    const int pr = (int)blockIdx.x / (kSigTile / 32) * 32, pc = (int)blockIdx.x % (kSigTile / 32) * 32;
+    const int r0 = I * kSigTile + pr, c0 = J * kSigTile + pc;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    if (r0 >= n || c0 >= n || (I == J && pc < pr)) return;   // uniform: nothing on or above the diagonal here
+    const float *src = part + ((int64_t)blockIdx.y * w.parts * kSigTile + pr) * kSigTile + pc + tx;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = ty + 8 * k;
+        float s = 0.f;
+#pragma unroll 4
+        for (int p = 0; p < w.parts; ++p) s += __ldcg(src + ((int64_t)p * kSigTile + r) * kSigTile);
+        const int row = r0 + r, col = c0 + tx;
+        if (rs != nullptr && row < n && col < n) s *= rs[row] * rs[col];
+        t[r][tx] = s;
+        if (row < n && col < n && col >= row) Sig[(int64_t)row * ldS + col] = s;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int c = ty + 8 * k;
+        const int row = r0 + tx, col = c0 + c;
+        if (row < n && col < n && col > row) Sig[(int64_t)col * ldS + row] = t[tx][c];
+    }
 }
 
 // H = bf16(L), D = bf16(L - H), row by row (4 columns per thread step).
@@ -323,8 +409,13 @@ static size_t sigma_ws_bytes(const mv_problem *P) {
     const size_t plane = align_up((size_t)P->n * (size_t)sigma_ldo(P->T) * 2, 256);
     if (P->dtype == MV_F32) return 2 * plane;
     if (P->dtype == MV_FP8_E4M3) return plane;
-    return 256;
+    return 0;
 }
+// Partials of cut tiles: fewer than `pairs` units of one tile each.  Room for
+// them is optional (without it no tile is cut); the SM count of the part,
+// so that the size does not depend on the current device.
+constexpr int kSigPairs = 152 / 2;
+constexpr size_t kSigPartBytes = (size_t)kSigPairs * kSigTile * kSigTile * 4;
 
 }  // namespace mv
 
@@ -334,7 +425,7 @@ extern "C" {
 
 size_t mv_sigma_workspace_size(const mv_problem *P) {
     if (sigma_check(P) != MV_OK) return 0;
-    return sigma_ws_bytes(P);
+    return sigma_ws_bytes(P) + kSigPartBytes;
 }
 
 int mv_sigma_form(const mv_problem *P, float *d_Sigma, int64_t ldS, void *d_ws, size_t ws_bytes, mv_stream_t stream) {
@@ -347,6 +438,12 @@ int mv_sigma_form(const mv_problem *P, float *d_Sigma, int64_t ldS, void *d_ws, 
     cudaStream_t s = (cudaStream_t)stream;
     const int n = (int)P->n, T = (int)P->T;
     const int nb = (n + kSigTile - 1) / kSigTile;
+    const int64_t tiles = (int64_t)nb * (nb + 1) / 2;
+    const int chunk = P->dtype == MV_F32 ? SigGeo<3>::CHUNK : SigGeo<1>::CHUNK;
+    const int chunks = ((T + kBK - 1) / kBK + chunk - 1) / chunk;
+    const bool room = d_ws != nullptr && ((uintptr_t)d_ws) % 256 == 0 && ws_bytes >= need + kSigPartBytes;
+    const SigSplit w = sigma_split(tiles, room ? std::min(sm_count() / 2, kSigPairs) : 1, chunks);
+    float *part = reinterpret_cast<float *>(reinterpret_cast<char *>(d_ws) + need);
     const int64_t ldo = sigma_ldo(T);
     const size_t plane = align_up((size_t)n * (size_t)ldo * 2, 256);
     CUtensorMap tmH, tmD;
@@ -354,39 +451,53 @@ int mv_sigma_form(const mv_problem *P, float *d_Sigma, int64_t ldS, void *d_ws, 
     const float *rs = nullptr;
     dim3 cgrid((unsigned)std::min<int64_t>((T / 4 + 255) / 256 + 1, 8), (unsigned)std::min(n, 4096));
     if (P->dtype == MV_BF16) {
-        MV_TRY(make_map_bf16(&tmH, P->L, n, T, P->ld, kSigTile));
+        MV_TRY(make_map_bf16(&tmH, P->L, n, T, P->ld, kSigHalf));
         tmD = tmH;
     } else if (P->dtype == MV_FP8_E4M3) {
         __nv_bfloat16 *B = reinterpret_cast<__nv_bfloat16 *>(d_ws);
         expand_fp8_kernel<<<cgrid, 256, 0, s>>>(reinterpret_cast<const uint8_t *>(P->L), P->ld, n, T, B, ldo);
-        MV_TRY(make_map_bf16(&tmH, B, n, T, ldo, kSigTile));
+        MV_TRY(make_map_bf16(&tmH, B, n, T, ldo, kSigHalf));
         tmD = tmH;
         rs = P->row_scale;
     } else {
         __nv_bfloat16 *H = reinterpret_cast<__nv_bfloat16 *>(d_ws);
         __nv_bfloat16 *D = reinterpret_cast<__nv_bfloat16 *>(reinterpret_cast<char *>(d_ws) + plane);
         split_hi_lo_kernel<<<cgrid, 256, 0, s>>>(reinterpret_cast<const float *>(P->L), P->ld, n, T, H, D, ldo);
-        MV_TRY(make_map_bf16(&tmH, H, n, T, ldo, kSigTile));
-        MV_TRY(make_map_bf16(&tmD, D, n, T, ldo, kSigTile));
+        MV_TRY(make_map_bf16(&tmH, H, n, T, ldo, kSigHalf));
+        MV_TRY(make_map_bf16(&tmD, D, n, T, ldo, kSigHalf));
         nseg = 3;
     }
     MV_CUDA_TRY(cudaGetLastError());
     static int attrs = -1;
     if (attrs < 0)
-        attrs = (cudaFuncSetAttribute(sigma_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        attrs = (cudaFuncSetAttribute(sigma_pair_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)kSigSmem) == cudaSuccess &&
-                 cudaFuncSetAttribute(sigma_gemm_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                 cudaFuncSetAttribute(sigma_pair_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)kSigSmem) == cudaSuccess)
                     ? MV_OK
                     : MV_ERR_CUDA;
     if (attrs != MV_OK) return record_message(MV_ERR_CUDA, "sigma GEMM: shared-memory attribute refused");
     int zero = 0;
     MV_CUDA_TRY(cudaMemcpyToSymbolAsync(g_gemm_err, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s));
-    const unsigned tiles = (unsigned)((int64_t)nb * (nb + 1) / 2);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * (unsigned)(w.whole + w.cut * w.parts));
+    cfg.blockDim = dim3(kSigThreads);
+    cfg.dynamicSmemBytes = kSigSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     if (nseg == 3)
-        sigma_gemm_kernel<3><<<tiles, kGemmThreads, kSigSmem, s>>>(tmH, tmD, n, T, nb, rs, d_Sigma, ldS);
+        MV_CUDA_TRY(cudaLaunchKernelEx(&cfg, sigma_pair_kernel<3>, tmH, tmD, n, T, nb, w, rs, d_Sigma, ldS, part));
     else
-        sigma_gemm_kernel<1><<<tiles, kGemmThreads, kSigSmem, s>>>(tmH, tmD, n, T, nb, rs, d_Sigma, ldS);
+        MV_CUDA_TRY(cudaLaunchKernelEx(&cfg, sigma_pair_kernel<1>, tmH, tmD, n, T, nb, w, rs, d_Sigma, ldS, part));
+    if (w.cut > 0)
+        sigma_join_kernel<<<dim3((kSigTile / 32) * (kSigTile / 32), (unsigned)w.cut), 256, 0, s>>>(part, w, nb, n, rs, d_Sigma,
+                                                                                                  ldS);
     MV_CUDA_TRY(cudaGetLastError());
     int err = 0;
     MV_CUDA_TRY(cudaMemcpyFromSymbolAsync(&err, g_gemm_err, sizeof(int), 0, cudaMemcpyDeviceToHost, s));
