@@ -7,11 +7,13 @@
 // sort), and every output is summed over its list in that order.
 //
 //  * MV_LAYOUT_TN (L^T stored T x n): a CTA takes 8 buckets and a chunk of
-//    256 x VEC assets; each thread adds, for each bucket, the signed 16-byte
-//    slices of the rows t of L^T in the bucket (a warp reads 512 contiguous
-//    bytes of a row), parks the 8 results in shared memory and writes them
-//    out as 8 consecutive floats of tilde L's row (n x m, row-major).
-//    Every row of L^T is read once in total: HBM-bound.
+//    256 x VEC assets.  The buckets' lists are one contiguous run, which the
+//    CTA fetches first and each thread then walks from end to end, kCsLoads
+//    signed 16-byte slices of rows of L^T in flight (a warp reads 512
+//    contiguous bytes of a row) whatever the bucket boundaries; each finished
+//    bucket parks its sum in shared memory, and the 8 results go out as 8
+//    consecutive floats of tilde L's row (n x m, row-major).  Every row of L^T
+//    is read once in total: HBM-bound.
 //  * MV_LAYOUT_NT (L stored n x T): a CTA stages one asset row of L in
 //    shared memory (T e bytes, at most 200 KB) and its threads gather the
 //    buckets from it.
@@ -19,12 +21,14 @@
 #include <algorithm>
 
 #include "mv_internal.cuh"
+#include "umma.cuh"
 
 namespace mv {
 
-constexpr int kCsThreads = 256;
+constexpr int kCsThreads = 256, kCsThreadsFew = 64;   // TN: per CTA, and where that leaves SMs idle
 constexpr int kCsGroup = 8;                   // buckets per CTA (TN)
-constexpr int kCsLoads = 4;                   // row slices in flight per thread (TN)
+constexpr int kCsLoads = 8;                   // row slices in flight per thread (TN)
+constexpr int kCsCacheMax = 2048;             // list entries a CTA keeps in shared memory, at most (TN)
 constexpr int kCsNtThreads = 512;
 constexpr size_t kCsNtMaxRow = 200 * 1024;    // staged row bytes (NT)
 constexpr int kCsMaxBucket = 4096;            // periods per bucket the in-place sort accepts
@@ -38,6 +42,9 @@ static size_t cs_ws_bytes(int64_t T, int64_t m) {
     return align_up(4 * (size_t)m, 256) * 2 + align_up(4 * ((size_t)m + 1), 256) + align_up(4 * (size_t)T, 256) + 256;
 }
 
+// Counters and the error word first: one memset clears them.
+static size_t cs_zero_bytes(int64_t m) { return 2 * align_up(4 * (size_t)m, 256) + 256; }
+
 static CsWs cs_carve(void *ws, int64_t T, int64_t m) {
     CsWs w;
     char *p = reinterpret_cast<char *>(ws);
@@ -45,15 +52,37 @@ static CsWs cs_carve(void *ws, int64_t T, int64_t m) {
     p += align_up(4 * (size_t)m, 256);
     w.fill = reinterpret_cast<int *>(p);
     p += align_up(4 * (size_t)m, 256);
+    w.err = reinterpret_cast<int *>(p);
+    p += 256;
     w.off = reinterpret_cast<int *>(p);
     p += align_up(4 * ((size_t)m + 1), 256);
     w.list = reinterpret_cast<unsigned *>(p);
-    p += align_up(4 * (size_t)T, 256);
-    w.err = reinterpret_cast<int *>(p);
     return w;
 }
 
+// The five kernels run as a chain of programmatic dependent launches: each
+// starts while the one before drains, waits for it, then lets the next start.
+__device__ __forceinline__ void cs_chain() {
+    umma::grid_dependency_wait();
+    umma::launch_dependents();
+}
+template <typename... Params, typename... Args>
+static cudaError_t cs_start(void (*kern)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
+
 __global__ void cs_count_kernel(const int *__restrict__ h, int T, int m, int *__restrict__ cnt, int *__restrict__ err) {
+    cs_chain();
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < T; t += gridDim.x * blockDim.x) {
         const int b = h[t];
         if (b < 0 || b >= m) {
@@ -67,6 +96,7 @@ __global__ void cs_count_kernel(const int *__restrict__ h, int T, int m, int *__
 // Exclusive scan of m counts by one block of 1024 threads (chunked).
 __global__ void __launch_bounds__(1024) cs_scan_kernel(const int *__restrict__ cnt, int m, int *__restrict__ off) {
     __shared__ int part[1024];
+    cs_chain();
     const int per = (m + 1023) / 1024;
     const int b0 = threadIdx.x * per, b1 = min(m, b0 + per);
     int s = 0;
@@ -89,6 +119,7 @@ __global__ void __launch_bounds__(1024) cs_scan_kernel(const int *__restrict__ c
 
 __global__ void cs_fill_kernel(const int *__restrict__ h, const int8_t *__restrict__ sign, int T, int m,
                                const int *__restrict__ off, int *__restrict__ fill, unsigned *__restrict__ list) {
+    cs_chain();
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < T; t += gridDim.x * blockDim.x) {
         const int b = h[t];
         if (b < 0 || b >= m) continue;
@@ -97,11 +128,15 @@ __global__ void cs_fill_kernel(const int *__restrict__ h, const int8_t *__restri
     }
 }
 
+constexpr int kCsRankMax = 1024;              // periods per bucket a warp sorts by rank
+constexpr int kCsSortThreads = 128;
+
 __device__ __forceinline__ unsigned cs_key(unsigned e) { return e & 0x7fffffffu; }
 
 // Ascending periods within one bucket of nb entries at list[p0..): up to 16
 // in registers through a fixed 16-input odd-even transposition network (a
-// uniform hash leaves a few periods per bucket), more by insertion in place.
+// uniform hash leaves a few periods per bucket), above kCsRankMax by
+// insertion in place.
 __device__ __forceinline__ void cs_sort_bucket(unsigned *__restrict__ list, int p0, int nb) {
     if (nb <= 16) {
         unsigned v[16];
@@ -133,75 +168,108 @@ __device__ __forceinline__ void cs_sort_bucket(unsigned *__restrict__ list, int 
     }
 }
 
-// Sort every bucket (a bucket above kCsMaxBucket periods is refused).
-__global__ void cs_sort_kernel(const int *__restrict__ off, int m, unsigned *__restrict__ list, int *__restrict__ err) {
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < m; b += gridDim.x * blockDim.x) {
-        const int p0 = off[b], nb = off[b + 1] - p0;
-        if (nb > kCsMaxBucket) {
+// Sort every bucket (a bucket above kCsMaxBucket periods is refused): a
+// thread per bucket, but 17 to kCsRankMax periods by the whole warp, each lane
+// placing its entries by counting the smaller keys (periods are distinct).
+// One thread inserting in global memory took most of the call where buckets
+// are long (89 periods: 0.4 of 0.65 ms at 1498 x 47924 to 540 columns).
+__global__ void __launch_bounds__(kCsSortThreads)
+cs_sort_kernel(const int *__restrict__ off, int m, unsigned *__restrict__ list, int *__restrict__ err) {
+    __shared__ unsigned buf[kCsSortThreads / kWarp][kCsRankMax];
+    cs_chain();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int total = (m + kWarp - 1) / kWarp * kWarp;         // whole warps take part in the ballots
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < total; b += gridDim.x * blockDim.x) {
+        const int p0 = b < m ? off[b] : 0, nb = b < m ? off[b + 1] - p0 : 0;
+        const bool by_rank = nb > 16 && nb <= kCsRankMax;
+        if (nb > kCsMaxBucket)
             atomicExch(err, 2);
-            continue;
+        else if (!by_rank)
+            cs_sort_bucket(list, p0, nb);
+        for (unsigned todo = __ballot_sync(0xffffffffu, by_rank); todo != 0; todo &= todo - 1) {
+            const int src = __ffs((int)todo) - 1;
+            const int q0 = __shfl_sync(0xffffffffu, p0, src), nq = __shfl_sync(0xffffffffu, nb, src);
+            for (int i = lane; i < nq; i += kWarp) buf[warp][i] = list[q0 + i];
+            __syncwarp();
+            for (int i = lane; i < nq; i += kWarp) {
+                const unsigned x = buf[warp][i];
+                int rank = 0;
+#pragma unroll 8
+                for (int k = 0; k < nq; ++k) rank += cs_key(buf[warp][k]) < cs_key(x) ? 1 : 0;
+                list[q0 + rank] = x;
+            }
+            __syncwarp();
         }
-        cs_sort_bucket(list, p0, nb);
     }
 }
 
-template <int DT>
-__global__ void __launch_bounds__(kCsThreads)
+template <int DT, int NT>
+__global__ void __launch_bounds__(NT)
 cs_tn_kernel(const void *__restrict__ Lt, int64_t ld, int n, int m, const int *__restrict__ off,
-             const unsigned *__restrict__ list, const float *__restrict__ rs, float *__restrict__ out, int64_t ldS) {
+             const unsigned *__restrict__ list, const float *__restrict__ rs, float *__restrict__ out, int64_t ldS,
+             int ncache) {
     using St = Store<DT>;
     constexpr int VEC = St::VEC;
-    constexpr int CHUNK = kCsThreads * VEC;
+    constexpr int CHUNK = NT * VEC;
     extern __shared__ __align__(16) float tile[];                 // [kCsGroup][CHUNK]
     const int j0 = blockIdx.x * kCsGroup;
     const int a0 = blockIdx.y * CHUNK;
     const int my = a0 + threadIdx.x * VEC;
     const char *base = reinterpret_cast<const char *>(Lt);
-    // the 9 bucket boundaries of the group, loaded together up front
-    int bnd[kCsGroup + 1];
+    cs_chain();
+    // the group's 9 bucket boundaries and its run of the list (what exceeds the cache is read as it comes)
+    __shared__ int bnd[kCsGroup + 1];
+    unsigned *cache = reinterpret_cast<unsigned *>(tile + kCsGroup * CHUNK);
+    if (threadIdx.x <= kCsGroup) bnd[threadIdx.x] = __ldg(off + min(j0 + (int)threadIdx.x, m));
+    __syncthreads();
+    const int p0 = bnd[0], p1 = bnd[kCsGroup];
+    for (int k = threadIdx.x; k < min(p1 - p0, ncache); k += NT) cache[k] = __ldg(list + p0 + k);
+    __syncthreads();
+    float acc[VEC];
 #pragma unroll
-    for (int g = 0; g <= kCsGroup; ++g) bnd[g] = __ldg(off + min(j0 + g, m));
+    for (int q = 0; q < VEC; ++q) acc[q] = 0.f;
+    int g = 0;
+    auto park = [&] {                              // bucket g is complete
 #pragma unroll
-    for (int g = 0; g < kCsGroup; ++g) {
-        float acc[VEC];
+        for (int q = 0; q < VEC; ++q) {
+            tile[g * CHUNK + threadIdx.x * VEC + q] = acc[q];
+            acc[q] = 0.f;
+        }
+        ++g;
+    };
+    for (int p = p0; p < p1; p += kCsLoads) {
+        unsigned e[kCsLoads];
+        uint4 u[kCsLoads];
 #pragma unroll
-        for (int q = 0; q < VEC; ++q) acc[q] = 0.f;
-        if (my < n) {
-            const int p1 = bnd[g + 1];
-            // kCsLoads list entries, then kCsLoads row slices in flight; the
-            // additions keep the ascending period order
-            for (int p = bnd[g]; p < p1; p += kCsLoads) {
-                unsigned e[kCsLoads];
-                uint4 u[kCsLoads];
-#pragma unroll
-                for (int k = 0; k < kCsLoads; ++k) e[k] = p + k < p1 ? __ldg(list + p + k) : 0u;
-#pragma unroll
-                for (int k = 0; k < kCsLoads; ++k)
-                    u[k] = p + k < p1 ? ld_stream16(base + ((int64_t)(e[k] & 0x7fffffffu) * ld + my) *
-                                                              (int64_t)sizeof(typename St::elem))
-                                      : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                for (int k = 0; k < kCsLoads; ++k) {
-                    if (p + k >= p1) break;
-                    float f[VEC];
-                    St::unpack(u[k], f);
-                    if (e[k] & 0x80000000u) {
-#pragma unroll
-                        for (int q = 0; q < VEC; ++q) acc[q] -= f[q];
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < VEC; ++q) acc[q] += f[q];
-                    }
-                }
-            }
+        for (int k = 0; k < kCsLoads; ++k) {
+            const int at = p + k - p0;
+            e[k] = p + k < p1 ? (at < ncache ? cache[at] : __ldg(list + p + k)) : 0u;
         }
 #pragma unroll
-        for (int q = 0; q < VEC; ++q) tile[g * CHUNK + threadIdx.x * VEC + q] = acc[q];
+        for (int k = 0; k < kCsLoads; ++k)
+            u[k] = my < n && p + k < p1 ? ld_stream16(base + ((int64_t)(e[k] & 0x7fffffffu) * ld + my) *
+                                                                 (int64_t)sizeof(typename St::elem))
+                                        : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int k = 0; k < kCsLoads; ++k) {
+            if (p + k >= p1) break;
+            while (p + k >= bnd[g + 1]) park();     // the same in every thread
+            float f[VEC];
+            St::unpack(u[k], f);
+            if (e[k] & 0x80000000u) {
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) acc[q] -= f[q];
+            } else {
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) acc[q] += f[q];
+            }
+        }
     }
+    while (g < kCsGroup) park();
     __syncthreads();
     // row a of tilde L gets the kCsGroup consecutive buckets j0 ..
     const bool full = j0 + kCsGroup <= m && (ldS & 3) == 0;
-    for (int k = threadIdx.x; k < CHUNK; k += kCsThreads) {
+    for (int k = threadIdx.x; k < CHUNK; k += NT) {
         const int a = a0 + k;
         if (a >= n) break;
         const float s = rs ? rs[a] : 1.f;
@@ -233,6 +301,7 @@ cs_nt_kernel(const void *__restrict__ L, int64_t ld, int T, int m, const int *__
     const char *src = reinterpret_cast<const char *>(L) + (int64_t)i * ld * es;
     for (int64_t o = (int64_t)threadIdx.x * 16; o < bytes; o += (int64_t)kCsNtThreads * 16)
         *reinterpret_cast<uint4 *>(row + o) = ld_stream16(src + o);
+    cs_chain();                                    // the row above does not depend on the lists
     __syncthreads();
     const E *r = reinterpret_cast<const E *>(row);
     const float s = rs ? rs[i] : 1.f;
@@ -264,19 +333,35 @@ static int cs_smem_attr(K k, size_t bytes) {
                : record_message(MV_ERR_CUDA, "countsketch: shared-memory attribute refused");
 }
 
+template <int DT, int NT>
+static int cs_launch_tn(const void *L, int64_t ld, int n, int T, int m, const CsWs &w, const float *rs, float *out, int64_t ldS,
+                        cudaStream_t s) {
+    constexpr int CHUNK = NT * Store<DT>::VEC;
+    // room for twice the average run (it holds nearly every one of a uniform
+    // hash); more would cost a resident CTA where the runs are short
+    const int ncache = (int)std::min<int64_t>(kCsCacheMax, std::max<int64_t>(64, 2 * (int64_t)kCsGroup * T / m));
+    const size_t smem = (size_t)kCsGroup * CHUNK * 4 + 4 * (size_t)ncache;
+    MV_TRY(cs_smem_attr(cs_tn_kernel<DT, NT>, smem));
+    dim3 grid((unsigned)((m + kCsGroup - 1) / kCsGroup), (unsigned)((n + CHUNK - 1) / CHUNK));
+    MV_CUDA_TRY(cs_start(cs_tn_kernel<DT, NT>, grid, NT, smem, s, L, ld, n, m, w.off, w.list, rs, out, ldS,
+                         ncache));
+    return MV_OK;
+}
+
 template <int DT>
 static int cs_launch(int layout, const void *L, int64_t ld, int n, int T, int m, const CsWs &w, const float *rs,
                      float *out, int64_t ldS, cudaStream_t s) {
     if (layout == MV_LAYOUT_TN) {
+        // narrow CTAs where wide ones would not give every SM four
         constexpr int CHUNK = kCsThreads * Store<DT>::VEC;
-        const size_t smem = (size_t)kCsGroup * CHUNK * 4;
-        MV_TRY(cs_smem_attr(cs_tn_kernel<DT>, smem));
-        dim3 grid((unsigned)((m + kCsGroup - 1) / kCsGroup), (unsigned)((n + CHUNK - 1) / CHUNK));
-        cs_tn_kernel<DT><<<grid, kCsThreads, smem, s>>>(L, ld, n, m, w.off, w.list, rs, out, ldS);
+        const int64_t wide = (int64_t)((m + kCsGroup - 1) / kCsGroup) * ((n + CHUNK - 1) / CHUNK);
+        if (wide < 4 * 152) return cs_launch_tn<DT, kCsThreadsFew>(L, ld, n, T, m, w, rs, out, ldS, s);
+        return cs_launch_tn<DT, kCsThreads>(L, ld, n, T, m, w, rs, out, ldS, s);
     } else {
         const size_t smem = ((size_t)T * dtype_size(DT) + 15) / 16 * 16;
         MV_TRY(cs_smem_attr(cs_nt_kernel<DT>, smem));
-        cs_nt_kernel<DT><<<(unsigned)n, kCsNtThreads, smem, s>>>(L, ld, T, m, w.off, w.list, rs, out, ldS);
+        MV_CUDA_TRY(cs_start(cs_nt_kernel<DT>, dim3((unsigned)n), kCsNtThreads, smem, s, L, ld, T, m, w.off, w.list, rs, out,
+                             ldS));
     }
     return MV_OK;
 }
@@ -313,14 +398,13 @@ int mv_countsketch(const void *d_L, int32_t dtype, int32_t layout, const float *
     (void)cudaGetLastError();
     cudaStream_t s = (cudaStream_t)stream;
     CsWs w = cs_carve(d_ws, T, m);
-    MV_CUDA_TRY(cudaMemsetAsync(w.cnt, 0, 4 * (size_t)m, s));
-    MV_CUDA_TRY(cudaMemsetAsync(w.fill, 0, 4 * (size_t)m, s));
-    MV_CUDA_TRY(cudaMemsetAsync(w.err, 0, sizeof(int), s));
+    MV_CUDA_TRY(cudaMemsetAsync(w.cnt, 0, cs_zero_bytes(m), s));
     const int tb = (int)std::min<int64_t>((T + 255) / 256, 4096);
-    cs_count_kernel<<<tb, 256, 0, s>>>(d_hash, (int)T, (int)m, w.cnt, w.err);
-    cs_scan_kernel<<<1, 1024, 0, s>>>(w.cnt, (int)m, w.off);
-    cs_fill_kernel<<<tb, 256, 0, s>>>(d_hash, d_sign, (int)T, (int)m, w.off, w.fill, w.list);
-    cs_sort_kernel<<<(unsigned)std::min<int64_t>((m + 255) / 256, 4096), 256, 0, s>>>(w.off, (int)m, w.list, w.err);
+    const int sb = (int)std::min<int64_t>((m + kCsSortThreads - 1) / kCsSortThreads, 4096);
+    MV_CUDA_TRY(cs_start(cs_count_kernel, dim3(tb), 256, 0, s, d_hash, (int)T, (int)m, w.cnt, w.err));
+    MV_CUDA_TRY(cs_start(cs_scan_kernel, dim3(1), 1024, 0, s, w.cnt, (int)m, w.off));
+    MV_CUDA_TRY(cs_start(cs_fill_kernel, dim3(tb), 256, 0, s, d_hash, d_sign, (int)T, (int)m, w.off, w.fill, w.list));
+    MV_CUDA_TRY(cs_start(cs_sort_kernel, dim3(sb), kCsSortThreads, 0, s, w.off, (int)m, w.list, w.err));
     const float *rs = dtype == MV_FP8_E4M3 ? d_row_scale : nullptr;
     switch (dtype) {
         case MV_F32: MV_TRY(cs_launch<MV_F32>(layout, d_L, ldL, (int)n, (int)T, (int)m, w, rs, d_L_sketch, ldS, s)); break;
