@@ -199,21 +199,55 @@ __global__ void __launch_bounds__(kProjNT) frontier_step_kernel(FArgs a) {
     cluster_barrier<CL>();
 }
 
-// L (n x T, ld ldL) -> L^T (T x n, ld ldT), BF16, 32x32 tiles through shared memory.
-template <typename E>
-__global__ void transpose_elem_kernel(const E *__restrict__ L, int n, int T, int64_t ldL, E *__restrict__ Lt,
-                                      int64_t ldT) {
-    __shared__ E tile[32][33];
-    const int t0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-        const int i = i0 + r, t = t0 + threadIdx.x;
-        tile[r][threadIdx.x] = (i < n && t < T) ? L[(int64_t)i * ldL + t] : E{};
+// L (n x T, ld ldL) -> L^T (T x n, ld ldT), elements of ES bytes (BF16, FP8):
+// square tiles through shared memory, 4 bytes (K elements) per lane both
+// ways, so a warp moves 128 bytes of a row at a time and a thread keeps its
+// 4 K loads in flight.  Both pitches are multiples of 16 bytes, so a word that
+// straddles the last period or asset stays inside its row; what of it does
+// not exist is not stored.  With single elements and 32 x 32 tiles
+// 5440 x 48374 BF16 took 490 us.
+template <int ES>
+__global__ void __launch_bounds__(256)
+transpose_kernel(const uint8_t *__restrict__ L, int n, int T, int64_t ldL, uint8_t *__restrict__ Lt, int64_t ldT) {
+    constexpr int K = 4 / ES, TILE = 32 * K, R = TILE / 8;
+    constexpr uint32_t MASK = ES == 2 ? 0xffffu : 0xffu;
+    __shared__ uint32_t tile[TILE][33];
+    const int t0 = blockIdx.x * TILE, i0 = blockIdx.y * TILE;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int t = t0 + K * lane;
+    uint32_t v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = i0 + warp + 8 * r;
+        v[r] = i < n && t < T ? __ldg(reinterpret_cast<const uint32_t *>(L + ((int64_t)i * ldL + t) * ES)) : 0u;
     }
+#pragma unroll
+    for (int r = 0; r < R; ++r) tile[warp + 8 * r][lane] = v[r];
     __syncthreads();
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-        const int t = t0 + r, i = i0 + threadIdx.x;
-        if (t < T && i < n) Lt[(int64_t)t * ldT + i] = tile[threadIdx.x][r];
+    const int i = i0 + K * lane;
+    if (i >= n) return;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int c = warp + 8 * r;                           // period within the tile
+        if (t0 + c >= T) break;
+        uint32_t w = 0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) w |= ((tile[K * lane + k][c / K] >> (c % K * 8 * ES)) & MASK) << (k * 8 * ES);
+        uint8_t *dst = Lt + ((int64_t)(t0 + c) * ldT + i) * ES;
+        if (i + K <= n) {
+            *reinterpret_cast<uint32_t *>(dst) = w;
+        } else {
+            for (int k = 0; i + k < n; ++k)
+                for (int b = 0; b < ES; ++b) dst[k * ES + b] = (uint8_t)(w >> (8 * (k * ES + b)));
+        }
     }
+}
+template <int ES>
+static void transpose(const void *L, int n, int T, int64_t ldL, void *Lt, int64_t ldT, cudaStream_t s) {
+    constexpr int TILE = 32 * (4 / ES);
+    const dim3 grid((unsigned)((T + TILE - 1) / TILE), (unsigned)((n + TILE - 1) / TILE));
+    transpose_kernel<ES><<<grid, 256, 0, s>>>(reinterpret_cast<const uint8_t *>(L), n, T, ldL,
+                                              reinterpret_cast<uint8_t *>(Lt), ldT);
 }
 
 // The FP32 factor as a BF16 pair: H = bf16(L), D = bf16(L - H), so that
@@ -506,13 +540,10 @@ static int frontier_solve(const mv_problem *P, const mv_problem *P_hi, const dou
 
     // L^T (T x n) once per call: the A operand of Z = L^T Y, and the stored
     // layout in which the power method's fused pass streams fastest.
-    const dim3 tgrid((unsigned)((p.T + 31) / 32), (unsigned)((p.n + 31) / 32));
     if (P->dtype == MV_FP8_E4M3)
-        transpose_elem_kernel<uint8_t><<<tgrid, dim3(32, 8), 0, s>>>(
-            reinterpret_cast<const uint8_t *>(P->L), p.n, p.T, P->ld, at<uint8_t>(d_ws, f.o_lt), f.ldLt);
+        transpose<1>(P->L, p.n, p.T, P->ld, at<void>(d_ws, f.o_lt), f.ldLt, s);
     else
-        transpose_elem_kernel<__nv_bfloat16><<<tgrid, dim3(32, 8), 0, s>>>(
-            reinterpret_cast<const __nv_bfloat16 *>(P->L), p.n, p.T, P->ld, at<__nv_bfloat16>(d_ws, f.o_lt), f.ldLt);
+        transpose<2>(P->L, p.n, p.T, P->ld, at<void>(d_ws, f.o_lt), f.ldLt, s);
     mv_problem Pt = *P;
     Pt.L = at<void>(d_ws, f.o_lt);
     Pt.ld = f.ldLt;
@@ -655,8 +686,8 @@ static int frontier_solve(const mv_problem *P, const mv_problem *P_hi, const dou
         __nv_bfloat16 *H = at<__nv_bfloat16>(d_ws, f.o_h), *D = at<__nv_bfloat16>(d_ws, f.o_d);
         __nv_bfloat16 *Ht = at<__nv_bfloat16>(d_ws, f.o_ht), *Dt = at<__nv_bfloat16>(d_ws, f.o_dt);
         hilo_kernel<<<152 * 8, 256, 0, s>>>(reinterpret_cast<const float *>(P_hi->L), p.n, p.T, P_hi->ld, H, D, f.ldH);
-        transpose_elem_kernel<__nv_bfloat16><<<tgrid, dim3(32, 8), 0, s>>>(H, p.n, p.T, f.ldH, Ht, f.ldLt);
-        transpose_elem_kernel<__nv_bfloat16><<<tgrid, dim3(32, 8), 0, s>>>(D, p.n, p.T, f.ldH, Dt, f.ldLt);
+        transpose<2>(H, p.n, p.T, f.ldH, Ht, f.ldLt, s);
+        transpose<2>(D, p.n, p.T, f.ldH, Dt, f.ldLt, s);
         CUtensorMap m2[6];
         MV_TRY(make_map_bf16(&m2[0], Ht, p.T, p.n, f.ldLt, kBM));
         MV_TRY(make_map_bf16(&m2[4], Dt, p.T, p.n, f.ldLt, kBM));
