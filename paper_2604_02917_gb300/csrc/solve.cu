@@ -577,7 +577,9 @@ __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char 
     cluster_arrive<CL>();
     proj_smem_init(&psm);
     ClusterProj<CL> P{&psm, el};
-    bool real = !(EARLY && a.early == 2);
+    // `done` cannot change while this step waits: every product either waited
+    // for the step before (then it is final) or left because it saw the flag.
+    bool real = !(EARLY && a.early == 2) || *(volatile int *)&st->done != 0;
     bool met = false;                      // the cluster's blocks have all started
     while (true) {
         // The made-up point: v = 2^-10, mu = 1 or 2, target 1.5 by equality; its
@@ -1318,6 +1320,62 @@ static int timing_events(int count, const cudaEvent_t **out) {
     return MV_OK;
 }
 
+// Host copies of the loop state, page-locked so that a copy does not hold the
+// host up, with an event behind each.  Two per solve in flight; returned
+// when the solve ends, and at most kPeeks kept for later solves.
+struct Peek {
+    SolveState *hs = nullptr;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    int dev = 0;
+};
+constexpr size_t kPeeks = 8;
+static std::mutex g_peek_mu;
+static std::vector<Peek> g_peeks;
+static void peek_free(Peek &p) {
+    for (cudaEvent_t e : p.ev)
+        if (e) cudaEventDestroy(e);
+    if (p.hs) cudaFreeHost(p.hs);
+    p = Peek{};
+}
+struct PeekLease {
+    Peek p;
+    bool ok = false;
+    PeekLease() {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return;
+        {
+            std::lock_guard<std::mutex> lock(g_peek_mu);
+            for (size_t i = 0; i < g_peeks.size(); ++i)
+                if (g_peeks[i].dev == dev) {
+                    p = g_peeks[i];
+                    g_peeks.erase(g_peeks.begin() + (long)i);
+                    ok = true;
+                    return;
+                }
+        }
+        p.dev = dev;
+        ok = cudaHostAlloc(reinterpret_cast<void **>(&p.hs), 2 * sizeof(SolveState), cudaHostAllocDefault) == cudaSuccess &&
+             cudaEventCreateWithFlags(&p.ev[0], cudaEventDisableTiming) == cudaSuccess &&
+             cudaEventCreateWithFlags(&p.ev[1], cudaEventDisableTiming) == cudaSuccess;
+        if (!ok) {
+            (void)cudaGetLastError();
+            peek_free(p);
+        }
+    }
+    ~PeekLease() {
+        if (!ok) return;
+        // after an error a copy may still be on its way into p.hs
+        for (cudaEvent_t e : p.ev) (void)cudaEventSynchronize(e);
+        std::lock_guard<std::mutex> lock(g_peek_mu);
+        if (g_peeks.size() < kPeeks)
+            g_peeks.push_back(p);
+        else
+            peek_free(p);
+    }
+    PeekLease(const PeekLease &) = delete;
+    PeekLease &operator=(const PeekLease &) = delete;
+};
+
 static std::mutex g_graph_mu;
 static std::unordered_map<GraphKey, cudaGraphExec_t, GraphKeyHash> g_graphs;
 
@@ -1627,6 +1685,29 @@ int mv_npga_solve(const mv_problem *P, const mv_solve_opts *O_in, double *d_x_in
     SolveState hs{};
     int k_prev = 0, timed = 0;
     double t_t = 0.0, t_n = 0.0, t_s = 0.0;
+    // With graphs the next chunk is launched before the last one's flag is
+    // read: the host's turn-round (about 13 us) runs beside it, and a chunk
+    // behind the end returns kernel by kernel (about 20 us, once).
+    if (exec) {
+        PeekLease peek;
+        if (peek.ok) {
+            auto launch = [&](int64_t c) -> int {
+                MV_CUDA_TRY(cudaGraphLaunch(exec, s));
+                launches += per_iter * chunk;
+                MV_CUDA_TRY(cudaMemcpyAsync(&peek.p.hs[c & 1], st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
+                MV_CUDA_TRY(cudaEventRecord(peek.p.ev[c & 1], s));
+                return MV_OK;
+            };
+            MV_TRY(launch(0));
+            for (int64_t c = 0; c < max_chunks; ++c) {
+                if (c + 1 < max_chunks) MV_TRY(launch(c + 1));
+                MV_CUDA_TRY(cudaEventSynchronize(peek.p.ev[c & 1]));
+                hs = peek.p.hs[c & 1];
+                if (hs.done) break;
+            }
+            max_chunks = 0;                               // the loop below is for the other cases
+        }
+    }
     for (int64_t c = 0; c < max_chunks; ++c) {
         if (exec) {
             MV_CUDA_TRY(cudaGraphLaunch(exec, s));
