@@ -73,6 +73,8 @@ template <int CL>
 __global__ void __launch_bounds__(kProjNT) adj_proj_kernel(AdjArgs a) {
     __shared__ ProjSmem psm;
     __shared__ double dsl[2 * kProjMaxCL * 5];
+    umma::grid_dependency_wait();          // launched beside the end of the kernel before it
+    umma::launch_dependents();
     const int rank = cluster_rank<CL>();
     const int n = a.n, nl = (n + CL - 1) / CL, r0 = min(n, rank * nl), r1 = min(n, r0 + nl);
     const double nu = a.nu_tape[a.j], beta = a.betas[*a.k0 + a.j];
@@ -120,6 +122,8 @@ __global__ void __launch_bounds__(kProjNT) adj_proj_kernel(AdjArgs a) {
 // y_bar = v_bar - alpha (2 L L^T v_bar + 2 gamma v_bar).
 __global__ void adj_finish_kernel(const double *__restrict__ vbar, const double *__restrict__ llv, double alpha,
                                   double gamma, double *__restrict__ ybar, int n) {
+    umma::grid_dependency_wait();          // launched beside the product
+    umma::launch_dependents();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) ybar[i] = vbar[i] - alpha * (2.0 * llv[i] + 2.0 * gamma * vbar[i]);
 }
@@ -138,11 +142,11 @@ static int adj_attrs() {
 
 static cudaError_t launch_adj_proj(int CL, const AdjArgs &a, cudaStream_t s) {
     switch (CL) {
-        case 1: return launch_cluster(adj_proj_kernel<1>, 1, 0, s, a);
-        case 2: return launch_cluster(adj_proj_kernel<2>, 2, 0, s, a);
-        case 4: return launch_cluster(adj_proj_kernel<4>, 4, 0, s, a);
-        case 8: return launch_cluster(adj_proj_kernel<8>, 8, 0, s, a);
-        default: return launch_cluster(adj_proj_kernel<16>, 16, 0, s, a);
+        case 1: return launch_cluster_pdl(adj_proj_kernel<1>, 1, 0, s, true, a);
+        case 2: return launch_cluster_pdl(adj_proj_kernel<2>, 2, 0, s, true, a);
+        case 4: return launch_cluster_pdl(adj_proj_kernel<4>, 4, 0, s, true, a);
+        case 8: return launch_cluster_pdl(adj_proj_kernel<8>, 8, 0, s, true, a);
+        default: return launch_cluster_pdl(adj_proj_kernel<16>, 16, 0, s, true, a);
     }
 }
 
@@ -305,7 +309,40 @@ int mv_npga_backward(const mv_problem *P, const mv_solve_opts *O_in, const doubl
     };
     int launches = 4;
     const int per_it = p.use_llt ? 2 : 3;
+    // recompute a segment forward from its checkpoint, recording y_k, z_k, x_{k+1}, nu_k:
+    // the kernels write them where the reverse sweep reads them (z_k by a copy
+    // where the two-pass product, whose vector stores want alignment, forms it)
+    float *VY = at<float>(ws, b.o_vy), *ZW = at<float>(ws, b.o_zw);
+    double *X1 = at<double>(ws, b.o_x1), *NU = at<double>(ws, b.o_nu);
+    auto recompute = [&](cudaStream_t cs, int len) -> int {
+        MV_CUDA_TRY(cudaMemcpyAsync(VY + (size_t)len * n, y32, 4 * (size_t)n, cudaMemcpyDeviceToDevice, cs));
+        for (int j = 0; j < len; ++j) {
+            const float *y_in = VY + (size_t)(len + j) * n;
+            float *z = ZW + (size_t)j * T;
+            const IterTape tape{y_in, j + 1 < len ? VY + (size_t)(len + j + 1) * n : y32, z, X1 + (size_t)j * n, NU + j};
+            MV_TRY(launch_iteration(p, P, &O, ws, cs, nullptr, &tape));
+            if (!p.use_llt)
+                MV_CUDA_TRY(cudaMemcpyAsync(z, at<float>(ws, p.o_z), 4 * (size_t)T, cudaMemcpyDeviceToDevice, cs));
+        }
+        return MV_OK;
+    };
+    // The forward of the last segment is its recomputation: nothing follows it,
+    // and the tape it records is the first the reverse sweep wants.
+    auto run_recompute = [&](int len) -> int {
+        if (len != C || !O.use_graph) return recompute(s, len);
+        GraphKey kr = graph_key(p, P, &O, -1000000 - C, nullptr);
+        kr.ws = ws;
+        cudaGraphExec_t er = nullptr;
+        MV_TRY(cached_graph(kr, [&](cudaStream_t cs) { return recompute(cs, C); }, &er));
+        MV_CUDA_TRY(cudaGraphLaunch(er, s));
+        return MV_OK;
+    };
     for (int c = 0; c < b.ncp; ++c) {
+        if (c == b.ncp - 1) {
+            MV_TRY(run_recompute(K - c * C));
+            launches += per_it * (K - c * C);
+            break;
+        }
         MV_TRY(save_cp(c));
         const int len = std::min(K, (c + 1) * C) - c * C;
         if (len == C && O.use_graph) {               // a full segment: one cached graph
@@ -341,8 +378,6 @@ int mv_npga_backward(const mv_problem *P, const mv_solve_opts *O_in, const doubl
     // ---- reverse sweep, segment by segment
     double *xbar = at<double>(ws, b.o_xbar), *ybar = at<double>(ws, b.o_ybar), *mubar = at<double>(ws, b.o_mubar);
     double *vbar = at<double>(ws, b.o_vbar);
-    float *VY = at<float>(ws, b.o_vy), *ZW = at<float>(ws, b.o_zw);
-    double *X1 = at<double>(ws, b.o_x1), *NU = at<double>(ws, b.o_nu);
     MV_CUDA_TRY(cudaMemcpyAsync(xbar, d_dloss_dx, 8 * (size_t)n, cudaMemcpyDeviceToDevice, s));
     MV_CUDA_TRY(cudaMemsetAsync(ybar, 0, 8 * (size_t)n, s));
     MV_CUDA_TRY(cudaMemsetAsync(mubar, 0, 8 * (size_t)n, s));
@@ -352,19 +387,6 @@ int mv_npga_backward(const mv_problem *P, const mv_solve_opts *O_in, const doubl
     MV_CUDA_TRY(cudaMemcpyAsync(betas, beta.data(), 8 * (size_t)K, cudaMemcpyHostToDevice, s));
     std::vector<int> k0s(b.ncp);
     for (int seg = 0; seg < b.ncp; ++seg) k0s[seg] = seg * C;
-    // recompute a segment forward from its checkpoint, recording y_k, z_k, x_{k+1}, nu_k
-    auto recompute = [&](cudaStream_t cs, int len) -> int {
-        for (int j = 0; j < len; ++j) {
-            MV_CUDA_TRY(cudaMemcpyAsync(VY + (size_t)(len + j) * n, y32, 4 * (size_t)n, cudaMemcpyDeviceToDevice, cs));
-            MV_TRY(launch_iteration(p, P, &O, ws, cs, nullptr));
-            MV_CUDA_TRY(cudaMemcpyAsync(ZW + (size_t)j * T, at<float>(ws, p.o_z), 4 * (size_t)T,
-                                        cudaMemcpyDeviceToDevice, cs));
-            MV_CUDA_TRY(cudaMemcpyAsync(X1 + (size_t)j * n, at<double>(ws, p.o_x), 8 * (size_t)n,
-                                        cudaMemcpyDeviceToDevice, cs));
-            MV_CUDA_TRY(cudaMemcpyAsync(NU + j, &st->nu, 8, cudaMemcpyDeviceToDevice, cs));
-        }
-        return MV_OK;
-    };
     // backward through the segment (iteration k0 + j, j = len - 1 .. 0)
     auto reverse = [&](cudaStream_t cs, int len) -> int {
         for (int j = len - 1; j >= 0; --j) {
@@ -386,30 +408,32 @@ int mv_npga_backward(const mv_problem *P, const mv_solve_opts *O_in, const doubl
             MV_CUDA_TRY(launch_adj_proj(p.cl, a, cs));
             // w = L^T v_bar (z buffer) and L w
             if (p.use_llt)
-                MV_TRY(launch_llt(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), nullptr, cs, at<float>(ws, p.o_z)));
-            else
+                MV_TRY(launch_llt(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), nullptr, cs, ZW + (size_t)(len + j) * T));
+            else {
                 gemv_pair(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), cs);
-            MV_CUDA_TRY(cudaMemcpyAsync(ZW + (size_t)(len + j) * T, at<float>(ws, p.o_z), 4 * (size_t)T,
-                                        cudaMemcpyDeviceToDevice, cs));
-            adj_finish_kernel<<<(n + 255) / 256, 256, 0, cs>>>(vbar, at<double>(ws, p.o_gy), alpha, P->gamma, ybar, n);
+                MV_CUDA_TRY(cudaMemcpyAsync(ZW + (size_t)(len + j) * T, at<float>(ws, p.o_z), 4 * (size_t)T,
+                                            cudaMemcpyDeviceToDevice, cs));
+            }
+            MV_CUDA_TRY(launch_grid(adj_finish_kernel, dim3((n + 255) / 256), dim3(256), 0, cs, p.use_llt, vbar,
+                                    at<double>(ws, p.o_gy), alpha, P->gamma, ybar, n));
         }
         return cudaGetLastError() == cudaSuccess ? MV_OK : MV_ERR_CUDA;
     };
     for (int seg = b.ncp - 1; seg >= 0; --seg) {
         const int k0 = seg * C, k1 = std::min(K, k0 + C), len = k1 - k0;
-        MV_TRY(load_cp(seg));
         MV_CUDA_TRY(cudaMemcpyAsync(k0d, &k0s[seg], sizeof(int), cudaMemcpyHostToDevice, s));
-        if (len == C && O.use_graph) {                // full segments replay two cached graphs
-            GraphKey kr = graph_key(p, P, &O, -1000000 - C, nullptr), kb = graph_key(p, P, &O, -2000000 - C, nullptr);
-            kr.ws = kb.ws = ws;
+        if (seg < b.ncp - 1) {
+            MV_TRY(load_cp(seg));
+            MV_TRY(run_recompute(len));
+        }
+        if (len == C && O.use_graph) {                // a full segment replays a cached graph
+            GraphKey kb = graph_key(p, P, &O, -2000000 - C, nullptr);
+            kb.ws = ws;
             kb.aux = alpha;                           // adj_finish bakes the step in
-            cudaGraphExec_t er = nullptr, eb = nullptr;
-            MV_TRY(cached_graph(kr, [&](cudaStream_t cs) { return recompute(cs, C); }, &er));
+            cudaGraphExec_t eb = nullptr;
             MV_TRY(cached_graph(kb, [&](cudaStream_t cs) { return reverse(cs, C); }, &eb));
-            MV_CUDA_TRY(cudaGraphLaunch(er, s));
             MV_CUDA_TRY(cudaGraphLaunch(eb, s));
         } else {
-            MV_TRY(recompute(s, len));
             MV_TRY(reverse(s, len));
         }
         launches += len * (per_it + 4);

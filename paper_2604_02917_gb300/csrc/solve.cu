@@ -533,6 +533,7 @@ struct StepArgs {
     double *gyw = nullptr;                 // backtracking: L L^T y (written), L L^T d, candidate x+
     const double *gd = nullptr;
     double *xp = nullptr;
+    double *x_tape = nullptr, *nu_tape = nullptr;   // copies of x_{k+1} and its multiplier (the adjoint)
 };
 
 
@@ -708,6 +709,7 @@ __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char 
             const double yn = xn + beta * (xn - e.x);
             if (real) {
                 a.x[gi] = xn;
+                if (a.x_tape != nullptr) a.x_tape[gi] = xn;
                 a.y[gi] = yn;
                 a.y32[gi] = (float)(yn * (a.row_scale ? (double)a.row_scale[gi] : 1.0));
             }
@@ -723,6 +725,7 @@ __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char 
             st->hint = P.scales();
             st->k = k + 1;
             st->nu = o.nu;
+            if (a.nu_tape != nullptr) *a.nu_tape = o.nu;
             st->tau = o.tau;
             if (o.status != MV_OK) st->proj_fail += 1;
             st->proj_steps += o.steps;
@@ -1176,7 +1179,7 @@ static int step_early(const Plan &p) {
 }
 
 static void launch_step(const Plan &p, const mv_problem *P, const mv_solve_opts *O, void *ws, cudaStream_t s,
-                        bool early = false) {
+                        bool early = false, const IterTape *tape = nullptr) {
     StepArgs a;
     a.st = at<SolveState>(ws, p.o_state);
     a.gy = at<double>(ws, p.o_gy);
@@ -1202,6 +1205,11 @@ static void launch_step(const Plan &p, const mv_problem *P, const mv_solve_opts 
     a.gyw = at<double>(ws, p.o_gy);
     a.gd = at<double>(ws, p.o_gd);
     a.xp = at<double>(ws, p.o_xp);
+    if (tape) {
+        a.y32 = tape->y_out;
+        a.x_tape = tape->x1;
+        a.nu_tape = tape->nu;
+    }
     const size_t sm = step_smem(p.n, p.cl);
     if (O->backtrack) {
         switch (p.cl) {
@@ -1276,9 +1284,9 @@ static int launch_product(const Plan &p, const mv_problem *P, const float *y32, 
 // gemv_n and the step kernel (ev[3] is the next iteration's ev[0]); with the
 // fused pass, ev[0..1] bracket it and ev[1..2] is empty.
 int launch_iteration(const Plan &p, const mv_problem *P, const mv_solve_opts *O, void *ws,
-                            cudaStream_t s, const cudaEvent_t *ev) {
+                            cudaStream_t s, const cudaEvent_t *ev, const IterTape *tape) {
     SolveState *st = at<SolveState>(ws, p.o_state);
-    const float *y32 = at<float>(ws, p.o_y32);
+    const float *y32 = tape ? tape->y_in : at<float>(ws, p.o_y32);
     // the product: L L^T y for the step, L L^T d for a backtracking trial
     double *gy = O->backtrack ? at<double>(ws, p.o_gd) : at<double>(ws, p.o_gy);
     const int *done = &st->done;
@@ -1287,11 +1295,11 @@ int launch_iteration(const Plan &p, const mv_problem *P, const mv_solve_opts *O,
         if (p.sig)
             MV_TRY(launch_symv(p, P, y32, ws, done, gy, nullptr, s));
         else
-            MV_TRY(launch_llt(p, P, y32, ws, done, gy, nullptr, s, p.want_z ? at<float>(ws, p.o_z) : nullptr,
+            MV_TRY(launch_llt(p, P, y32, ws, done, gy, nullptr, s, tape ? tape->z : (p.want_z ? at<float>(ws, p.o_z) : nullptr),
                               kLoopPdl && ev == nullptr));   // timed runs keep launches apart
         if (ev) cudaEventRecord(ev[1], s);
         if (ev) cudaEventRecord(ev[2], s);
-        launch_step(p, P, O, ws, s, kLoopPdl && ev == nullptr);
+        launch_step(p, P, O, ws, s, kLoopPdl && ev == nullptr, tape);
         if (ev) cudaEventRecord(ev[3], s);
         return MV_OK;
     }
@@ -1299,7 +1307,7 @@ int launch_iteration(const Plan &p, const mv_problem *P, const mv_solve_opts *O,
     if (ev) cudaEventRecord(ev[1], s);
     launch_g(p, P, at<float>(ws, p.o_z), ws, done, gy, nullptr, s, kLoopPdl && ev == nullptr);
     if (ev) cudaEventRecord(ev[2], s);
-    launch_step(p, P, O, ws, s, kLoopPdl && ev == nullptr);
+    launch_step(p, P, O, ws, s, kLoopPdl && ev == nullptr, tape);
     if (ev) cudaEventRecord(ev[3], s);
     return MV_OK;
 }

@@ -124,8 +124,16 @@ void gemv_pair(const Plan &p, const mv_problem *P, const float *y32, void *ws, c
 void gemv_t_only(const Plan &p, const mv_problem *P, const float *y32, void *ws, cudaStream_t s);
 void launch_init_x(const Plan &p, const mv_problem *P, const mv_solve_opts *O, const double *x_in, void *ws,
                    cudaStream_t s);
+// Where an iteration that is recorded (the adjoint's tape) reads its product's
+// input and leaves what the reverse sweep needs.  z only with the fused pass.
+struct IterTape {
+    const float *y_in;                     // y_k, FP32
+    float *y_out;                          // y_{k+1}, FP32
+    float *z;                              // L^T y_k
+    double *x1, *nu;                       // x_{k+1} and the return row's multiplier
+};
 int launch_iteration(const Plan &p, const mv_problem *P, const mv_solve_opts *O, void *ws, cudaStream_t s,
-                     const cudaEvent_t *ev);
+                     const cudaEvent_t *ev, const IterTape *tape = nullptr);
 GraphKey graph_key(const Plan &p, const mv_problem *P, const mv_solve_opts *O, int chunk, const void *ev);
 // The cached executable graph of `key`, capturing `enqueue(stream)` into it on first use.
 int cached_graph(const GraphKey &key, const std::function<int(cudaStream_t)> &enqueue, cudaGraphExec_t *out);
