@@ -107,11 +107,16 @@ __device__ __forceinline__ void chunk_store(const float (&acc)[128], int row, in
     }
 }
 
+// With gridDim.z = 2 one launch forms two products of the same shape (plane 1:
+// A1 B1^T into C1), for shapes whose tiles fill a fraction of the SMs.
 template <int BN, int NA>
 __global__ void __launch_bounds__(GemmChunkCfg<BN, NA>::THREADS, 1)
-gemm_chunk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                  const __grid_constant__ CUtensorMap tmA2, float *__restrict__ C, int M, int N, int K, int64_t ldc,
-                  GemmEpi e, int raster) {
+gemm_chunk_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
+                  const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmA1,
+                  const __grid_constant__ CUtensorMap tmB1, float *__restrict__ C0, float *__restrict__ C1, int M, int N,
+                  int K, int64_t ldc, GemmEpi e, int raster) {
+    const CUtensorMap *tmA = blockIdx.z ? &tmA1 : &tmA0, *tmB = blockIdx.z ? &tmB1 : &tmB0;
+    float *C = blockIdx.z ? C1 : C0;
     using Cfg = GemmChunkCfg<BN, NA>;
     constexpr int S = Cfg::S;
     constexpr int CH = kChunkSteps;
@@ -160,8 +165,8 @@ gemm_chunk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
     if (warp == 0) {
         if (lane == 0) {
-            umma::prefetch_tensormap(&tmA);
-            umma::prefetch_tensormap(&tmB);
+            umma::prefetch_tensormap(tmA);
+            umma::prefetch_tensormap(tmB);
             if (NA > 1) umma::prefetch_tensormap(&tmA2);
             for (int kt = 0; kt < nk; ++kt) {
                 const int s = kt % S;
@@ -171,11 +176,11 @@ gemm_chunk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     break;
                 }
                 umma::mbar_arrive_expect_tx(full0 + 8 * s, Cfg::STAGE);
-                umma::tma_load_2d(umma::smem_u32(sA + s * NA * Cfg::A_BYTES), &tmA, kt * kBK, m0, full0 + 8 * s);
+                umma::tma_load_2d(umma::smem_u32(sA + s * NA * Cfg::A_BYTES), tmA, kt * kBK, m0, full0 + 8 * s);
                 if (NA > 1)
                     umma::tma_load_2d(umma::smem_u32(sA + (s * NA + 1) * Cfg::A_BYTES), &tmA2, kt * kBK, m0,
                                       full0 + 8 * s);
-                umma::tma_load_2d(umma::smem_u32(sB + s * Cfg::B_BYTES), &tmB, kt * kBK, n0, full0 + 8 * s);
+                umma::tma_load_2d(umma::smem_u32(sB + s * Cfg::B_BYTES), tmB, kt * kBK, n0, full0 + 8 * s);
             }
         }
         __syncwarp();
@@ -466,11 +471,13 @@ static int gemmc_set_attrs() {
 // Enqueue C = epilogue(A B^T) with prebuilt tensor maps (capturable; K >= 1).
 template <int BN, int NA>
 static void gemmc_launch(const CUtensorMap &ta, const CUtensorMap &tb, const CUtensorMap *ta2, int64_t M, int64_t N,
-                         int64_t K, float *C, int64_t ldc, const GemmEpi &e, cudaStream_t s, int raster = 1) {
+                         int64_t K, float *C, int64_t ldc, const GemmEpi &e, cudaStream_t s, int raster = 1,
+                         const CUtensorMap *ta1 = nullptr, const CUtensorMap *tb1 = nullptr, float *C1 = nullptr) {
     using Cfg = GemmChunkCfg<BN, NA>;
-    dim3 grid((unsigned)((M + kBM - 1) / kBM), (unsigned)((N + BN - 1) / BN));
-    gemm_chunk_kernel<BN, NA><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(ta, tb, ta2 ? *ta2 : ta, C, (int)M, (int)N,
-                                                                    (int)K, ldc, e, raster);
+    dim3 grid((unsigned)((M + kBM - 1) / kBM), (unsigned)((N + BN - 1) / BN), ta1 ? 2 : 1);
+    gemm_chunk_kernel<BN, NA><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(ta, tb, ta2 ? *ta2 : ta, ta1 ? *ta1 : ta,
+                                                                    tb1 ? *tb1 : tb, C, C1, (int)M, (int)N, (int)K, ldc, e,
+                                                                    raster);
 }
 
 template <int NA>
@@ -548,6 +555,22 @@ static int gemmc(const void *A, const void *A2, int64_t M, int64_t lda, const vo
         MV_CUDA_TRY(cudaGetLastError());
         return MV_OK;
     }
+}
+
+// C0 = A0 B0^T and C1 = A1 B1^T (same shapes and pitches) in one launch.
+template <int BN>
+static int gemmc_two(const void *A0, const void *B0, float *C0, const void *A1, const void *B1, float *C1, int64_t M,
+                     int64_t lda, int64_t N, int64_t ldb, int64_t K, int64_t ldc, cudaStream_t s) {
+    static_assert(BN < 256, "the 256-column tiles run on CTA pairs");
+    CUtensorMap ta, tb, ta1, tb1;
+    MV_TRY(make_map_bf16(&ta, A0, M, K, lda, kBM));
+    MV_TRY(make_map_bf16(&tb, B0, N, K, ldb, BN));
+    MV_TRY(make_map_bf16(&ta1, A1, M, K, lda, kBM));
+    MV_TRY(make_map_bf16(&tb1, B1, N, K, ldb, BN));
+    MV_TRY((gemmc_set_attrs<BN, 1>()));
+    gemmc_launch<BN, 1>(ta, tb, nullptr, M, N, K, C0, ldc, GemmEpi{}, s, 1, &ta1, &tb1, C1);
+    MV_CUDA_TRY(cudaGetLastError());
+    return MV_OK;
 }
 
 // The translation unit's GEMM error word: clear before, read after (blocking).

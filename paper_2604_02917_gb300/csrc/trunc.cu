@@ -161,13 +161,39 @@ static __global__ void lowdin_start_kernel(const float *__restrict__ G, int b, i
     }
 }
 
-// T = 1.5 I - 0.5 P.
-static __global__ void ns_t_kernel(const float *__restrict__ P, int b, int64_t ld, float *__restrict__ T) {
-    const int64_t total = (int64_t)b * b;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(idx / b), j = (int)(idx - (int64_t)i * b);
-        T[(int64_t)i * ld + j] = (i == j ? 1.5f : 0.0f) - 0.5f * P[(int64_t)i * ld + j];
+// Operands of a Newton--Schulz product from b x b FP32 matrices X_z (plane z of
+// the grid): the three-piece splits of X_z by rows (side 0) and of X_z^T (side
+// 1), b x 6b BF16 each (b is a multiple of 64).  With STEP the matrix split is
+// T = 1.5 I - 0.5 X_z instead.
+struct NsPieces {
+    const float *X[2];
+    __nv_bfloat16 *rows[2], *cols[2];
+};
+template <bool STEP>
+static __global__ void __launch_bounds__(256) ns_pieces_kernel(NsPieces a, int b, int64_t ld) {
+    __shared__ float tile[32][33];
+    const float *X = a.X[blockIdx.z];
+    __nv_bfloat16 *rows = a.rows[blockIdx.z], *cols = a.cols[blockIdx.z];
+    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t ldo = 6 * (int64_t)b;
+#pragma unroll
+    for (int j = ty; j < 32; j += 8) {
+        const int r = r0 + j, c = c0 + tx;
+        float x = X[(int64_t)r * ld + c];
+        if (STEP) x = (r == c ? 1.5f : 0.0f) - 0.5f * x;
+        tile[j][tx] = x;
+        __nv_bfloat16 *o = rows + (int64_t)r * ldo + c;
+#pragma unroll
+        for (int seg = 0; seg < kSplit3; ++seg) o[(int64_t)seg * b] = split3_get(x, split3_piece(0, seg));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = ty; j < 32; j += 8) {
+        const float x = tile[tx][j];
+        __nv_bfloat16 *o = cols + (int64_t)(c0 + j) * ldo + r0 + tx;
+#pragma unroll
+        for (int seg = 0; seg < kSplit3; ++seg) o[(int64_t)seg * b] = split3_get(x, split3_piece(1, seg));
     }
 }
 
@@ -409,17 +435,17 @@ static int orth(const Ctx &c, const float *Y, float *Q) {
         for (int it = 0; it < its; ++it) {
             // P = Z Ya; T = (3I - P)/2; Yb = Ya T; Z <- T Z.  C = A B^T with A's rows and
             // the right factor's columns (its transposed pieces): no product relies on a
-            // symmetry that rounding only keeps approximately.
-            MV_TRY(split_rows(c, Z, b, b, Wb, Wb, 0, sp0));
-            MV_TRY(split_t(c, Ya, b, b, Wb, Wb, 1, sp1));
+            // symmetry that rounding only keeps approximately.  A product of b = 640
+            // has 25 tiles, so the chain of launches is what counts: one for the
+            // pieces of Z and Ya, one for T's (over those of the first product,
+            // which is done), and the last two products together.  (Six splits,
+            // T and three products of their own took 120 us per step.)
+            const NsPieces in{{Z, Ya}, {sp0, yt0}, {yt1, sp1}};
+            ns_pieces_kernel<false><<<dim3((unsigned)(b / 32), (unsigned)(b / 32), 2), 256, 0, c.s>>>(in, (int)b, Wb);
             MV_TRY(gemm6<128>(c, sp0, b, sp1, b, Wb, P, Wb));
-            ns_t_kernel<<<grid_for(b * b), 256, 0, c.s>>>(P, (int)b, Wb, Tm);
-            MV_TRY(split_rows(c, Ya, b, b, Wb, Wb, 0, sp0));
-            MV_TRY(split_t(c, Tm, b, b, Wb, Wb, 1, sp1));
-            MV_TRY(gemm6<128>(c, sp0, b, sp1, b, Wb, Yb, Wb));
-            MV_TRY(split_rows(c, Tm, b, b, Wb, Wb, 0, sp0));
-            MV_TRY(split_t(c, Z, b, b, Wb, Wb, 1, sp1));
-            MV_TRY(gemm6<128>(c, sp0, b, sp1, b, Wb, P, Wb));      // P = T Z
+            const NsPieces step{{P, nullptr}, {sp0, nullptr}, {sp1, nullptr}};
+            ns_pieces_kernel<true><<<dim3((unsigned)(b / 32), (unsigned)(b / 32), 1), 256, 0, c.s>>>(step, (int)b, Wb);
+            MV_TRY(gemmc_two<128>(yt0, sp1, Yb, sp0, yt1, P, b, 6 * Wb, b, 6 * Wb, 6 * Wb, Wb, c.s));   // P = T Z
             std::swap(Ya, Yb);
             std::swap(Z, P);
         }
