@@ -354,22 +354,31 @@ transpose_center_kernel(const float *__restrict__ R, int64_t ldR, int64_t n, int
     SquareSum q;
     const bool inside = i0 + kTile <= n;               // every asset of the tile exists (and ldM >= n)
     const float *src = R + (i0 - i_base + warp) * ldR + lane;
-    for (int t0 = tb; t0 < te; t0 += kTileT) {
-        const bool full = inside && te - t0 >= kTileT;
-        float x[RPW][H];
-        if (full) {
+    // the next tile's loads go out before this tile is centred
+    float x[RPW][H], nx[RPW][H];
+    auto fetch = [&](int t0, float (&v)[RPW][H]) {
+        if (inside && te - t0 >= kTileT) {
 #pragma unroll
             for (int j = 0; j < RPW; ++j)
 #pragma unroll
-                for (int h = 0; h < H; ++h) x[j][h] = src[(int64_t)(j * W) * ldR + t0 + h * kWarp];
+                for (int h = 0; h < H; ++h) v[j][h] = src[(int64_t)(j * W) * ldR + t0 + h * kWarp];
         } else {
 #pragma unroll
             for (int j = 0; j < RPW; ++j)
 #pragma unroll
                 for (int h = 0; h < H; ++h)
-                    x[j][h] = i0 + warp + j * W < n && lane + h * kWarp < te - t0 ? src[(int64_t)(j * W) * ldR + t0 + h * kWarp]
+                    v[j][h] = i0 + warp + j * W < n && lane + h * kWarp < te - t0 ? src[(int64_t)(j * W) * ldR + t0 + h * kWarp]
                                                                                    : 0.f;
         }
+    };
+    fetch(tb, nx);
+    for (int t0 = tb; t0 < te; t0 += kTileT) {
+        const bool full = inside && te - t0 >= kTileT;
+#pragma unroll
+        for (int j = 0; j < RPW; ++j)
+#pragma unroll
+            for (int h = 0; h < H; ++h) x[j][h] = nx[j][h];
+        if (t0 + kTileT < te) fetch(t0 + kTileT, nx);
 #pragma unroll
         for (int j = 0; j < RPW; ++j) {
             const int a = warp + j * W;
