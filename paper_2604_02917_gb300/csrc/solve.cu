@@ -305,45 +305,123 @@ step_size_sigma_kernel(SolveState *st, const float *__restrict__ u, const double
 // beta_{j+1} is negligible against alpha_j + beta_j: K_{j+1} is then
 // invariant under A and the Ritz values are eigenvalues.  No
 // reorthogonalisation: a lost orthogonality only repeats converged Ritz
-// values.  One block of kLanczosThreads; the loops are unrolled so that
-// each thread keeps several loads in flight (the vectors sit in L2).
+// values.  One block of kLanczosThreads.  Bound: latency, so up to
+// kLanczosKeep entries per thread (n <= 8192) are loaded once, all together,
+// q_j and q_{j-1} ahead of the wait for the product (a programmatic dependent
+// launch), and stay in registers through the three phases; and the FP64 sums
+// over the threads take the adds they need (block_sum_tree).  Reading the
+// vectors in each phase and reducing by butterflies took 13 us at n = 5440.
 constexpr int kLanczosThreads = 1024;
+constexpr int kLanczosKeep = 8;
 
+// The sum that block_sum<1> forms over 1024 threads, in the same tree (lane
+// halves within each warp, then the 32 warp sums the same way), but each level
+// adds on as few warps as it fills: a butterfly repeats every add on 32
+// lanes, 10 x 16 cycles of the SM's FP64 pipe per warp against 31 in all per
+// 32 values.  buf: 1024 doubles.  Every thread gets the sum.
+__device__ __forceinline__ double block_sum_tree(double v, double *buf) {
+    // after the level of width w, buf[warp * w + lane], lane < w, holds the warp's partials
+    const int t = threadIdx.x;
+    buf[t] = v;
+    __syncthreads();
+#pragma unroll
+    for (int w = 16; w >= 1; w >>= 1) {
+        double x = 0.0;
+        const bool on = t < 32 * w;
+        if (on) {
+            const int warp = t / w, lane = t % w;
+            x = buf[warp * 2 * w + lane] + buf[warp * 2 * w + lane + w];
+        }
+        __syncthreads();
+        if (on) buf[t] = x;
+        __syncthreads();
+    }
+    if (t < 32) {
+        const double x = warp_sum(buf[t]);
+        if (t == 0) buf[32] = x;
+    }
+    __syncthreads();
+    const double r = buf[32];
+    __syncthreads();
+    return r;
+}
+
+template <bool KEEP>
 __global__ void __launch_bounds__(kLanczosThreads)
 lanczos_kernel(const float *__restrict__ w, const float *__restrict__ qj, float *__restrict__ qprev,
                double *__restrict__ lan, const float *__restrict__ row_scale, float *__restrict__ y32, int n, int j) {
+    __shared__ double red[kLanczosThreads];
+    constexpr int E = KEEP ? kLanczosKeep : 1;
+    float q[E], p[E], v[E];
+    if constexpr (KEEP) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const int i = threadIdx.x + k * kLanczosThreads;
+            q[k] = i < n ? qj[i] : 0.f;
+            p[k] = i < n && j > 0 ? qprev[i] : 0.f;
+        }
+    }
+    umma::grid_dependency_wait();
     umma::launch_dependents();     // the next fused pass may start streaming L
-    __shared__ double red[kLanczosThreads / kWarp + 1];
     if (lan[1] != 0.0) return;     // the same value in every thread: written below, after the barriers
     const double b = j > 0 ? lan[2 + kMaxLanczos + j - 1] : 0.0;
     const float bf = (float)b;
     float pa = 0.f;
+    if constexpr (KEEP) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const int i = threadIdx.x + k * kLanczosThreads;
+            v[k] = i < n ? __ldcg(w + i) : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < E; ++k)
+            if (threadIdx.x + k * kLanczosThreads < n) pa = fmaf(q[k], v[k], pa);
+    } else {
 #pragma unroll 4
-    for (int i = threadIdx.x; i < n; i += kLanczosThreads) pa = fmaf(qj[i], w[i], pa);
-    double v[1] = {(double)pa};
-    block_sum<1, kLanczosThreads>(v, red);
-    const double a = v[0];
+        for (int i = threadIdx.x; i < n; i += kLanczosThreads) pa = fmaf(qj[i], w[i], pa);
+    }
+    const double a = block_sum_tree((double)pa, red);
     const float af = (float)a;
     float ps = 0.f;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < n; i += kLanczosThreads) {
-        float r = fmaf(-af, qj[i], w[i]);
-        if (j > 0) r = fmaf(-bf, qprev[i], r);
-        ps = fmaf(r, r, ps);
-    }
-    double ss[1] = {(double)ps};
-    block_sum<1, kLanczosThreads>(ss, red);
-    const double bn = sqrt(ss[0]);
-    const bool stop = !(bn > 1e-12 * (fabs(a) + b));
-    if (!stop) {
-        const float inv = (float)(1.0 / bn);
+    if constexpr (KEEP) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            float r = fmaf(-af, q[k], v[k]);
+            if (j > 0) r = fmaf(-bf, p[k], r);
+            if (threadIdx.x + k * kLanczosThreads < n) ps = fmaf(r, r, ps);
+            v[k] = r;
+        }
+    } else {
 #pragma unroll 4
         for (int i = threadIdx.x; i < n; i += kLanczosThreads) {
             float r = fmaf(-af, qj[i], w[i]);
             if (j > 0) r = fmaf(-bf, qprev[i], r);
-            const float q = r * inv;
-            qprev[i] = q;
-            y32[i] = row_scale ? q * row_scale[i] : q;
+            ps = fmaf(r, r, ps);
+        }
+    }
+    const double ss = block_sum_tree((double)ps, red);
+    const double bn = sqrt(ss);
+    const bool stop = !(bn > 1e-12 * (fabs(a) + b));
+    if (!stop) {
+        const float inv = (float)(1.0 / bn);
+        auto publish = [&](int i, float r) {
+            const float x = r * inv;
+            qprev[i] = x;
+            y32[i] = row_scale ? x * row_scale[i] : x;
+        };
+        if constexpr (KEEP) {
+#pragma unroll
+            for (int k = 0; k < E; ++k) {
+                const int i = threadIdx.x + k * kLanczosThreads;
+                if (i < n) publish(i, v[k]);
+            }
+        } else {
+#pragma unroll 4
+            for (int i = threadIdx.x; i < n; i += kLanczosThreads) {
+                float r = fmaf(-af, qj[i], w[i]);
+                if (j > 0) r = fmaf(-bf, qprev[i], r);
+                publish(i, r);
+            }
         }
     }
     if (threadIdx.x == 0) {
@@ -352,6 +430,15 @@ lanczos_kernel(const float *__restrict__ w, const float *__restrict__ qj, float 
         lan[0] = (double)(j + 1);
         if (stop) lan[1] = 1.0;
     }
+}
+
+// pdl: as a programmatic dependent of the product before it.
+static void start_lanczos(const float *w, const float *qj, float *qprev, double *lan, const float *rs, float *y32, int n,
+                          int j, cudaStream_t s, bool pdl) {
+    if (n <= kLanczosKeep * kLanczosThreads)
+        launch_grid(lanczos_kernel<true>, dim3(1), dim3(kLanczosThreads), 0, s, pdl, w, qj, qprev, lan, rs, y32, n, j);
+    else
+        launch_grid(lanczos_kernel<false>, dim3(1), dim3(kLanczosThreads), 0, s, pdl, w, qj, qprev, lan, rs, y32, n, j);
 }
 
 // Number of eigenvalues below x of the symmetric tridiagonal matrix with
@@ -1489,8 +1576,7 @@ static int launch_lanczos(const Plan &p, const mv_problem *P, int steps, void *w
             gemv_pair(p, P, y32, ws, nullptr, wd, s, w, kLoopPdl);
             *count += 3;
         }
-        lanczos_kernel<<<1, kLanczosThreads, 0, s>>>(w, q[j & 1], q[(j + 1) & 1], at<double>(ws, p.o_lan), rs, y32,
-                                                  p.n, j);
+        start_lanczos(w, q[j & 1], q[(j + 1) & 1], at<double>(ws, p.o_lan), rs, y32, p.n, j, s, kLoopPdl);
     }
     return cudaGetLastError() == cudaSuccess ? MV_OK : MV_ERR_CUDA;
 }
@@ -1513,7 +1599,7 @@ void launch_setup(SolveState *st, const double *mu, const double *r0, const floa
 }
 void launch_lanczos_step(const float *w, const float *qj, float *qprev, double *lan, const float *rs, float *y32,
                          int n, int j, cudaStream_t s) {
-    lanczos_kernel<<<1, kLanczosThreads, 0, s>>>(w, qj, qprev, lan, rs, y32, n, j);
+    start_lanczos(w, qj, qprev, lan, rs, y32, n, j, s, false);
 }
 void launch_lanczos_step_size(SolveState *st, const double *lan, double gamma, double safety, double alpha,
                               cudaStream_t s) {
