@@ -296,7 +296,7 @@ gemv_n_kernel(const void *__restrict__ L, int64_t ld, int n, int T, const float 
 //  * gemv_n: one row per warp instead of four, eight 16-byte loads at once;
 //  * both are launched as programmatic dependents and load L, which no
 //    kernel before them writes, ahead of the wait for their input vector.
-// The last block's sum over the splits keeps 64 (gemv_t) loads in flight:
+// The last block's sum over the splits keeps 32 loads in flight (gemv_t):
 // at 5440 x 512 it adds 85 splits, 22 round trips in the wide form.
 constexpr int kLatRows = 64;                 // rows per split the latency gemv_t holds
 constexpr int kLatSub = 4;                   // its column groups per strip of the wide form
@@ -323,7 +323,7 @@ __device__ __forceinline__ uint32_t ld_stream4(const void *p) {
 // of columns per thread), rows of split blockIdx.y.  Parameters as
 // gemv_t_body; tickets has one entry per b.
 template <int DT>
-__global__ void __launch_bounds__(kGemvThreads)
+__global__ void __launch_bounds__(kGemvThreads, 2)
 gemv_t_lat_kernel(const void *__restrict__ L, int64_t ld, int n, int T, const float *__restrict__ y32,
                   float *__restrict__ zpart, int64_t zstride, float *__restrict__ z, unsigned *__restrict__ tickets,
                   int rows_per_split, const volatile int *done, double *__restrict__ z64,
@@ -370,8 +370,8 @@ gemv_t_lat_kernel(const void *__restrict__ L, int64_t ld, int n, int T, const fl
         __syncthreads();
         if (!s_last) return;
         __threadfence();
-        // splits in order, 64 / CV of them in flight
-        constexpr int FL = kLatRows / CV;
+        // splits in order, 32 / CV of them in flight (64 took 188 registers, one block per SM)
+        constexpr int FL = 32 / CV;
 #pragma unroll
         for (int e = 0; e < CV; ++e) acc[e] = 0.f;
         const float *q = zpart + col;

@@ -732,7 +732,9 @@ __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char 
 
         // L L^T x^k by linearity from the product at y^k; the point to project:
         // x - alpha grad f(x) on a KKT test, else the gradient step from y^k.
-        auto from_y = [&](const Elem &e) { return e.y - alpha * (2.0 * e.gy + 2.0 * gamma * e.y); };
+        // (grouping fixed here, so that which product of the sum is fused is not the compiler's choice)
+        auto down = [&](double at, double g) { return __fma_rn(-alpha, __fma_rn(2.0, g, __dmul_rn(2.0 * gamma, at)), at); };
+        auto from_y = [&](const Elem &e) { return down(e.y, e.gy); };
         // f(i, element) over the thread's elements (all of them private to it)
         auto each = [&](auto f) {
 #pragma unroll
@@ -746,7 +748,7 @@ __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char 
             const double gxi = (k == 0) ? e.gy : (e.gy + beta_prev * e.gx) * inv1pb;
             if (real) a.gx[r0 + i] = gxi;
             el.mu[i] = e.mu;
-            el.v[i] = check ? e.x - alpha * (2.0 * gxi + 2.0 * gamma * e.x) : from_y(e);
+            el.v[i] = check ? down(e.x, gxi) : from_y(e);
         });
         if (!met) cluster_wait<CL>();
         met = true;
