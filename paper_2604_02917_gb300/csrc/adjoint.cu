@@ -269,7 +269,8 @@ int mv_npga_backward(const mv_problem *P, const mv_solve_opts *O_in, const doubl
     if (!(O.alpha > 0.0)) {
         for (int it = 0; it < O.power_iters; ++it) {
             if (p.use_llt)
-                MV_TRY(launch_llt(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), at<float>(ws, p.o_g32), s));
+                MV_TRY(launch_llt(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), at<float>(ws, p.o_g32), s, nullptr,
+                                  true));
             else
                 gemv_pair(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), s, at<float>(ws, p.o_g32));
             launch_power_norm(at<float>(ws, p.o_g32), nullptr, y32, n, s);
@@ -408,7 +409,8 @@ int mv_npga_backward(const mv_problem *P, const mv_solve_opts *O_in, const doubl
             MV_CUDA_TRY(launch_adj_proj(p.cl, a, cs));
             // w = L^T v_bar (z buffer) and L w
             if (p.use_llt)
-                MV_TRY(launch_llt(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), nullptr, cs, ZW + (size_t)(len + j) * T));
+                MV_TRY(launch_llt(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), nullptr, cs, ZW + (size_t)(len + j) * T,
+                                  true));
             else {
                 gemv_pair(p, P, y32, ws, nullptr, at<double>(ws, p.o_gy), cs);
                 MV_CUDA_TRY(cudaMemcpyAsync(ZW + (size_t)(len + j) * T, at<float>(ws, p.o_z), 4 * (size_t)T,

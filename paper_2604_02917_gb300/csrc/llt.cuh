@@ -267,7 +267,7 @@ llt_kernel(const __grid_constant__ CUtensorMap tmL, const LltArgs a) {
     constexpr int V4 = EPC / 4;                        // float4 pieces of one chunk's partials
     constexpr int RPT = kLltRowsPerThread;
     namespace cg = cooperative_groups;
-    umma::launch_dependents();                           // launched the plain way: the step may start beside this pass
+    if (!a.early) umma::launch_dependents();             // else after the wait below
     if (a.done != nullptr && *(const volatile int *)a.done) return;
 
     extern __shared__ uint8_t smem_raw[];
@@ -313,9 +313,20 @@ llt_kernel(const __grid_constant__ CUtensorMap tmL, const LltArgs a) {
             umma::tma_load_2d(dst + (uint32_t)(i * a.box_rows * RB), &tmL, b * W, row0 + i * a.box_rows,
                               full0 + 8 * s);
     };
-    if (warp == kLltConsumerWarps && lane == 0) {
+    const bool producer = warp == kLltConsumerWarps && lane == 0;
+    if (producer) {                                      // L is read-only: ahead of the wait too
         umma::prefetch_tensormap(&tmL);
         for (int j = 0; j < kLltStages && j < nj; ++j) issue(j);
+    }
+    if (a.early) {                                       // y, done and the scratch are the predecessor's
+        umma::grid_dependency_wait();
+        umma::launch_dependents();
+        if (a.done != nullptr && *(const volatile int *)a.done) {
+            if (producer)                                // the issued stages land before the CTA leaves
+                for (int j = 0; j < kLltStages && j < nj; ++j)
+                    if (!umma::mbar_wait(full0 + 8 * j, 0u, kLltWaitNs)) atomicExch(a.err, 4);
+            return;
+        }
     }
     for (int i = tid; i < a.rpc; i += kLltThreads) {
         const int r = row0 + i;

@@ -146,7 +146,7 @@ int llt_launch(const LltPlan &lp, int dt, const void *L, int64_t n, int64_t T, i
     a.nbox = lp.nbox;
     a.nb = lp.nb;
     a.G = lp.G;
-    a.early = (pdl && lp.tn) ? 1 : 0;
+    a.early = pdl ? 1 : 0;
     cudaError_t e;
     if (lp.tn)
         e = dt == MV_F32    ? llt_launch_tn_f32(lp.C, lp.G, lp.smem, &map, a, s)

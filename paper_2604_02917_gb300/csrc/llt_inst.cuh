@@ -65,7 +65,7 @@ template <int C, int RB>
 cudaError_t launch(int G, size_t smem, const void *map, const LltArgs &a, cudaStream_t s) {
     if (attrs<C, RB>() != MV_OK) return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = config(C, G, smem, s, attr);
+    const cudaLaunchConfig_t cfg = config(C, G, smem, s, attr, a.early != 0);
     return cudaLaunchKernelEx(&cfg, llt_kernel<MV_LLT_DT, C, RB>, *reinterpret_cast<const CUtensorMap *>(map), a);
 }
 
