@@ -107,14 +107,32 @@ __device__ __forceinline__ void chunk_store(const float (&acc)[128], int row, in
     }
 }
 
+// Tile lin of the pair form's launch order (256 x 256 tiles): grouped raster
+// over pairs of row tiles as in gemm.cuh.
+__device__ __forceinline__ void pair_tile(int lin, int M, int N, int raster, int &pr, int &ct) {
+    constexpr int rows = kRasterRows / 2;
+    const int npr = (M + 2 * kBM - 1) / (2 * kBM), nct = (N + 255) / 256;
+    if (raster && npr > rows) {
+        const int per = rows * nct, g = lin / per, first = g * rows;
+        const int gh = min(npr - first, rows), rem = lin - g * per;
+        pr = first + rem % gh;
+        ct = rem / gh;
+    } else {
+        pr = lin % npr;
+        ct = lin / npr;
+    }
+}
+
 // With gridDim.z = 2 one launch forms two products of the same shape (plane 1:
-// A1 B1^T into C1), for shapes whose tiles fill a fraction of the SMs.
+// A1 B1^T into C1), for shapes whose tiles fill a fraction of the SMs.  tail >= 0
+// (BN = 128): the quarters of the pair form's tiles tail, tail + 1, ..., four
+// CTAs each, started beside the pair form's last full wave.
 template <int BN, int NA>
 __global__ void __launch_bounds__(GemmChunkCfg<BN, NA>::THREADS, 1)
 gemm_chunk_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
                   const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmA1,
                   const __grid_constant__ CUtensorMap tmB1, float *__restrict__ C0, float *__restrict__ C1, int M, int N,
-                  int K, int64_t ldc, GemmEpi e, int raster) {
+                  int K, int64_t ldc, GemmEpi e, int raster, int tail) {
     const CUtensorMap *tmA = blockIdx.z ? &tmA1 : &tmA0, *tmB = blockIdx.z ? &tmB1 : &tmB0;
     float *C = blockIdx.z ? C1 : C0;
     using Cfg = GemmChunkCfg<BN, NA>;
@@ -131,13 +149,20 @@ gemm_chunk_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constan
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int rt = blockIdx.x, ct = blockIdx.y;
-    if (raster && (int)gridDim.x > kRasterRows) {        // grouped raster (see gemm.cuh)
+    if (tail < 0 && raster && (int)gridDim.x > kRasterRows) {        // grouped raster (see gemm.cuh)
         const int nrt = (int)gridDim.x, nct = (int)gridDim.y;
         const int lin = (int)blockIdx.x + nrt * (int)blockIdx.y;
         const int per = kRasterRows * nct, g = lin / per, first = g * kRasterRows;
         const int gh = min(nrt - first, kRasterRows), rem = lin - g * per;
         rt = first + rem % gh;
         ct = rem / gh;
+    }
+    if (tail >= 0) {
+        int pr, pc;
+        pair_tile(tail + ((int)blockIdx.x >> 2), M, N, raster, pr, pc);
+        rt = 2 * pr + ((int)blockIdx.x & 1);
+        ct = 2 * pc + (((int)blockIdx.x >> 1) & 1);
+        if (rt * kBM >= M || ct * BN >= N) return;       // a quarter outside C (never the first of a tile)
     }
     const int m0 = rt * kBM, n0 = ct * BN;
     const int nk = (K + kBK - 1) / kBK;
@@ -255,6 +280,7 @@ gemm_chunk_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constan
     __syncthreads();
     umma::fence_after_sync();
     if (warp == 1) umma::tmem_dealloc(tmem, Cfg::TMEM_COLS);
+    if (tail >= 0) umma::grid_dependency_wait();         // this launch's end is also the full waves' end
 }
 
 // ------------------------------------------------------------------ CTA-pair form
@@ -306,17 +332,8 @@ gemm_chunk_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = umma::cluster_ctarank();            // 0: issues the MMAs
-    // the pair's tile (pr, ct); grouped raster over pairs as in gemm.cuh
-    const int npr = (int)gridDim.x >> 1, nct = (int)gridDim.y;
-    int pr = (int)blockIdx.x >> 1, ct = (int)blockIdx.y;
-    if (raster && npr > kRasterRows / 2) {
-        const int rows = kRasterRows / 2;
-        const int lin = pr + npr * (int)blockIdx.y;
-        const int per = rows * nct, g = lin / per, first = g * rows;
-        const int gh = min(npr - first, rows), rem = lin - g * per;
-        pr = first + rem % gh;
-        ct = rem / gh;
-    }
+    int pr, ct;                                               // the pair's tile
+    pair_tile((int)blockIdx.x >> 1, M, N, raster, pr, ct);
     const int m0 = (2 * pr + (int)rank) * kBM;                // this CTA's rows of A and of D
     const int n0 = ct * BN;                                    // the pair's columns
     const int nb0 = n0 + (int)rank * (BN / 2);                 // this CTA's half of B
@@ -341,6 +358,7 @@ gemm_chunk_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     umma::fence_before_sync();
     cooperative_groups::this_cluster().sync();                                 // both CTAs' barriers exist
     umma::fence_after_sync();
+    umma::launch_dependents();                                                 // the tail's quarters (they read no output)
     const uint32_t tmem = *tmem_slot;
     const uint32_t full_r0 = umma::mapa_rank(full0, 0);         // rank 0's full[0], cluster address
 
@@ -477,7 +495,7 @@ static void gemmc_launch(const CUtensorMap &ta, const CUtensorMap &tb, const CUt
     dim3 grid((unsigned)((M + kBM - 1) / kBM), (unsigned)((N + BN - 1) / BN), ta1 ? 2 : 1);
     gemm_chunk_kernel<BN, NA><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(ta, tb, ta2 ? *ta2 : ta, ta1 ? *ta1 : ta,
                                                                     tb1 ? *tb1 : tb, C, C1, (int)M, (int)N, (int)K, ldc, e,
-                                                                    raster);
+                                                                    raster, -1);
 }
 
 template <int NA>
@@ -493,40 +511,65 @@ static int gemmc_pair_set_attrs() {
 
 // gemmc<256> on CTA pairs (256 x 256 tiles; clusters of 2 along M).  Tensor
 // maps: A boxes of 128 rows, B boxes of 128 rows (half a tile).
+//
+// A pair takes a wave's time for a tile however few tiles the last wave has
+// (10 waves for the 704 tiles of 5440 x 8192, 20 tiles in the last).  A last
+// wave at most half full is therefore run as 128 x 128 quarters on single
+// CTAs, one round on all SMs at about half the time (above half it would
+// take two rounds); every entry keeps its order of additions.  BF16 calls:
+// 1733 x 9001 to 1000 (28 tiles) 117 -> 103 us, 3000 x 20000 to 2048 (96)
+// 324 -> 304 us, 5440 x 48374 to 2048 (176) 999 -> 962 us, to 8192 (704,
+// under the power cap) 3.44 -> 3.40 ms.  The quarters
+// are a programmatic dependent of the full waves: they start on the SMs that
+// those leave, and end after them.
+constexpr int kPairs = 152 / 2;                     // CTA pairs that run at once
+template <int NA>
+static int gemmc_pair_run(const CUtensorMap &ta, const CUtensorMap &tb, const CUtensorMap &ta2, int64_t M, int64_t N,
+                          int64_t K, float *C, int64_t ldc, const GemmEpi &e, cudaStream_t s, int raster) {
+    const int tiles = (int)(((M + 2 * kBM - 1) / (2 * kBM)) * ((N + 255) / 256));
+    const int tail = tiles % kPairs <= kPairs / 2 ? tiles % kPairs : 0, full = tiles - tail;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cudaError_t err = cudaSuccess;
+    if (full > 0) {
+        MV_TRY(gemmc_pair_set_attrs<NA>());
+        cfg.gridDim = dim3(2u * (unsigned)full);
+        cfg.blockDim = dim3(GemmPairCfg<NA>::THREADS);
+        cfg.dynamicSmemBytes = GemmPairCfg<NA>::SMEM;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.numAttrs = 1;
+        err = cudaLaunchKernelEx(&cfg, gemm_chunk_pair_kernel<NA>, ta, tb, ta2, C, (int)M, (int)N, (int)K, ldc, e,
+                                 raster);
+    }
+    if (tail > 0 && err == cudaSuccess) {
+        MV_TRY((gemmc_set_attrs<128, NA>()));
+        cfg.gridDim = dim3(4u * (unsigned)tail);
+        cfg.blockDim = dim3(GemmChunkCfg<128, NA>::THREADS);
+        cfg.dynamicSmemBytes = GemmChunkCfg<128, NA>::SMEM;
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.numAttrs = full > 0 ? 1 : 0;
+        err = cudaLaunchKernelEx(&cfg, gemm_chunk_kernel<128, NA>, ta, tb, ta2, ta, tb, C, (float *)nullptr, (int)M,
+                                 (int)N, (int)K, ldc, e, raster, full);
+    }
+    if (err != cudaSuccess) return record_cuda_error(err, "chunked pair GEMM launch", __FILE__, __LINE__);
+    return MV_OK;
+}
+
 static int gemmc_pair(const void *A, const void *A2, int64_t M, int64_t lda, const void *B, int64_t N, int64_t ldb,
                       int64_t K, float *C, int64_t ldc, const GemmEpi &e, cudaStream_t s, int raster = 1) {
     if (K < 1) return record_message(MV_ERR_INVALID_ARG, "chunked GEMM: K must be >= 1");
     CUtensorMap ta, tb, ta2;
     MV_TRY(make_map_bf16(&ta, A, M, K, lda, kBM));
     MV_TRY(make_map_bf16(&tb, B, N, K, ldb, 128));
-    if (A2) MV_TRY(make_map_bf16(&ta2, A2, M, K, lda, kBM));
-    const unsigned pairs = (unsigned)((M + 2 * kBM - 1) / (2 * kBM));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * pairs, (unsigned)((N + 255) / 256));
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t err;
-    if (A2) {
-        MV_TRY(gemmc_pair_set_attrs<2>());
-        cfg.blockDim = dim3(GemmPairCfg<2>::THREADS);
-        cfg.dynamicSmemBytes = GemmPairCfg<2>::SMEM;
-        err = cudaLaunchKernelEx(&cfg, gemm_chunk_pair_kernel<2>, ta, tb, ta2, C, (int)M, (int)N, (int)K, ldc, e,
-                                 raster);
-    } else {
-        MV_TRY(gemmc_pair_set_attrs<1>());
-        cfg.blockDim = dim3(GemmPairCfg<1>::THREADS);
-        cfg.dynamicSmemBytes = GemmPairCfg<1>::SMEM;
-        err = cudaLaunchKernelEx(&cfg, gemm_chunk_pair_kernel<1>, ta, tb, ta, C, (int)M, (int)N, (int)K, ldc, e,
-                                 raster);
-    }
-    if (err != cudaSuccess) return record_cuda_error(err, "chunked pair GEMM launch", __FILE__, __LINE__);
-    return MV_OK;
+    if (A2 == nullptr) return gemmc_pair_run<1>(ta, tb, ta, M, N, K, C, ldc, e, s, raster);
+    MV_TRY(make_map_bf16(&ta2, A2, M, K, lda, kBM));
+    return gemmc_pair_run<2>(ta, tb, ta2, M, N, K, C, ldc, e, s, raster);
 }
 
 // 256-column tiles run on CTA pairs.
