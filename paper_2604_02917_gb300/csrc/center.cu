@@ -40,13 +40,14 @@ int record_message(int status, const char *msg) {
     return status;
 }
 
-// Sum of FP32 values, exact but for the final rounding.  A value is a 24-bit
-// significand m (signed) times 2^(e - 150); m << (e - eb) is added to a
-// 64-bit integer while e lies in [eb, eb + 30] (under 2^54 each, so 256 of
+// Sum of FP32 values: exact within a flush, whose total (up to 256 values) is
+// rounded to FP64 and added in FP64, as are the threads' sums.  A value is a
+// 24-bit significand m (signed) times 2^(e - 150); m << (e - eb) is added to
+// a 64-bit integer while e lies in [eb, eb + 30] (under 2^54 each, so 256 of
 // them fit), eb being set so that the first value seen has 8 octaves of
-// headroom.  Anything outside that window (a value 2^8 above or 2^-22 below
-// the first, infinities, NaN) is added in FP64; a larger value also moves
-// the window.  About 10 integer operations per value, against an FP64
+// headroom (fewer above 2^119: the window ends below the field 255).
+// Anything outside that window (a value 2^8 above or 2^-22 below the first,
+// infinities, NaN) is added in FP64; a larger value also moves the window.  About 10 integer operations per value, against an FP64
 // conversion and addition at 2 per clock and SM.
 struct RowSum {
     long long acc = 0;
@@ -63,7 +64,8 @@ struct RowSum {
         const int e = (int)(b >> 23);
         if (e >= 1 && e < 255 && (eb == 1 << 20 || e > eb + 30)) {
             flush();
-            eb = e > 23 ? e - 22 : 1;      // never 0: the significand of e = 0 has no implicit bit
+            // never 0: the significand of e = 0 has no implicit bit; at most 224: field 255 stays outside
+            eb = e > 23 ? min(e - 22, 224) : 1;
             add_inside(x);
         } else {
             wide += (double)x;
