@@ -15,8 +15,10 @@
 //    (RowSum);
 //  * centred entry: an FP32 pair with a proven error bound, FP64 when the
 //    bound leaves the rounding open (centred());
-//  * sum of squares: an FP32 pair per thread (SquareSum).
-// With FP64 per entry 5440 x 48374 FP32 took 3.55 ms.
+//  * sum of squares: FP32 pairs, 16 entries at a time (SquareSum).
+// With FP64 per entry 5440 x 48374 FP32 took 3.55 ms; so it takes 0.57 ms (0.74 ms
+// transposed) at the same error of the trace: 0.9e-16 (root mean square over
+// panels of 2000 x 20000) against 1.4e-16.
 #include <stdio.h>
 #include <string.h>
 
@@ -108,17 +110,20 @@ struct RowSum {
 // Constants of one row: mean and c = 1/sqrt(T-1) as FP32 pairs, and the
 // absolute part of the error bound of centred().  `wide` is infinite where
 // the FP32 range cannot be relied on (the row's largest |R| outside
-// [2^-30, 2^50], infinities or NaN): every entry then takes the FP64 path.
+// [2^-30, 2^50], infinities or NaN), and in small panels: every entry then
+// takes the FP64 path.  A square of a pair is off by 2^-49 or so; over kPairMin
+// of them that averages to FP64's own error, over fewer it would not.
+constexpr int64_t kPairMin = 1 << 16;
 struct RowConst {
     float mh, ml, ch, cl, wide;
 };
-__device__ __forceinline__ RowConst row_const(double mean, double c, float amax) {
+__device__ __forceinline__ RowConst row_const(double mean, double c, float amax, bool small) {
     RowConst k;
     k.mh = (float)mean;
     k.ml = (float)(mean - (double)k.mh);
     k.ch = (float)c;
     k.cl = (float)(c - (double)k.ch);
-    const bool ok = amax >= 0x1p-30f && amax <= 0x1p50f && fabsf(k.mh) <= 0x1p50f;
+    const bool ok = !small && amax >= 0x1p-30f && amax <= 0x1p50f && fabsf(k.mh) <= 0x1p50f;
     k.wide = ok ? fmaf(fabsf(k.mh) * k.ch, 0x1p-44f, 0x1p-120f) : INFINITY;
     return k;
 }
@@ -129,21 +134,36 @@ __device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
 
-// Sum of squares of FP32 pairs (p, r), two at a time: s + c carries about 48
-// bits per thread; values centred in FP64 are added in FP64.
+// Sum of squares of FP32 pairs (s, e), two at a time, without the factor c^2
+// (which would bring in the error of c as a pair; the blocks divide by T - 1
+// in FP64).  (s + e)^2 = s^2 + (2 s e + e^2), the first square as a product
+// and its error, the second term rounded as one sum: every rounding is to
+// nearest of a sum whose last bits vary, so none has a preferred sign (added
+// after 2 s e, e^2 would be lost each time: 7e-16 of the sum).  The pair
+// (h, l) that collects them (Knuth's error-free addition) goes to FP64 every
+// kSquareFlush additions (4: 0.59 and 0.74 ms for 0.57 and 0.74, the same
+// error).  Values centred in FP64 are added in FP64.
+constexpr int kSquareFlush = 8;
 struct SquareSum {
-    float2 s = make_float2(0.f, 0.f), c = make_float2(0.f, 0.f);
+    float2 h = make_float2(0.f, 0.f), l = make_float2(0.f, 0.f);
     double wide = 0.0;
-    __device__ __forceinline__ void add(float2 p, float2 r) {
-        const float2 q = __fmul2_rn(p, p);
-        float2 e = __ffma2_rn(p, p, neg2(q));                       // p^2 = q + e exactly
-        e = __ffma2_rn(__ffma2_rn(splat(2.f), p, r), r, e);
-        const float2 t = __fadd2_rn(s, q), bb = sub2(t, s);         // s + q = t + (rounding error), exactly
-        c = __fadd2_rn(c, __fadd2_rn(__fadd2_rn(sub2(s, sub2(t, bb)), sub2(q, bb)), e));
-        s = t;
+    __device__ __forceinline__ void add(float2 s, float2 e) {
+        const float2 q = __fmul2_rn(s, s);
+        const float2 m = __ffma2_rn(__fadd2_rn(s, s), e, __fmul2_rn(e, e));
+        const float2 r = __fadd2_rn(__ffma2_rn(s, s, neg2(q)), m);
+        const float2 t = __fadd2_rn(h, q), bb = sub2(t, h);         // h + q = t + (rounding error), exactly
+        l = __fadd2_rn(l, __fadd2_rn(__fadd2_rn(sub2(h, sub2(t, bb)), sub2(q, bb)), r));
+        h = t;
     }
-    __device__ __forceinline__ double total() const {
-        return wide + (((double)s.x + (double)c.x) + ((double)s.y + (double)c.y));
+    __device__ __forceinline__ void flush() {
+        const float t = h.x + h.y, bb = t - h.x;                    // the two lanes' pairs as one
+        const float r = ((h.x - (t - bb)) + (h.y - bb)) + (l.x + l.y);
+        wide += (double)t + (double)r;
+        h = l = make_float2(0.f, 0.f);
+    }
+    __device__ __forceinline__ double total() {
+        flush();
+        return wide;
     }
 };
 
@@ -157,13 +177,14 @@ struct SquareSum {
 // 2^18) d is formed in FP64.  BF16 adds one case: an FP32 value on a BF16 tie
 // does not say which way the FP64 value rounds.  Returns the values to store
 // (for BF16 already rounded to it on the FP64 path) and adds the squares of
-// the first `use` entries to q.
+// x - mean, to FP64 or as the pair (s, e), of the first `use` entries to q.
 template <int DT>
 __device__ __forceinline__ float2 centred(float2 x, const RowConst &k, double mean, double c, int use, SquareSum &q) {
     const float2 mh = splat(k.mh), ch = splat(k.ch);
-    const float2 s = sub2(x, mh), bb = sub2(s, x);
-    const float2 e = sub2(sub2(sub2(x, sub2(s, bb)), __fadd2_rn(mh, bb)), splat(k.ml));
-    float2 p = __fmul2_rn(s, ch);
+    float2 s = sub2(x, mh);
+    const float2 bb = sub2(s, x);
+    float2 e = sub2(sub2(sub2(x, sub2(s, bb)), __fadd2_rn(mh, bb)), splat(k.ml));
+    const float2 p = __fmul2_rn(s, ch);
     float2 r = __ffma2_rn(s, ch, neg2(p));
     r = __ffma2_rn(s, splat(k.cl), r);
     r = __ffma2_rn(e, ch, r);
@@ -177,20 +198,20 @@ __device__ __forceinline__ float2 centred(float2 x, const RowConst &k, double me
     }
     if (wx || wy || use < 2) {
         auto in64 = [&](float v) {
-            const double d = ((double)v - mean) * c;
-            q.wide = fma(d, d, q.wide);
+            const double u = (double)v - mean, d = u * c;
+            q.wide = fma(u, u, q.wide);
             return DT == MV_BF16 ? __bfloat162float(__double2bfloat16(d)) : (float)d;
         };
         if (wx || use < 1) {
             if (use >= 1) f.x = in64(x.x);
-            p.x = r.x = 0.f;
+            s.x = e.x = 0.f;
         }
         if (wy || use < 2) {
             if (use >= 2) f.y = in64(x.y);
-            p.y = r.y = 0.f;
+            s.y = e.y = 0.f;
         }
     }
-    q.add(p, r);
+    q.add(s, e);
     return f;
 }
 
@@ -223,7 +244,7 @@ template <int DT, bool WRITE, int NT>
 __global__ void __launch_bounds__(NT)
 center_kernel(const float *__restrict__ R, int64_t ldR, unsigned T, void *__restrict__ L, int64_t ldL,
               float *__restrict__ row_scale, double *__restrict__ mu, double *__restrict__ rowsq,
-              float *__restrict__ amax_out, int64_t i_base) {
+              float *__restrict__ amax_out, int64_t i_base, bool small) {
     constexpr int U = kCenterUnroll;
     __shared__ double red[NT / kWarp + 1];
     __shared__ float s_lo[NT / kWarp], s_hi[NT / kWarp];
@@ -287,7 +308,7 @@ center_kernel(const float *__restrict__ R, int64_t ldR, unsigned T, void *__rest
         ra = fmaxf(fabsf(xmin), fabsf(xmax));
     }
     if constexpr (WRITE) {
-        const RowConst k = row_const(mean, c, ra);
+        const RowConst k = row_const(mean, c, ra, small);
         SquareSum q;
         const int64_t o = i * ldL;
         auto write2 = [&](float2 x, unsigned ta, unsigned tb, int use) {
@@ -296,12 +317,15 @@ center_kernel(const float *__restrict__ R, int64_t ldR, unsigned T, void *__rest
             if (use > 1) store_elem<DT>(L, o + tb, f.y, inv_scale);
         };
         t = threadIdx.x;
+        int adds = 0;
         for (; t + (U - 1) * NT < T; t += U * NT) {
             float x[U];
 #pragma unroll
             for (int j = 0; j < U; ++j) x[j] = r[t + j * NT];
 #pragma unroll
             for (int j = 0; j < U; j += 2) write2(make_float2(x[j], x[j + 1]), t + j * NT, t + (j + 1) * NT, 2);
+            adds += U / 2;
+            if (adds % kSquareFlush == 0) q.flush();
         }
         for (; t < T; t += 2 * NT) {
             const bool two = t + NT < T;
@@ -311,7 +335,7 @@ center_kernel(const float *__restrict__ R, int64_t ldR, unsigned T, void *__rest
         double v[1] = {q.total()};
         __syncthreads();
         block_sum<1, NT>(v, red);
-        if (threadIdx.x == 0) rowsq[i] = v[0];
+        if (threadIdx.x == 0) rowsq[i] = v[0] / (double)(T - 1);
     } else if (threadIdx.x == 0) {
         amax_out[i] = ra;
     }
@@ -333,7 +357,8 @@ template <int DT>
 __global__ void __launch_bounds__(kTransThreads)
 transpose_center_kernel(const float *__restrict__ R, int64_t ldR, int64_t n, int T, void *__restrict__ M, int64_t ldM,
                         const float *__restrict__ row_scale, const double *__restrict__ mu,
-                        const float *__restrict__ amax, double *__restrict__ sqpart, int64_t i_base, int slices) {
+                        const float *__restrict__ amax, double *__restrict__ sqpart, int64_t i_base, int slices,
+                        bool small) {
     constexpr int W = kTransThreads / kWarp, RPW = kTile / W;   // warps, asset rows per warp
     constexpr int H = kTileT / kWarp;                           // loads per row and tile
     __shared__ float tile[kTile][kTileT + 1];
@@ -349,7 +374,7 @@ transpose_center_kernel(const float *__restrict__ R, int64_t ldR, int64_t n, int
     if (threadIdx.x < kTile) {
         const int64_t i = i0 + threadIdx.x;
         s_mean[threadIdx.x] = i < n ? mu[i] : 0.0;
-        s_k[threadIdx.x] = row_const(s_mean[threadIdx.x], c, i < n ? amax[i] : 1.f);
+        s_k[threadIdx.x] = row_const(s_mean[threadIdx.x], c, i < n ? amax[i] : 1.f, small);
     }
     __syncthreads();
     const float inv = (DT == MV_FP8_E4M3 && i0 + lane < n) ? 1.f / row_scale[i0 + lane] : 1.f;
@@ -394,6 +419,7 @@ transpose_center_kernel(const float *__restrict__ R, int64_t ldR, int64_t n, int
                 tile[a][lane + h * kWarp] = use > 0 ? f.x : 0.f;
                 tile[a][lane + (h + 1) * kWarp] = use > 1 ? f.y : 0.f;
             }
+            if ((j + 1) * H % (2 * kSquareFlush) == 0) q.flush();
         }
         __syncthreads();
         if (i0 + lane < ldM) {
@@ -406,7 +432,7 @@ transpose_center_kernel(const float *__restrict__ R, int64_t ldR, int64_t n, int
     }
     double v[1] = {q.total()};
     block_sum<1, kTransThreads>(v, red);
-    if (threadIdx.x == 0 && i0 < n) sqpart[(i0 / kTile) * slices + slice] = v[0];
+    if (threadIdx.x == 0 && i0 < n) sqpart[(i0 / kTile) * slices + slice] = v[0] / (double)(T - 1);
 }
 
 // trace(Sigma): the sum of the blocks' partials, in a fixed order.
@@ -437,17 +463,18 @@ static void center_chunk(const float *R_rows, int64_t ldR, int64_t n, int64_t T,
                          int64_t ldL, float *d_row_scale, double *d_mu, double *rowsq, float *amax, int64_t i0,
                          int64_t i1, int slices, cudaStream_t s) {
     const unsigned rows = (unsigned)(i1 - i0);
+    const bool small = n * T < kPairMin;
     const bool few = rows < 152 * 8;                           // one row per block: about 8 blocks of 128 per SM
     const int64_t wend = (tn && i1 == n) ? ldL : i1;          // transposed: columns written by this chunk
     const dim3 tgrid((unsigned)slices, (unsigned)((wend - i0 + kTile - 1) / kTile));
 #define MV_CENTER_ROWS(DT, WRITE, NT, RS)                                                                        \
     center_kernel<DT, WRITE, NT><<<rows, NT, 0, s>>>(R_rows, ldR, (unsigned)T, WRITE ? d_L : nullptr, ldL, RS,   \
-                                                     d_mu, rowsq, amax, i0)
+                                                     d_mu, rowsq, amax, i0, small)
 #define MV_CENTER_CASE(DT, RS)                                                                                   \
     if (tn) {                                                                                                    \
         if (few) MV_CENTER_ROWS(DT, false, kRowThreadsFew, RS); else MV_CENTER_ROWS(DT, false, kRowThreads, RS); \
         transpose_center_kernel<DT><<<tgrid, kTransThreads, 0, s>>>(R_rows, ldR, n, (int)T, d_L, ldL, RS, d_mu,  \
-                                                                    amax, rowsq, i0, slices);                    \
+                                                                    amax, rowsq, i0, slices, small);             \
     } else {                                                                                                     \
         if (few) MV_CENTER_ROWS(DT, true, kRowThreadsFew, RS); else MV_CENTER_ROWS(DT, true, kRowThreads, RS);   \
     }
