@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(kProjNT) adj_proj_kernel(AdjArgs a) {
     const int n = a.n, nl = (n + CL - 1) / CL, r0 = min(n, rank * nl), r1 = min(n, r0 + nl);
     const double nu = a.nu_tape[a.j], beta = a.betas[*a.k0 + a.j];
     const bool active = a.eq || nu != 0.0;
+    cluster_arrive<CL>();
     proj_smem_init(&psm);
     double s[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // |S|, sum mu, sum mu^2, sum a, sum mu a
     for (int i = r0 + threadIdx.x; i < r1; i += kProjNT) {
@@ -91,6 +92,7 @@ __global__ void __launch_bounds__(kProjNT) adj_proj_kernel(AdjArgs a) {
             s[4] = fma(m, ab, s[4]);
         }
     }
+    cluster_wait<CL>();
     cluster_sums<CL, 5>(&psm, s, dsl);
     double c1 = 0.0, c2 = 0.0;
     const double det = s[0] * s[2] - s[1] * s[1];

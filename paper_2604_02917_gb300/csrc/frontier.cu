@@ -57,12 +57,14 @@ __global__ void __launch_bounds__(kProjNT) frontier_init_kernel(FArgs a) {
     const int n = a.n, nl = (n + CL - 1) / CL, r0 = min(n, rank * nl), r1 = min(n, r0 + nl);
     ProjElems el = carve_elems(dsm, nl);
     el.n = r1 - r0;
+    cluster_arrive<CL>();
     proj_smem_init(&psm);
     for (int i = threadIdx.x; i < el.n; i += kProjNT) {
         el.v[i] = 1.0 / n;
         el.mu[i] = a.mu[r0 + i];
     }
     __syncthreads();
+    cluster_wait<CL>();
     ClusterProj<CL> P{&psm, el};
     P.prepare();
     const ProjOut o = P.solve(a.Rt[b], a.mode, a.st->mu_min, a.st->mu_max, 0.0, -INFINITY, kProjBudget);
@@ -96,7 +98,8 @@ __global__ void __launch_bounds__(kProjNT) frontier_step_kernel(FArgs a) {
     __shared__ double sc[3];
     const int b = blockIdx.x / CL, rank = cluster_rank<CL>();
     FState *fs = a.fs + b;
-    if (*(volatile int *)&fs->done) return;      // uniform over the cluster (see npga_step_kernel)
+    if (*(volatile int *)&fs->done) return;      // uniform over the cluster: written after the wait below
+    cluster_arrive<CL>();
     const int n = a.n, nl = (n + CL - 1) / CL, r0 = min(n, rank * nl), r1 = min(n, r0 + nl);
     const int k = fs->k;
     const double beta_prev = fs->beta_prev, inv1pb = fs->inv1pb, t = fs->t, alpha = a.st->alpha;
@@ -130,6 +133,7 @@ __global__ void __launch_bounds__(kProjNT) frontier_step_kernel(FArgs a) {
         }
     }
     __syncthreads();
+    cluster_wait<CL>();
     ClusterProj<CL> P{&psm, el};
     if (check) {
         P.prepare(hint);

@@ -17,6 +17,7 @@ project_batch_kernel(const double *__restrict__ v, const double *__restrict__ mu
     const int r1 = min(n, r0 + nl);
     ProjElems el = carve_elems(dsm, nl);
     el.n = r1 - r0;
+    cluster_arrive<CL>();
     proj_smem_init(&psm);
     const double *vb = v + (int64_t)b * n;
     double mn = INFINITY, mx = -INFINITY;
@@ -28,6 +29,7 @@ project_batch_kernel(const double *__restrict__ v, const double *__restrict__ mu
         mx = fmax(mx, m);
     }
     __syncthreads();
+    cluster_wait<CL>();
     ClusterProj<CL> P{&psm, el};
     P.reduce_minmax(mn, mx);
     P.prepare();

@@ -227,9 +227,9 @@ __device__ __forceinline__ void cluster_barrier() {
     }
 }
 
-// The same barrier in two halves, for work between them; the first exchange
-// of a kernel must follow one, since a peer's shared memory may only be
-// written once the peer runs.
+// The same barrier in two halves, for work between them.  Every kernel that
+// exchanges has one before its first exchange (arrive on entry, wait behind
+// the loads): a peer's shared memory may only be written once the peer runs.
 template <int CL>
 __device__ __forceinline__ void cluster_arrive() {
     if constexpr (CL > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");

@@ -534,12 +534,14 @@ __device__ __forceinline__ void init_x_body(SolveState *st, const double *__rest
     if (x_in == nullptr) {
         ProjElems el = carve_elems(dsm, nl);
         el.n = r1 - r0;
+        cluster_arrive<CL>();
         proj_smem_init(&psm);
         for (int i = threadIdx.x; i < el.n; i += kProjNT) {
             el.v[i] = 1.0 / n;
             el.mu[i] = mu[r0 + i];
         }
         __syncthreads();
+        cluster_wait<CL>();
         ClusterProj<CL> P{&psm, el};
         P.dyk = dyk_slice(dyk, rank, nl);
         P.dyk_iters = dyk_iters;
@@ -880,7 +882,8 @@ __global__ void variant_setup_kernel(SolveState *st, int momentum, double m_f, i
 template <int CL>
 __device__ __forceinline__ void npga_bt_step_body(const StepArgs &a, unsigned char *dsm, ProjSmem &psm) {
     SolveState *st = a.st;
-    if (*(volatile int *)&st->done) return;
+    if (*(volatile int *)&st->done) return;        // uniform over the cluster: written after the wait below
+    cluster_arrive<CL>();
     const int n = a.n;
     const int rank = cluster_rank<CL>();
     const int nl = (n + CL - 1) / CL;
@@ -902,6 +905,7 @@ __device__ __forceinline__ void npga_bt_step_body(const StepArgs &a, unsigned ch
     double tn = t, beta = st->beta_prev;
     bool accepted = false, rejected = false, numeric = false;
     for (int i = threadIdx.x; i < el.n; i += kProjNT) el.mu[i] = a.mu[r0 + i];
+    cluster_wait<CL>();
     if (started) {
         double s1 = 0.0, s2 = 0.0;
         for (int i = threadIdx.x; i < el.n; i += kProjNT) {
