@@ -268,7 +268,10 @@ llt_kernel(const __grid_constant__ CUtensorMap tmL, const LltArgs a) {
     constexpr int RPT = kLltRowsPerThread;
     namespace cg = cooperative_groups;
     if (!a.early) umma::launch_dependents();             // else after the wait below
-    if (a.done != nullptr && *(const volatile int *)a.done) return;
+    if (a.done != nullptr && *(const volatile int *)a.done) {
+        if (a.early) umma::grid_dependency_wait();       // what starts behind this pass relies on its having waited
+        return;
+    }
 
     extern __shared__ uint8_t smem_raw[];
     // aligned up to 1024 bytes by pointer arithmetic on the shared array (an
@@ -515,7 +518,10 @@ __device__ __forceinline__ void lltt_body(const CUtensorMap *tm, const LltArgs &
     constexpr int RPT = (ES == 4) ? 2 : 1;               // column chunks per thread in phase B
     namespace cg = cooperative_groups;
     if (!a.early) umma::launch_dependents();             // else after the wait below
-    if (a.done != nullptr && *(const volatile int *)a.done) return;
+    if (a.done != nullptr && *(const volatile int *)a.done) {
+        if (a.early) umma::grid_dependency_wait();       // what starts behind this pass relies on its having waited
+        return;
+    }
 
     extern __shared__ uint8_t smem_raw[];
     // aligned up to 1024 bytes by pointer arithmetic on the shared array (an
