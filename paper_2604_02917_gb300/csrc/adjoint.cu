@@ -121,9 +121,11 @@ __global__ void __launch_bounds__(kProjNT) adj_proj_kernel(AdjArgs a) {
     cluster_barrier<CL>();
 }
 
-// y_bar = v_bar - alpha (2 L L^T v_bar + 2 gamma v_bar).
-__global__ void adj_finish_kernel(const double *__restrict__ vbar, const double *__restrict__ llv, double alpha,
-                                  double gamma, double *__restrict__ ybar, int n) {
+// y_bar = v_bar - alpha (2 L L^T v_bar + 2 gamma v_bar).  (v_bar and L L^T v_bar
+// come from kernels that may still run when this one starts: plain pointers,
+// no read-only loads.)
+__global__ void adj_finish_kernel(const double *vbar, const double *llv, double alpha, double gamma,
+                                  double *__restrict__ ybar, int n) {
     umma::grid_dependency_wait();          // launched beside the product
     umma::launch_dependents();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;

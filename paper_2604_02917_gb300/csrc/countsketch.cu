@@ -62,6 +62,10 @@ static CsWs cs_carve(void *ws, int64_t T, int64_t m) {
 
 // The five kernels run as a chain of programmatic dependent launches: each
 // starts while the one before drains, waits for it, then lets the next start.
+// What the ones before wrote (counts, offsets, list) is read by ordinary loads
+// through plain pointers: the read-only path, which const __restrict__ and
+// __ldg ask for, is for memory that nobody writes while the kernel lives, and
+// this kernel may be alive before the writes.
 __device__ __forceinline__ void cs_chain() {
     umma::grid_dependency_wait();
     umma::launch_dependents();
@@ -94,7 +98,7 @@ __global__ void cs_count_kernel(const int *__restrict__ h, int T, int m, int *__
 }
 
 // Exclusive scan of m counts by one block of 1024 threads (chunked).
-__global__ void __launch_bounds__(1024) cs_scan_kernel(const int *__restrict__ cnt, int m, int *__restrict__ off) {
+__global__ void __launch_bounds__(1024) cs_scan_kernel(const int *cnt, int m, int *off) {
     __shared__ int part[1024];
     cs_chain();
     const int per = (m + 1023) / 1024;
@@ -118,7 +122,7 @@ __global__ void __launch_bounds__(1024) cs_scan_kernel(const int *__restrict__ c
 }
 
 __global__ void cs_fill_kernel(const int *__restrict__ h, const int8_t *__restrict__ sign, int T, int m,
-                               const int *__restrict__ off, int *__restrict__ fill, unsigned *__restrict__ list) {
+                               const int *off, int *__restrict__ fill, unsigned *list) {
     cs_chain();
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < T; t += gridDim.x * blockDim.x) {
         const int b = h[t];
@@ -137,7 +141,7 @@ __device__ __forceinline__ unsigned cs_key(unsigned e) { return e & 0x7fffffffu;
 // in registers through a fixed 16-input odd-even transposition network (a
 // uniform hash leaves a few periods per bucket), above kCsRankMax by
 // insertion in place.
-__device__ __forceinline__ void cs_sort_bucket(unsigned *__restrict__ list, int p0, int nb) {
+__device__ __forceinline__ void cs_sort_bucket(unsigned *list, int p0, int nb) {
     if (nb <= 16) {
         unsigned v[16];
 #pragma unroll
@@ -174,7 +178,7 @@ __device__ __forceinline__ void cs_sort_bucket(unsigned *__restrict__ list, int 
 // One thread inserting in global memory took most of the call where buckets
 // are long (89 periods: 0.4 of 0.65 ms at 1498 x 47924 to 540 columns).
 __global__ void __launch_bounds__(kCsSortThreads)
-cs_sort_kernel(const int *__restrict__ off, int m, unsigned *__restrict__ list, int *__restrict__ err) {
+cs_sort_kernel(const int *off, int m, unsigned *list, int *__restrict__ err) {
     __shared__ unsigned buf[kCsSortThreads / kWarp][kCsRankMax];
     cs_chain();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -205,8 +209,8 @@ cs_sort_kernel(const int *__restrict__ off, int m, unsigned *__restrict__ list, 
 
 template <int DT, int NT>
 __global__ void __launch_bounds__(NT)
-cs_tn_kernel(const void *__restrict__ Lt, int64_t ld, int n, int m, const int *__restrict__ off,
-             const unsigned *__restrict__ list, const float *__restrict__ rs, float *__restrict__ out, int64_t ldS,
+cs_tn_kernel(const void *__restrict__ Lt, int64_t ld, int n, int m, const int *off,
+             const unsigned *list, const float *__restrict__ rs, float *__restrict__ out, int64_t ldS,
              int ncache) {
     using St = Store<DT>;
     constexpr int VEC = St::VEC;
@@ -220,10 +224,10 @@ cs_tn_kernel(const void *__restrict__ Lt, int64_t ld, int n, int m, const int *_
     // the group's 9 bucket boundaries and its run of the list (what exceeds the cache is read as it comes)
     __shared__ int bnd[kCsGroup + 1];
     unsigned *cache = reinterpret_cast<unsigned *>(tile + kCsGroup * CHUNK);
-    if (threadIdx.x <= kCsGroup) bnd[threadIdx.x] = __ldg(off + min(j0 + (int)threadIdx.x, m));
+    if (threadIdx.x <= kCsGroup) bnd[threadIdx.x] = off[min(j0 + (int)threadIdx.x, m)];
     __syncthreads();
     const int p0 = bnd[0], p1 = bnd[kCsGroup];
-    for (int k = threadIdx.x; k < min(p1 - p0, ncache); k += NT) cache[k] = __ldg(list + p0 + k);
+    for (int k = threadIdx.x; k < min(p1 - p0, ncache); k += NT) cache[k] = list[p0 + k];
     __syncthreads();
     float acc[VEC];
 #pragma unroll
@@ -243,7 +247,7 @@ cs_tn_kernel(const void *__restrict__ Lt, int64_t ld, int n, int m, const int *_
 #pragma unroll
         for (int k = 0; k < kCsLoads; ++k) {
             const int at = p + k - p0;
-            e[k] = p + k < p1 ? (at < ncache ? cache[at] : __ldg(list + p + k)) : 0u;
+            e[k] = p + k < p1 ? (at < ncache ? cache[at] : list[p + k]) : 0u;
         }
 #pragma unroll
         for (int k = 0; k < kCsLoads; ++k)
@@ -290,8 +294,8 @@ cs_tn_kernel(const void *__restrict__ Lt, int64_t ld, int n, int m, const int *_
 
 template <int DT>
 __global__ void __launch_bounds__(kCsNtThreads)
-cs_nt_kernel(const void *__restrict__ L, int64_t ld, int T, int m, const int *__restrict__ off,
-             const unsigned *__restrict__ list, const float *__restrict__ rs, float *__restrict__ out, int64_t ldS) {
+cs_nt_kernel(const void *__restrict__ L, int64_t ld, int T, int m, const int *off,
+             const unsigned *list, const float *__restrict__ rs, float *__restrict__ out, int64_t ldS) {
     using St = Store<DT>;
     using E = typename St::elem;
     extern __shared__ __align__(16) unsigned char row[];
@@ -309,7 +313,7 @@ cs_nt_kernel(const void *__restrict__ L, int64_t ld, int T, int m, const int *__
         float acc = 0.f;
         const int p1 = off[j + 1];
         for (int p = off[j]; p < p1; ++p) {
-            const unsigned e = __ldg(list + p);
+            const unsigned e = list[p];
             const int t = (int)(e & 0x7fffffffu);
             float x;
             if constexpr (DT == MV_F32) {

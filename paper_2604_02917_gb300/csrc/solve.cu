@@ -308,7 +308,8 @@ step_size_sigma_kernel(SolveState *st, const float *__restrict__ u, const double
 // values.  One block of kLanczosThreads.  Bound: latency, so up to
 // kLanczosKeep entries per thread (n <= 8192) are loaded once, all together,
 // q_j and q_{j-1} ahead of the wait for the product (a programmatic dependent
-// launch), and stay in registers through the three phases; and the FP64 sums
+// launch; w and the record, which kernels before this one may still be
+// writing when it starts, go through plain pointers), and stay in registers through the three phases; and the FP64 sums
 // over the threads take the adds they need (block_sum_tree).  Reading the
 // vectors in each phase and reducing by butterflies took 13 us at n = 5440.
 constexpr int kLanczosThreads = 1024;
@@ -348,8 +349,8 @@ __device__ __forceinline__ double block_sum_tree(double v, double *buf) {
 
 template <bool KEEP>
 __global__ void __launch_bounds__(kLanczosThreads)
-lanczos_kernel(const float *__restrict__ w, const float *__restrict__ qj, float *__restrict__ qprev,
-               double *__restrict__ lan, const float *__restrict__ row_scale, float *__restrict__ y32, int n, int j) {
+lanczos_kernel(const float *w, const float *__restrict__ qj, float *__restrict__ qprev, double *lan,
+               const float *__restrict__ row_scale, float *__restrict__ y32, int n, int j) {
     __shared__ double red[kLanczosThreads];
     constexpr int E = KEEP ? kLanczosKeep : 1;
     float q[E], p[E], v[E];

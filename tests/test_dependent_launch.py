@@ -43,3 +43,21 @@ def test_no_way_out_before_the_wait(name):
     body = DEPENDENT[name][1]
     first = WAIT.search(body).start()
     assert not re.search(r"\breturn\b(?! Elem)", re.sub(r"\[&\][^{};]*\{[^{}]*\}", "", body[:first]))
+
+
+# Inputs of the calls and vectors complete before the predecessor started (the Lanczos q_j: two products back).
+# Everything else a dependent kernel reads may be written while it is already alive, so the read-only path
+# (const __restrict__, __ldg) is closed to it; __ldcg is a coherent load that stays behind the wait.
+SETTLED = {"L", "Lt", "h", "sign", "rs", "row_scale", "cscale", "qj"}
+
+
+@pytest.mark.parametrize("name", sorted(DEPENDENT))
+def test_no_read_only_loads_of_a_running_predecessors_output(name):
+    params, body = DEPENDENT[name]
+    for p in re.findall(r"\bconst\s+[\w:]+\s*\*\s*__restrict__\s*(\w+)", params):
+        if p in SETTLED:
+            continue
+        uses = re.findall(rf"(?<!\.)\b{p}\b", body)
+        assert len(uses) == len(re.findall(rf"__ldcg\({p}\b", body)), f"{name}: {p}"
+    for expr in re.findall(r"__ldg\((\w+)", body):
+        assert expr in SETTLED, f"{name}: __ldg({expr}"
