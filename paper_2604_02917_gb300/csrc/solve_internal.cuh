@@ -74,11 +74,14 @@ inline T_ *at(void *ws, size_t off) {
     return reinterpret_cast<T_ *>(reinterpret_cast<char *>(ws) + off);
 }
 
-// One cached graph per distinct (problem, options, workspace) triple.
+// One cached graph per distinct (problem, options, workspace) triple.  The
+// layout decides the kernels and the workspace offsets, the step's cluster
+// size (which can be set by hand) the offsets; n, T and ld do not tell them
+// apart where n = T or both have the same pitch.
 struct GraphKey {
     const void *L, *mu, *rs, *ws;
     int64_t n, T, ld;
-    int dt, mode, kkt_every, max_iter, chunk, fused;
+    int dt, layout, cl, mode, kkt_every, max_iter, chunk, fused;
     double R, gamma, eps;
     const void *ev;
     int momentum, backtrack, budget, dyk_iters;
@@ -86,7 +89,7 @@ struct GraphKey {
     double aux = 0.0;                    // any further scalar baked into the graph (the adjoint's alpha)
     bool operator==(const GraphKey &o) const {
         return L == o.L && mu == o.mu && rs == o.rs && ws == o.ws && n == o.n && T == o.T && ld == o.ld &&
-               dt == o.dt && mode == o.mode && kkt_every == o.kkt_every && max_iter == o.max_iter &&
+               dt == o.dt && layout == o.layout && cl == o.cl && mode == o.mode && kkt_every == o.kkt_every && max_iter == o.max_iter &&
                chunk == o.chunk && fused == o.fused && R == o.R && gamma == o.gamma && eps == o.eps && ev == o.ev &&
                momentum == o.momentum && backtrack == o.backtrack && budget == o.budget &&
                dyk_iters == o.dyk_iters && bt_rho == o.bt_rho && m_f == o.m_f && aux == o.aux;
