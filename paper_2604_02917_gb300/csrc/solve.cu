@@ -1442,9 +1442,9 @@ static void peek_free(Peek &p) {
 struct PeekLease {
     Peek p;
     bool ok = false;
-    PeekLease() {
+    explicit PeekLease(bool wanted) {
         int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) return;
+        if (!wanted || cudaGetDevice(&dev) != cudaSuccess) return;
         {
             std::lock_guard<std::mutex> lock(g_peek_mu);
             for (size_t i = 0; i < g_peeks.size(); ++i)
@@ -1786,28 +1786,39 @@ int mv_npga_solve(const mv_problem *P, const mv_solve_opts *O_in, double *d_x_in
     SolveState hs{};
     int k_prev = 0, timed = 0;
     double t_t = 0.0, t_n = 0.0, t_s = 0.0;
-    // With graphs the next chunk is launched before the last one's flag is
-    // read: the host's turn-round (about 13 us) runs beside it, and a chunk
-    // behind the end returns kernel by kernel (about 20 us, once).
-    if (exec) {
-        PeekLease peek;
-        if (peek.ok) {
-            auto launch = [&](int64_t c) -> int {
-                MV_CUDA_TRY(cudaGraphLaunch(exec, s));
-                launches += per_iter * chunk;
-                MV_CUDA_TRY(cudaMemcpyAsync(&peek.p.hs[c & 1], st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
-                MV_CUDA_TRY(cudaEventRecord(peek.p.ev[c & 1], s));
-                return MV_OK;
-            };
-            MV_TRY(launch(0));
-            for (int64_t c = 0; c < max_chunks; ++c) {
-                if (c + 1 < max_chunks) MV_TRY(launch(c + 1));
-                MV_CUDA_TRY(cudaEventSynchronize(peek.p.ev[c & 1]));
-                hs = peek.p.hs[c & 1];
-                if (hs.done) break;
-            }
-            max_chunks = 0;                               // the loop below is for the other cases
+    // With graphs a chunk may be launched before the flag of the one before it
+    // is read: the host's turn-round (about 13 us) then runs beside it.  If the
+    // solve ends in the earlier chunk, the later one's kernels only return one
+    // by one, which takes longer (20 to 30 us), so it goes ahead where the
+    // residuals say that it will be needed: the fall of the last chunk, once
+    // more, does not reach eps, and max_iter lies beyond.  A solve of one or two
+    // chunks runs them one at a time (a warm start that stops at its first
+    // test, 200 x 1000: 149 us, with a chunk always ahead 180 us).
+    PeekLease peek(exec != nullptr);                      // until the last copies are enqueued: it waits for a chunk ahead
+    if (peek.ok) {
+        auto launch = [&](int64_t c) -> int {
+            MV_CUDA_TRY(cudaGraphLaunch(exec, s));
+            launches += per_iter * chunk;
+            MV_CUDA_TRY(cudaMemcpyAsync(&peek.p.hs[c & 1], st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
+            MV_CUDA_TRY(cudaEventRecord(peek.p.ev[c & 1], s));
+            return MV_OK;
+        };
+        double kkt[2] = {INFINITY, INFINITY};             // of the last two chunks read
+        auto needed = [&](int64_t c) {                    // chunk c, with chunk c - 1 in flight and c - 2 read
+            if (c < 3 || hs.k + chunk > O.max_iter) return false;
+            return !(kkt[1] * std::min(1.0, kkt[1] / kkt[0]) <= O.eps);
+        };
+        MV_TRY(launch(0));
+        for (int64_t c = 0, sent = 1; c < max_chunks; ++c) {
+            if (sent == c + 1 && sent < max_chunks && needed(sent)) MV_TRY(launch(sent++));
+            MV_CUDA_TRY(cudaEventSynchronize(peek.p.ev[c & 1]));
+            hs = peek.p.hs[c & 1];
+            if (hs.done) break;
+            kkt[0] = kkt[1];
+            kkt[1] = hs.kkt;
+            if (sent == c + 1 && sent < max_chunks) MV_TRY(launch(sent++));
         }
+        max_chunks = 0;                                   // the loop below is for the other cases
     }
     for (int64_t c = 0; c < max_chunks; ++c) {
         if (exec) {
