@@ -289,7 +289,7 @@ gemv_n_kernel(const void *__restrict__ L, int64_t ld, int n, int T, const float 
 // ---------------------------------------------------------------- latency forms
 // The same two products for matrices that do not fill the machine (compressed
 // factors, small universes), where a launch is a chain of L2 round trips, not
-// a stream.  Every value is formed by the same additions in the same order as
+// a stream (make_plan draws the line, with both forms' times).  Every value is formed by the same additions in the same order as
 // above, so the forms agree bit for bit; what differs is who forms it:
 //  * gemv_t: 4 bytes of columns per thread instead of 16, four times the
 //    blocks, all rows of a split (at most 64) loaded at once;

@@ -73,9 +73,21 @@ Plan make_plan(int dt, int64_t n, int64_t T, int64_t ld, int grouped_rows, bool 
     p.n_splits = (int)((gc + p.n_cols - 1) / p.n_cols);
     // The latency forms (gemv.cuh).  gemv_t: where a split's rows fit its
     // registers and its tickets (kLatSub per strip) the 256 bytes the wide
-    // form's take anyway.  gemv_n: where the wide grid leaves SMs idle or
-    // with one block (2 per SM).
-    p.t_lat = grouped_rows <= 0 && p.t_rows <= kLatRows && p.t_blocks <= 64 / kLatSub;
+    // form's take anyway, and the matrix is small: its 4-byte loads and four
+    // times the blocks cost more the more strips there are to a row and the more
+    // blocks in all, and strips x blocks is where the two forms cross (both
+    // gemvs of a gradient, us, latency against wide form; strips x blocks in
+    // brackets): FP32 4000 x 4000 [1008] 45.6 / 46.5, 20000 x 2000 [1252] 86.5 /
+    // 87.1, 7000 x 4000 [1760] 66.4 / 61.5, 7000 x 16000 [28160] 193 / 176; BF16
+    // 7000 x 4000 [440] 62.7 / 64.0, 10000 x 4000 [628] 77.5 / 70.3, 7000 x 32000
+    // [28160] 254 / 176; FP8, whose unpacking the wide form does on a quarter of
+    // the threads, stays ahead to four strips: 20000 x 8000 [1252] 163 / 202,
+    // 14000 x 16000 [3504] 180 / 188, 7000 x 32000 [7040] 167 / 159, 7000 x 64000
+    // [28160] 288 / 224.
+    // gemv_n: where the wide grid leaves SMs idle or with one block (2 per SM).
+    const int64_t lat_max = dt == MV_BF16 ? 448 : 1280;
+    p.t_lat = grouped_rows <= 0 && p.t_rows <= kLatRows && p.t_blocks <= 64 / kLatSub &&
+              ((dt == MV_FP8_E4M3 && p.t_blocks <= 4) || (int64_t)p.t_blocks * p.t_blocks * p.t_splits <= lat_max);
     p.t_ticks = p.t_lat ? p.t_blocks * kLatSub : p.t_blocks;
     p.n_lat = grouped_rows <= 0 && (int64_t)p.n_groups * p.n_splits < 2 * (int64_t)sms;
     size_t off = 0;
