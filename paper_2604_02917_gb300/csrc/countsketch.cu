@@ -132,75 +132,70 @@ __global__ void cs_fill_kernel(const int *__restrict__ h, const int8_t *__restri
     }
 }
 
-constexpr int kCsRankMax = 1024;              // periods per bucket a warp sorts by rank
-constexpr int kCsSortThreads = 128;
+constexpr int kCsShort = 16;                  // periods per bucket that one thread sorts
 
 __device__ __forceinline__ unsigned cs_key(unsigned e) { return e & 0x7fffffffu; }
 
-// Ascending periods within one bucket of nb entries at list[p0..): up to 16
-// in registers through a fixed 16-input odd-even transposition network (a
-// uniform hash leaves a few periods per bucket), above kCsRankMax by
-// insertion in place.
+// Ascending periods within one bucket of nb <= kCsShort entries at
+// list[p0..), in registers through a fixed odd-even transposition network (a
+// uniform hash leaves a few periods per bucket).
 __device__ __forceinline__ void cs_sort_bucket(unsigned *list, int p0, int nb) {
-    if (nb <= 16) {
-        unsigned v[16];
+    unsigned v[kCsShort];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = i < nb ? list[p0 + i] : 0xffffffffu;   // padding sorts last
+    for (int i = 0; i < kCsShort; ++i) v[i] = i < nb ? list[p0 + i] : 0xffffffffu;   // padding sorts last
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
+    for (int r = 0; r < kCsShort; ++r) {
 #pragma unroll
-            for (int i = r & 1; i + 1 < 16; i += 2) {
-                const unsigned x = v[i], y = v[i + 1];
-                const bool sw = cs_key(x) > cs_key(y);
-                v[i] = sw ? y : x;
-                v[i + 1] = sw ? x : y;
-            }
+        for (int i = r & 1; i + 1 < kCsShort; i += 2) {
+            const unsigned x = v[i], y = v[i + 1];
+            const bool sw = cs_key(x) > cs_key(y);
+            v[i] = sw ? y : x;
+            v[i + 1] = sw ? x : y;
         }
+    }
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
-            if (i < nb) list[p0 + i] = v[i];
-        return;
-    }
-    for (int p = p0 + 1; p < p0 + nb; ++p) {
-        const unsigned x = list[p];
-        int q = p - 1;
-        while (q >= p0 && cs_key(list[q]) > cs_key(x)) {
-            list[q + 1] = list[q];
-            --q;
-        }
-        list[q + 1] = x;
-    }
+    for (int i = 0; i < kCsShort; ++i)
+        if (i < nb) list[p0 + i] = v[i];
 }
 
-// Sort every bucket (a bucket above kCsMaxBucket periods is refused): a
-// thread per bucket, but 17 to kCsRankMax periods by the whole warp, each lane
-// placing its entries by counting the smaller keys (periods are distinct).
-// One thread inserting in global memory took most of the call where buckets
-// are long (89 periods: 0.4 of 0.65 ms at 1498 x 47924 to 540 columns).
-__global__ void __launch_bounds__(kCsSortThreads)
-cs_sort_kernel(const int *off, int m, unsigned *list, int *__restrict__ err) {
-    __shared__ unsigned buf[kCsSortThreads / kWarp][kCsRankMax];
+// Sort every bucket (a bucket above kCsMaxBucket periods is refused): short
+// ones a thread each, longer ones by the whole warp, each lane placing its
+// entries by counting the smaller keys (periods are distinct): nb^2 / 128
+// reads of four keys from shared memory, a few ms at worst.  A warp takes
+// `per` buckets, 32, or one where the average bucket is long.  (One thread
+// inserting in global memory took most of the call where buckets are long:
+// 100 x 30000 to 20 columns, 1500 periods each, 54 ms, and 234 ms in blocks of
+// four warps; now 0.52 ms.)
+__global__ void __launch_bounds__(kWarp)
+cs_sort_kernel(const int *off, int m, int per, unsigned *list, int *__restrict__ err) {
+    __shared__ __align__(16) unsigned buf[kCsMaxBucket];   // (period, sign) as 2 t + sign: the same order
     cs_chain();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int total = (m + kWarp - 1) / kWarp * kWarp;         // whole warps take part in the ballots
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < total; b += gridDim.x * blockDim.x) {
-        const int p0 = b < m ? off[b] : 0, nb = b < m ? off[b + 1] - p0 : 0;
-        const bool by_rank = nb > 16 && nb <= kCsRankMax;
+    const int lane = threadIdx.x;
+    for (int b0 = blockIdx.x * per; b0 < m; b0 += gridDim.x * per) {
+        const int b = b0 + lane;
+        const bool mine = lane < per && b < m;
+        const int p0 = mine ? off[b] : 0, nb = mine ? off[b + 1] - p0 : 0;
         if (nb > kCsMaxBucket)
             atomicExch(err, 2);
-        else if (!by_rank)
+        else if (nb <= kCsShort)
             cs_sort_bucket(list, p0, nb);
-        for (unsigned todo = __ballot_sync(0xffffffffu, by_rank); todo != 0; todo &= todo - 1) {
+        for (unsigned todo = __ballot_sync(0xffffffffu, nb > kCsShort && nb <= kCsMaxBucket); todo != 0; todo &= todo - 1) {
             const int src = __ffs((int)todo) - 1;
             const int q0 = __shfl_sync(0xffffffffu, p0, src), nq = __shfl_sync(0xffffffffu, nb, src);
-            for (int i = lane; i < nq; i += kWarp) buf[warp][i] = list[q0 + i];
+            for (int i = lane; i < nq + (-nq & 3); i += kWarp) {
+                const unsigned e = i < nq ? list[q0 + i] : 0u;
+                buf[i] = i < nq ? (e << 1) | (e >> 31) : 0xffffffffu;      // the padding counts nowhere
+            }
             __syncwarp();
             for (int i = lane; i < nq; i += kWarp) {
-                const unsigned x = buf[warp][i];
+                const unsigned x = buf[i];
                 int rank = 0;
-#pragma unroll 8
-                for (int k = 0; k < nq; ++k) rank += cs_key(buf[warp][k]) < cs_key(x) ? 1 : 0;
-                list[q0 + rank] = x;
+#pragma unroll 4
+                for (int k = 0; k < nq; k += 4) {
+                    const uint4 y = *reinterpret_cast<const uint4 *>(buf + k);
+                    rank += (y.x < x ? 1 : 0) + (y.y < x ? 1 : 0) + (y.z < x ? 1 : 0) + (y.w < x ? 1 : 0);
+                }
+                list[q0 + rank] = (x >> 1) | (x << 31);
             }
             __syncwarp();
         }
@@ -404,11 +399,12 @@ int mv_countsketch(const void *d_L, int32_t dtype, int32_t layout, const float *
     CsWs w = cs_carve(d_ws, T, m);
     MV_CUDA_TRY(cudaMemsetAsync(w.cnt, 0, cs_zero_bytes(m), s));
     const int tb = (int)std::min<int64_t>((T + 255) / 256, 4096);
-    const int sb = (int)std::min<int64_t>((m + kCsSortThreads - 1) / kCsSortThreads, 4096);
+    const int per = T > (int64_t)kCsShort * m ? 1 : kWarp;       // buckets per warp of the sort
+    const int sb = (int)std::min<int64_t>((m + per - 1) / per, 4096);
     MV_CUDA_TRY(cs_start(cs_count_kernel, dim3(tb), 256, 0, s, d_hash, (int)T, (int)m, w.cnt, w.err));
     MV_CUDA_TRY(cs_start(cs_scan_kernel, dim3(1), 1024, 0, s, w.cnt, (int)m, w.off));
     MV_CUDA_TRY(cs_start(cs_fill_kernel, dim3(tb), 256, 0, s, d_hash, d_sign, (int)T, (int)m, w.off, w.fill, w.list));
-    MV_CUDA_TRY(cs_start(cs_sort_kernel, dim3(sb), kCsSortThreads, 0, s, w.off, (int)m, w.list, w.err));
+    MV_CUDA_TRY(cs_start(cs_sort_kernel, dim3(sb), kWarp, 0, s, w.off, (int)m, per, w.list, w.err));
     const float *rs = dtype == MV_FP8_E4M3 ? d_row_scale : nullptr;
     switch (dtype) {
         case MV_F32: MV_TRY(cs_launch<MV_F32>(layout, d_L, ldL, (int)n, (int)T, (int)m, w, rs, d_L_sketch, ldS, s)); break;
