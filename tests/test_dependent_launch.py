@@ -33,7 +33,7 @@ for _path in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.jo
 def test_the_kernels_are_found():
     assert set(DEPENDENT) == {"llt_kernel", "lltt_body", "gemv_t_lat_kernel", "gemv_n_lat_kernel", "lanczos_kernel",
                               "npga_step_body", "adj_proj_kernel", "adj_finish_kernel", "cs_count_kernel",
-                              "cs_scan_kernel", "cs_fill_kernel", "cs_sort_kernel", "cs_tn_kernel", "cs_nt_kernel",
+                              "cs_scan_kernel", "cs_fill_kernel", "cs_sort_kernel", "cs_tn_kernel",
                               "gemm_chunk_kernel"}
 
 
