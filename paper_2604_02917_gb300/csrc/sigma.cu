@@ -28,7 +28,14 @@
 // last N mod P run whole; those last r tiles would leave most of a wave
 // idle, so each is cut into floor(P / r) K-ranges whose partial sums go to
 // the workspace and are added in range order by a second kernel.  With few
-// tiles (small n) all of them are cut.
+// tiles (small n) all of them are cut, from two chunks on (kernels' time, cut
+// against whole: 300 x 2000 BF16 13.1 / 19.2 us, 2000 x 1000 FP32 30.7 / 31.3,
+// 1500 x 5000 FP32 55.8 / 89.5).
+//
+// Every store of the epilogue and of the joining kernel covers 128 bytes of a
+// row.  With the accumulators' own layout, one row per lane, the epilogue alone
+// held a small or short-T call up (300 x 700 BF16: 27.5 us of kernel, now 13.0;
+// 4000 x 700 51 -> 29; 2500 x 3000 29).
 //
 // Pipeline per CTA as in gemm_chunk.cuh's pair kernel: warp 0 (one thread)
 // TMA producer, warp 1 of rank 0 (one thread) MMA issuer, warps 2..9 the
@@ -280,10 +287,9 @@ sigma_pair_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant
         if (!ok) {
             if (lane == 0) atomicExch(&g_gemm_err, 3);
         } else if (slot >= 0) {                              // a K-range's partial, added by sigma_join_kernel
-            float *dst = part + ((int64_t)slot * kSigTile + (int)rank * kSigHalf + 32 * q + lane) * kSigTile + grp * 128;
+            float *dst = part + (int64_t)slot * kSigTile * kSigTile + ((((int)rank * 4 + q) * 2 + grp) * 128) * 32 + lane;
 #pragma unroll
-            for (int j = 0; j < 128; j += 4)
-                *reinterpret_cast<float4 *>(dst + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+            for (int j = 0; j < 128; ++j) dst[j * 32] = acc[j];
         } else {
             const bool diag = I == J;
             const float sr = (rs != nullptr && row < n) ? rs[row] : 1.f;
@@ -291,22 +297,34 @@ sigma_pair_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant
 #pragma unroll
                 for (int j = 0; j < 128; ++j) acc[j] *= sr * (cb + j < n ? __ldg(rs + cb + j) : 0.f);
             }
-            if (row < n) {
-                float *srow = Sig + (int64_t)row * ldS;
-                if (!diag && cb + 128 <= n) {
+            // Rows of the tile: the accumulators hold one row per lane, and a
+            // store of 32 rows costs 32 memory sectors, so each 32 x 32 piece is
+            // turned in shared memory (the stages are free: the last chunk's
+            // MMAs have read them all) and written 128 bytes of a row at a time.
+            const int r0 = m0 + 32 * q, rows = min(32, n - r0), cols = min(128, n - cb);
+            float *turn = reinterpret_cast<float *>(smem) + (warp - 2) * (32 * 33);
+            if (rows > 0 && cols > 0) {
 #pragma unroll
-                    for (int j = 0; j < 128; j += 4)
-                        *reinterpret_cast<float4 *>(srow + cb + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
-                } else {
+                for (int p = 0; p < 4; ++p) {
+                    const int c = cb + p * 32, col = c + lane;
+                    if (p * 32 >= cols || (diag && c + 31 < r0)) continue;      // nothing to store: the same in every lane
 #pragma unroll
-                    for (int j = 0; j < 128; ++j)
-                        if (cb + j < n && (!diag || cb + j >= row)) srow[cb + j] = acc[j];
+                    for (int j = 0; j < 32; ++j) turn[lane * 33 + j] = acc[p * 32 + j];
+                    __syncwarp();
+                    float *dst = Sig + (int64_t)r0 * ldS + col;
+                    const int last = col >= n ? 0 : (diag ? min(rows, col - r0 + 1) : rows);   // rows of this column
+#pragma unroll 8
+                    for (int r = 0; r < rows; ++r, dst += ldS)
+                        if (r < last) *dst = turn[r * 33 + lane];
+                    __syncwarp();
                 }
-            }
-            // mirror: for fixed j the 32 lanes write 32 consecutive floats
+                // mirror: for fixed j the 32 lanes write 32 consecutive floats
+                float *dst = Sig + (int64_t)cb * ldS + row;
+                const int first = row >= n ? cols : (diag ? row - cb + 1 : 0);                   // columns above the diagonal
 #pragma unroll
-            for (int j = 0; j < 128; ++j)
-                if (row < n && cb + j < n && (!diag || cb + j > row)) Sig[(int64_t)(cb + j) * ldS + row] = acc[j];
+                for (int j = 0; j < 128; ++j, dst += ldS)
+                    if (j >= first && j < cols) *dst = acc[j];
+            }
         }
     }
     umma::fence_before_sync();
@@ -316,7 +334,9 @@ sigma_pair_kernel(const __grid_constant__ CUtensorMap tmH, const __grid_constant
 }
 
 // The cut tiles: partials added in range order, scaled, written with their
-// mirror.  One block of 32 x 8 threads per 32 x 32 piece of a tile.
+// mirror.  One block of 32 x 8 threads per 32 x 32 piece of a tile.  A partial
+// is stored as the epilogue's warps hold it, 32 rows by 128 columns each, the
+// rows of a column side by side (both sides then move whole 128-byte lines).
 __global__ void __launch_bounds__(256)
 sigma_join_kernel(const float *__restrict__ part, SigSplit w, int nb, int n, const float *__restrict__ rs,
                   float *__restrict__ Sig, int64_t ldS) {
@@ -327,24 +347,26 @@ sigma_join_kernel(const float *__restrict__ part, SigSplit w, int nb, int n, con
     const int r0 = I * kSigTile + pr, c0 = J * kSigTile + pc;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     if (r0 >= n || c0 >= n || (I == J && pc < pr)) return;   // uniform: nothing on or above the diagonal here
-    const float *src = part + ((int64_t)blockIdx.y * w.parts * kSigTile + pr) * kSigTile + pc + tx;
+    const float *src = part + (int64_t)blockIdx.y * w.parts * kSigTile * kSigTile +
+                       (((pr / 32) * 2 + pc / 128) * 128 + pc % 128) * 32 + tx;
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int p = 0; p < w.parts; ++p)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s[k] += __ldcg(src + (int64_t)p * kSigTile * kSigTile + (ty + 8 * k) * 32);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int r = ty + 8 * k;
-        float s = 0.f;
-#pragma unroll 4
-        for (int p = 0; p < w.parts; ++p) s += __ldcg(src + ((int64_t)p * kSigTile + r) * kSigTile);
-        const int row = r0 + r, col = c0 + tx;
-        if (rs != nullptr && row < n && col < n) s *= rs[row] * rs[col];
-        t[r][tx] = s;
-        if (row < n && col < n && col >= row) Sig[(int64_t)row * ldS + col] = s;
+        const int c = ty + 8 * k, row = r0 + tx, col = c0 + c;
+        if (rs != nullptr && row < n && col < n) s[k] *= rs[row] * rs[col];
+        t[c][tx] = s[k];
+        if (row < n && col < n && col >= row) Sig[(int64_t)col * ldS + row] = s[k];
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int c = ty + 8 * k;
-        const int row = r0 + tx, col = c0 + c;
-        if (row < n && col < n && col > row) Sig[(int64_t)col * ldS + row] = t[tx][c];
+        const int r = ty + 8 * k;
+        const int row = r0 + r, col = c0 + tx;
+        if (row < n && col < n && col > row) Sig[(int64_t)row * ldS + col] = t[tx][r];
     }
 }
 
