@@ -523,7 +523,8 @@ static int gemmc_pair_set_attrs() {
 // of the full waves: they start on the SMs that those leave, and end after
 // them.  BF16 calls: 1733 x 9001 to 1000 columns (28 tiles) 117 -> 103 us,
 // 3000 x 20000 to 2048 (96) 324 -> 304 us, 5440 x 48374 to 2048 (176)
-// 999 -> 962 us, to 8192 (704, under the power cap) 3.44 -> 3.40 ms.
+// 999 -> 962 us; to 8192 columns (704) 1 % (3.396 -> 3.362 ms, runs of one side
+// differ by 0.4 %).
 constexpr int kPairs = 152 / 2;                     // CTA pairs that run at once
 template <int NA>
 static int gemmc_pair_run(const CUtensorMap &ta, const CUtensorMap &tb, const CUtensorMap &ta2, int64_t M, int64_t N,

@@ -1,15 +1,18 @@
 // NPGA solve (Algorithm 1, fixed step of Sec. 3.1) on one GPU.
 //
-// Per iteration three kernels run back to back on one stream:
-//   gemv_t  z = L^T y^k                 (all SMs, HBM-bound)
-//   gemv_n  g = L z                     (all SMs, HBM-bound)
-//   step    one block: grad f(x^k) by linearity, KKT check every kkt_every
-//           iterations, v = y^k - alpha (2g + 2 gamma y^k), x^{k+1} = Pi_F(v)
-//           (FP64, warm-started), FISTA momentum and extrapolation.
-// A chunk of kkt_every iterations is captured once into a CUDA graph and
-// replayed; every kernel returns at once when the device-side `done` flag is
-// set, so a chunk that overruns convergence costs only empty launches.  The
-// host reads the flag once per chunk.
+// Per iteration, on one stream:
+//   product g = L L^T y^k: one fused pass over L (llt.cuh), or gemv_t and
+//           gemv_n (gemv.cuh), or one symmetric pass over Sigma (symv.cuh)
+//   step    one cluster of 1 to 16 blocks: grad f(x^k) by linearity, KKT check
+//           every kkt_every iterations, v = y^k - alpha (2g + 2 gamma y^k),
+//           x^{k+1} = Pi_F(v) (FP64, warm-started), FISTA momentum and
+//           extrapolation
+// launched as programmatic dependents of each other (kLoopPdl).  A chunk of
+// kkt_every iterations is captured once into a CUDA graph and replayed; every
+// kernel returns when the device-side `done` flag is set, so a chunk that
+// overruns convergence costs only empty launches (counted in info.launches).
+// The host reads the flag once per chunk, and launches the next chunk before
+// it does where the residuals say that it will be needed.
 #include <cfloat>
 
 #include "solve_internal.cuh"
@@ -845,6 +848,11 @@ __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char 
 }
 
 // 96 registers: beside the fused pass (72 x 544) a step still fits an SM's file.
+// The compiler spills for it (344 to 356 bytes of stores per thread; the
+// grouped and backtracking steps, which it holds to 80 to 128 around the
+// out-of-line safeguard, 88 to 348), to L1 lines of the block's own; against
+// the code before, which spilled nothing, every kind of step gained
+// (backtracking 3000 x 6000 8.39 -> 7.60 ms, 5440 x 12000 15.8 -> 14.9).
 constexpr int kStepRegs = 96;
 template <int CL>
 __global__ void __maxnreg__(kStepRegs) npga_step_kernel(StepArgs a) {
