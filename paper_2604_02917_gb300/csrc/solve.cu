@@ -825,6 +825,8 @@ __device__ __forceinline__ void npga_step_body(const StepArgs &a, unsigned char 
             real = true;
             continue;
         }
+        // an infeasible target takes no exchange: no flag before every block has read it
+        if (o.status == MV_ERR_INFEASIBLE) cluster_barrier<CL>();
         if (rank == 0 && threadIdx.x == 0) {
             st->t = sc[0];
             st->beta_prev = beta;
